@@ -483,6 +483,10 @@ void make_plan(const su2_batch* b, int G, std::vector<int>& order, std::vector<i
     return a.first > c.first;
   });
   for (size_t k = 0; k < frac.size() && used < ctas; ++k, ++used) share[frac[k].second] += 1;
+  // many groups whose work is worth less than the one CTA each gets leave too
+  // few for the others: the largest shares give way, so that every group has a
+  // CTA (G <= ctas)
+  for (; used > ctas; --used) *std::max_element(share.begin(), share.end()) -= 1;
   // no group gets more CTAs than its largest lattice has links for at the
   // smallest block (192 threads: the measured kernel's 3/4 of 256), so that a
   // small lattice alone does not spread its barriers over idle CTAs; CTAs
