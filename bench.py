@@ -299,7 +299,8 @@ def batch_source_sha():
     """Hash of the batched kernel's sources (code only) and build flags."""
     h = hashlib.sha256()
     pkg = os.path.join(ROOT, "paper_1010_4834_gb300")
-    for f in ("su2_batch.cu", "su2_device.cuh", "su2_hb_link.cuh", "su2_kernel_util.cuh", "su2_internal.h"):
+    for f in ("su2_batch.cu", "su2_batch.h", "su2_batch_kernel.cuh", "su2_device.cuh", "su2_fixed.cuh", "su2_hb_link.cuh",
+              "su2_kernel_util.cuh", "su2_internal.h"):
         with open(os.path.join(pkg, "csrc", f), encoding="utf-8") as fh:
             h.update(_code_only(fh.read()).encode())
     with open(os.path.join(pkg, "build.py"), encoding="utf-8") as fh:
@@ -446,8 +447,8 @@ def source_sha():
     """Hash of the heat-bath kernels' sources (code only) and build flags."""
     h = hashlib.sha256()
     pkg = os.path.join(ROOT, "paper_1010_4834_gb300")
-    for f in (os.path.join(pkg, "csrc", "su2_device.cuh"), os.path.join(pkg, "csrc", "su2_heatbath.cu"),
-              os.path.join(pkg, "csrc", "su2_hb_link.cuh"), os.path.join(pkg, "csrc", "su2_pair.cu"),
+    for f in (os.path.join(pkg, "csrc", "su2_device.cuh"), os.path.join(pkg, "csrc", "su2_heatbath.cuh"),
+              os.path.join(pkg, "csrc", "su2_hb_link.cuh"), os.path.join(pkg, "csrc", "su2_pair.cu"), os.path.join(pkg, "csrc", "su2_fixed.cuh"),
               os.path.join(pkg, "csrc", "su2_kernel_util.cuh"), os.path.join(pkg, "csrc", "su2_internal.h"),
               os.path.join(pkg, "build.py")):
         with open(f, encoding="utf-8") as fh:

@@ -72,7 +72,7 @@ extern "C" {
 #define SU2_HOT 1  /* every link Haar-random (Section 2, Eq. 4)               */
 
 /* link storage precision */
-#define SU2_F64 0  /* FP64 links, FP64 arithmetic                             */
+#define SU2_F64 0  /* FP64 links; FP64 and 58-bit fixed-point arithmetic      */
 #define SU2_F32 1  /* FP32 links, FP32 arithmetic, FP64 reductions            */
 #define SU2_F16Q 2 /* binary16 quaternion storage, normalised on load, FP32   */
 
@@ -325,8 +325,9 @@ int su2_ape_smear(su2_lattice* h, double alpha, int n);
  * (1/2) Tr of the R x T loop.  1 <= Rmax <= min(N0,N1,N2), 1 <= Tmax <= N3,
  * Rmax, Tmax <= 32.  use_smeared = 1 takes the spatial links from the last
  * su2_ape_smear (SU2_ESTATE if there is none since the last sweep or
- * set_links); temporal links are always the chain's.  For Rmax, Tmax <= 16
- * and N3 / 8 in {1, 2, 4, 6, 8} the loops are evaluated in temporal gauge
+ * set_links); temporal links are always the chain's.  For Rmax, Tmax <= 16,
+ * N3 <= 64 and planes that fit a multiprocessor's shared memory (spatial extents
+ * to 64; FP64: unit quaternions only) the loops are evaluated in temporal gauge
  * (the loop is gauge invariant: after the transform each is one dot
  * product of two spatial lines), which equals the direct product up to
  * rounding; other shapes multiply the loops out.  Synchronises.

@@ -1,0 +1,8 @@
+#include "su2_batch_kernel.cuh"
+
+namespace su2 {
+
+template cudaError_t launch_batch_groups<kF16Q, false>(int, int, const BatchArgs&, cudaStream_t);
+template int batch_blocks_per_sm<kF16Q, false>(int);
+
+}  // namespace su2

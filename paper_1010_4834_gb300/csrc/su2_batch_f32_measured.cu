@@ -1,0 +1,8 @@
+#include "su2_batch_kernel.cuh"
+
+namespace su2 {
+
+template cudaError_t launch_batch_groups<kF32, true>(int, int, const BatchArgs&, cudaStream_t);
+template int batch_blocks_per_sm<kF32, true>(int);
+
+}  // namespace su2

@@ -740,8 +740,26 @@ extern "C" int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smea
   if (use_smeared && !h->smeared) return fail(SU2_ESTATE, "no smeared links since the last update");
   DeviceGuard dg(h->device);
   const void* spatial = use_smeared ? h->ape[h->smeared - 1] : h->links;
-  SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, h->stream));
-  return fetch_out(h, Rmax * Tmax, out);
+  const int n = Rmax * Tmax;
+  if (h->prec != SU2_F64) {
+    SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, nullptr, h->stream));
+    return fetch_out(h, n, out);
+  }
+  // FP64: the fixed-point kernel reports links that are not unit quaternions
+  // (a store filled from outside) in the word behind the results; the loops are
+  // then multiplied out in FP64
+  double* flag = h->scratch.out + n;
+  SU2_CU(cudaMemsetAsync(flag, 0, sizeof *flag, h->stream));
+  SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, flag, h->stream));
+  double got[32 * 32 + 1];
+  int rc = fetch_out(h, n + 1, got);
+  if (rc) return rc;
+  if (got[n] != 0.0) {
+    SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, nullptr, h->stream));
+    return fetch_out(h, n, out);
+  }
+  std::memcpy(out, got, n * sizeof(double));
+  return SU2_OK;
 }
 
 // The device-visible address of page-locked host memory (cudaHostAlloc,

@@ -15,6 +15,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "su2_fixed.cuh"
+
 namespace su2 {
 
 // ---------------------------------------------------------------------------
@@ -86,12 +88,57 @@ template <class R> __device__ __forceinline__ R qdot(const Quat<R>& a, const Qua
   return a.w * b.w + a.x * b.x + a.y * b.y + a.z * b.z;
 }
 
+// Products with every rounding spelled out: a sum of two products leaves the
+// compiler the choice which of them it fuses, and kernels that must agree bit
+// for bit (plain, measured and small-lattice substeps, batches, time slabs) did
+// differ.  FP32 fuses as the kernels were compiled before: the first product of
+// each sum, or the first positive one.
+template <> __device__ __forceinline__ float qdot<float>(const Quat<float>& a, const Quat<float>& b) {
+  return fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x))));
+}
+template <> __device__ __forceinline__ Quat<float> qmul<float>(const Quat<float>& a, const Quat<float>& b) {
+  return qmake<float>(fmaf(-a.z, b.z, fmaf(-a.y, b.y, fmaf(a.w, b.w, __fmul_rn(-a.x, b.x)))),
+                      fmaf(a.z, b.y, fmaf(-a.y, b.z, fmaf(a.w, b.x, __fmul_rn(a.x, b.w)))),
+                      fmaf(a.x, b.z, fmaf(-a.z, b.x, fmaf(a.w, b.y, __fmul_rn(a.y, b.w)))),
+                      fmaf(a.y, b.x, fmaf(-a.x, b.y, fmaf(a.w, b.z, __fmul_rn(a.z, b.w)))));
+}
+template <> __device__ __forceinline__ Quat<float> qmul_nd<float>(const Quat<float>& a, const Quat<float>& b) {
+  return qmake<float>(fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x)))),
+                      fmaf(-a.z, b.y, fmaf(a.y, b.z, fmaf(a.x, b.w, __fmul_rn(-a.w, b.x)))),
+                      fmaf(-a.x, b.z, fmaf(a.z, b.x, fmaf(a.y, b.w, __fmul_rn(-a.w, b.y)))),
+                      fmaf(-a.y, b.x, fmaf(a.x, b.y, fmaf(a.z, b.w, __fmul_rn(-a.w, b.z)))));
+}
+template <> __device__ __forceinline__ Quat<float> qmul_dn<float>(const Quat<float>& a, const Quat<float>& b) {
+  return qmul<float>(qmake<float>(a.w, -a.x, -a.y, -a.z), b);
+}
+template <> __device__ __forceinline__ double qdot<double>(const Quat<double>& a, const Quat<double>& b) {
+  return __fma_rn(a.z, b.z, __fma_rn(a.y, b.y, __fma_rn(a.x, b.x, __dmul_rn(a.w, b.w))));
+}
+template <> __device__ __forceinline__ Quat<double> qmul<double>(const Quat<double>& a, const Quat<double>& b) {
+  Quat<double> r;
+  r.w = __fma_rn(-a.z, b.z, __fma_rn(-a.y, b.y, __fma_rn(-a.x, b.x, __dmul_rn(a.w, b.w))));
+  r.x = __fma_rn(a.z, b.y, __fma_rn(-a.y, b.z, __fma_rn(a.x, b.w, __dmul_rn(a.w, b.x))));
+  r.y = __fma_rn(a.x, b.z, __fma_rn(-a.z, b.x, __fma_rn(a.y, b.w, __dmul_rn(a.w, b.y))));
+  r.z = __fma_rn(a.y, b.x, __fma_rn(-a.x, b.y, __fma_rn(a.z, b.w, __dmul_rn(a.w, b.z))));
+  return r;
+}
+template <> __device__ __forceinline__ Quat<double> qmul_nd<double>(const Quat<double>& a, const Quat<double>& b) {
+  return qmul<double>(a, qmake<double>(b.w, -b.x, -b.y, -b.z));
+}
+template <> __device__ __forceinline__ Quat<double> qmul_dn<double>(const Quat<double>& a, const Quat<double>& b) {
+  return qmul<double>(qmake<double>(a.w, -a.x, -a.y, -a.z), b);
+}
+
 template <class R> __device__ __forceinline__ void qacc(Quat<R>& a, const Quat<R>& b) {
   a.w += b.w; a.x += b.x; a.y += b.y; a.z += b.z;
 }
 
 template <class R> __device__ __forceinline__ Quat<R> qscale(const Quat<R>& a, R s) {
   return qmake<R>(a.w * s, a.x * s, a.y * s, a.z * s);
+}
+
+template <> __device__ __forceinline__ Quat<double> qscale<double>(const Quat<double>& a, double s) {
+  return qmake<double>(__dmul_rn(a.w, s), __dmul_rn(a.x, s), __dmul_rn(a.y, s), __dmul_rn(a.z, s));
 }
 
 template <class R> __device__ __forceinline__ Quat<R> qone() { return qmake<R>(1, 0, 0, 0); }
@@ -176,13 +223,57 @@ template <> __device__ __forceinline__ float u01<float>(uint32_t x) {
 // ---------------------------------------------------------------------------
 template <class R> struct Math;
 
+// FP64 roots and reciprocals from an FP32 approximation of the significand
+// (2^-22, taken and put back by bit operations: the FP64 pipe also does the
+// conversions) and one third-order step: 5, 6 and 3 FP64 operations, where
+// 1/sqrt(v), sqrt(v) and a division take about 20, 10 and 10.  Errors below
+// one unit in the last place of v > 0 normal.
+__device__ __forceinline__ float significand32(double v, int exponent) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  return __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | ((uint32_t)(127 + exponent) << 23));
+}
+// f 2^k, f > 0
+__device__ __forceinline__ double widen(float f, int k) {
+  const uint32_t b = __float_as_uint(f);
+  return __hiloint2double((int)((b >> 3) + ((uint32_t)(1023 - 127 + k) << 20)), (int)(b << 29));
+}
+// 1/sqrt(v) to 2^-22
+__device__ __forceinline__ double rsqrt_seed(double v) {
+  const int e = __double2hiint(v) >> 20;          // v = m 4^k, 1 <= m < 4
+  return widen(rsqrtf(significand32(v, (e & 1) ^ 1)), 512 - ((e + 1) >> 1));
+}
+__device__ __forceinline__ double rsqrt64(double v) {
+  const double y = rsqrt_seed(v);
+  const double h = __fma_rn(-__dmul_rn(v, y), y, 1.0);
+  return __fma_rn(__dmul_rn(y, h), __fma_rn(h, 0.375, 0.5), y);
+}
+// sqrt(max(v, 0))
+__device__ __forceinline__ double sqrt64(double v) {
+  if (__double2hiint(v) < 0x00100000) return 0.0;  // v <= 0 or subnormal
+  const double y = rsqrt_seed(v);
+  const double g = __dmul_rn(v, y);
+  const double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
+  const double s = __fma_rn(g, __fma_rn(-g, h, 0.5), g);
+  return __fma_rn(__fma_rn(-s, s, v), h, s);
+}
+// 1/(2 a), a > 0
+__device__ __forceinline__ double half_inverse64(double a) {
+  const int e = __double2hiint(a) >> 20;
+  if (e > 2040) return 0.0;                       // a above 2^1017, infinity
+  float f = significand32(a, 0);
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(f));
+  const double y = widen(f, 1023 - e);
+  const double d = __fma_rn(-a, y, 1.0);
+  const double z = __fma_rn(y, __fma_rn(d, d, d), y);
+  return __hiloint2double(__double2hiint(z) - (1 << 20), __double2loint(z));
+}
+
 template <> struct Math<double> {
   static __device__ __forceinline__ double log_fast(double v) { return log(v); }
   static __device__ __forceinline__ double log_acc(double v) { return log(v); }
-  static __device__ __forceinline__ double cos2pi(double u) { return cospi(2.0 * u); }
   static __device__ __forceinline__ void sincos2pi(double u, double* s, double* c) { sincospi(2.0 * u, s, c); }
-  static __device__ __forceinline__ double sqrt0(double v) { return sqrt(fmax(v, 0.0)); }
-  static __device__ __forceinline__ double rsqrt(double v) { return 1.0 / sqrt(v); }
+  static __device__ __forceinline__ double sqrt0(double v) { return sqrt64(v); }
+  static __device__ __forceinline__ double rsqrt(double v) { return rsqrt64(v); }
   static __device__ __forceinline__ double div(double a, double b) { return a / b; }
   static __device__ __forceinline__ double exp(double v) { return ::exp(v); }
   static constexpr double kTiny = 1e-300;
@@ -224,6 +315,33 @@ template <class R> __device__ __forceinline__ Quat<R> haar_from(uint4 r) {
   return qscale(z, M::rsqrt(qdot(z, z)));
 }
 
+// FP64 links and sums in fixed point and back.
+__device__ __forceinline__ FixQuat fix_of(const Quat<double>& q, int conj, FixBad& bad) {
+  return fix_link((uint32_t)__double2loint(q.w), (uint32_t)__double2hiint(q.w), (uint32_t)__double2loint(q.x),
+                        (uint32_t)__double2hiint(q.x), (uint32_t)__double2loint(q.y), (uint32_t)__double2hiint(q.y),
+                        (uint32_t)__double2loint(q.z), (uint32_t)__double2hiint(q.z), conj, bad);
+}
+
+__device__ __forceinline__ Quat<double> fix_sum_to_double(const FixSum& s) {
+  return qmake<double>(fix_to_double(fix_fold(s.hw, s.mw)), fix_to_double(fix_fold(s.hx, s.mx)),
+                       fix_to_double(fix_fold(s.hy, s.my)), fix_to_double(fix_fold(s.hz, s.mz)));
+}
+
+// A link that must be a unit quaternion to 2^-29, whatever its components
+// (zero, tiny); `bad` is raised otherwise.
+__device__ __forceinline__ FixQuat fix_unit_link(const Quat<double>& q, bool& bad) {
+  FixQuat f;
+  f.w = fix_from_any((uint32_t)__double2loint(q.w), (uint32_t)__double2hiint(q.w));
+  f.x = fix_from_any((uint32_t)__double2loint(q.x), (uint32_t)__double2hiint(q.x));
+  f.y = fix_from_any((uint32_t)__double2loint(q.y), (uint32_t)__double2hiint(q.y));
+  f.z = fix_from_any((uint32_t)__double2loint(q.z), (uint32_t)__double2hiint(q.z));
+  // components below 2 (the conversion's range) and |q|^2 within 2^-28 of one
+  const uint32_t top = (uint32_t)(__double2hiint(q.w) | __double2hiint(q.x) | __double2hiint(q.y) | __double2hiint(q.z));
+  const int64_t off = fix_dot(f, f, -((int64_t)1 << kFixFrac)) + ((int64_t)1 << (kFixFrac - 28));
+  bad |= (top & 0x40000000u) != 0u || (uint64_t)off >> (kFixFrac - 27) != 0u;
+  return f;
+}
+
 // ---------------------------------------------------------------------------
 // Heat-bath parameters shared by a launch (passed as a __grid_constant__
 // kernel parameter).
@@ -242,30 +360,95 @@ struct HBParams {
 //                      accept if u3^2 <= 1 - delta, a0 = 1 - 2 delta.
 //   Creutz:            a0 = 1 + ln(e^{-2 alpha} + (1 - e^{-2 alpha}) u0)/alpha,
 //                      accept if u1^2 <= 1 - a0^2.
+// A Kennedy-Pendleton trial's numbers, s = -2 alpha delta and u3, do not
+// depend on the links (the small-lattice kernel draws them ahead).
+// FP64 lattices draw in fixed point (su2_fixed.cuh): -2 alpha delta in units of
+// 2^-57, u3^2 and a0 in units of 2^-62.
+template <class R> struct TrialNumbers { R s, u3; };
+template <> struct TrialNumbers<double> { uint64_t s, u3; };
+template <class R> struct DrawTypes { using A0 = R; using W = Quat<R>; };
+template <> struct DrawTypes<double> { using A0 = int64_t; using W = FixQuat; };
+template <class R> using A0Of = typename DrawTypes<R>::A0;
+template <class R> using WOf = typename DrawTypes<R>::W;
+
+template <class R> __device__ __forceinline__ TrialNumbers<R> trial_numbers(uint4 r) {
+  TrialNumbers<R> t;
+  if constexpr (sizeof(R) == 8) {
+    t.s = ((uint64_t)fix_neg_log(r.x) >> 1) + fix_umulhi((uint64_t)fix_neg_log(r.z), fix_cos2(r.y));
+    const uint64_t z = (2 * (uint64_t)r.w + 1) << 31;
+    t.u3 = fix_umulhi(z, z) >> 2;
+  } else {
+    using M = Math<R>;
+    const R u0 = u01<R>(r.x), u1 = u01<R>(r.y), u2 = u01<R>(r.z);
+    t.u3 = u01<R>(r.w);
+    const R c = M::cos2pi(u1);
+    t.s = M::log_fast(u0) + c * c * M::log_fast(u2);
+  }
+  return t;
+}
+
+__device__ __forceinline__ bool trial_decide(const TrialNumbers<float>& t, float inv2a, float* a0) {
+  const float delta = -(t.s) * inv2a;
+  if (t.u3 * t.u3 <= 1.0f - delta) { *a0 = 1.0f - 2.0f * delta; return true; }
+  return false;
+}
+__device__ __forceinline__ bool trial_decide(const TrialNumbers<double>& t, double inv2a, int64_t* a0) {
+  // delta = s 2^-57 inv2a in units of 2^-62, inv2a = 1.m 2^e: the 64-bit
+  // significand times s, shifted by e + 6
+  const uint32_t lo = (uint32_t)__double2loint(inv2a), hi = (uint32_t)__double2hiint(inv2a);
+  const uint64_t m = (((uint64_t)(hi | 0x100000u) << 32) | lo) << 11;
+  const uint64_t p = fix_umulhi(t.s, m);
+  const int sh = (int)(hi >> 20) - 1023 + 6;
+  constexpr uint64_t one = (uint64_t)1 << 62;
+  uint64_t delta = fix_shr(p, (uint32_t)(sh < 0 ? -sh : 0));
+  if (sh > 0) {
+    if (fix_shr(p, (uint32_t)(sh < 62 ? 62 - sh : 0)) != 0u) return false;   // delta >= 1
+    delta = p << sh;
+  }
+  if (delta > one || t.u3 > one - delta) return false;
+  *a0 = (int64_t)(one - 2 * delta);
+  return true;
+}
+template <class R>
+__device__ __forceinline__ bool creutz_decide(R u0, R u1, R alpha, R e, A0Of<R>* a0) {
+  using M = Math<R>;
+  const R cand = R(1) + M::div(M::log_fast(e + (R(1) - e) * u0), alpha);
+  if (!(u1 * u1 <= R(1) - cand * cand)) return false;
+  if constexpr (sizeof(R) == 8) *a0 = __double2ll_rn(__dmul_rn(cand, 0x1p62));
+  else *a0 = cand;
+  return true;
+}
+// The Kennedy-Pendleton trial in FP64 throughout, for small alpha: delta =
+// s / (2 alpha) magnifies the 2^-57 of the fixed-point logarithms.
+constexpr double kFixMinAlpha = 0.25;
+static __device__ __noinline__ bool trial_small_alpha(uint4 r, double inv2a, int64_t* a0) {
+  const double u0 = u01<double>(r.x), u1 = u01<double>(r.y), u2 = u01<double>(r.z), u3 = u01<double>(r.w);
+  const double c = cospi(2.0 * u1);
+  const double delta = -(log(u0) + c * c * log(u2)) * inv2a;
+  if (!(u3 * u3 <= 1.0 - delta)) return false;
+  *a0 = __double2ll_rn(__dmul_rn(__fma_rn(-2.0, delta, 1.0), 0x1p62));
+  return true;
+}
 // *rt receives the draw's four Philox words (compose_link reads the FP32
 // direction from them).
 template <class R>
-__device__ __forceinline__ bool trial_a0(R alpha, R inv2a, R e, uint4 ctr, int n, const HBParams& hp, R* a0,
+__device__ __forceinline__ bool trial_a0(R alpha, R inv2a, R e, uint4 ctr, int n, const HBParams& hp, A0Of<R>* a0,
                                          uint4* rt) {
-  using M = Math<R>;
   ctr.w = (uint32_t)n;
   const uint4 r = philox(ctr, hp.rk);
   *rt = r;
-  if (hp.sampler == 0) {
-    const R u0 = u01<R>(r.x), u1 = u01<R>(r.y), u2 = u01<R>(r.z), u3 = u01<R>(r.w);
-    const R c = M::cos2pi(u1);
-    const R delta = -(M::log_fast(u0) + c * c * M::log_fast(u2)) * inv2a;
-    if (u3 * u3 <= R(1) - delta) { *a0 = R(1) - R(2) * delta; return true; }
-  } else {
-    const R u0 = u01<R>(r.x), u1 = u01<R>(r.y);
-    const R cand = R(1) + M::div(M::log_fast(e + (R(1) - e) * u0), alpha);
-    if (u1 * u1 <= R(1) - cand * cand) { *a0 = cand; return true; }
+  if (hp.sampler != 0) return creutz_decide<R>(u01<R>(r.x), u01<R>(r.y), alpha, e, a0);
+  if constexpr (sizeof(R) == 8) {
+    if (__builtin_expect(!(alpha >= kFixMinAlpha), 0)) return trial_small_alpha(r, inv2a, a0);
   }
-  return false;
+  return trial_decide(trial_numbers<R>(r), inv2a, a0);
 }
 
 // The per-link constants of the trials.
-template <class R> __device__ __forceinline__ R trial_inv2a(R alpha) { return Math<R>::div(R(0.5), alpha); }
+template <class R> __device__ __forceinline__ R trial_inv2a(R alpha) {
+  if constexpr (sizeof(R) == 8) return half_inverse64(alpha);
+  else return Math<R>::div(R(0.5), alpha);
+}
 template <class R> __device__ __forceinline__ R trial_e(R alpha, int sampler) {
   return sampler ? Math<R>::exp(R(-2) * alpha) : R(0);
 }
@@ -273,8 +456,8 @@ template <class R> __device__ __forceinline__ R trial_e(R alpha, int sampler) {
 // Trials first..max_tries; returns the trial that accepted, 0 if none; *rt
 // holds the accepting trial's Philox words.
 template <class R>
-__device__ __forceinline__ int sample_a0_from(int first, R alpha, R inv2a, R e, uint4 ctr, const HBParams& hp, R* a0,
-                                              uint4* rt) {
+__device__ __forceinline__ int sample_a0_from(int first, R alpha, R inv2a, R e, uint4 ctr, const HBParams& hp,
+                                              A0Of<R>* a0, uint4* rt) {
   for (int n = first; n <= hp.max_tries; ++n)
     if (trial_a0<R>(alpha, inv2a, e, ctr, n, hp, a0, rt)) return n;
   return 0;
@@ -289,33 +472,104 @@ __device__ __forceinline__ int sample_a0_from(int first, R alpha, R inv2a, R e, 
 //         trial's uniforms), cos theta = (2c + 1) 2^-18 - 1 and
 //         phi = 2 pi (f + 1/2) 2^-18; one Philox block per accepted trial
 //         instead of two (the 64^4 FP32 substep 187.6 -> 179.2 us).
-template <class R> __device__ __forceinline__ void link_direction(uint4 ctr, uint4 rt, const HBParams& hp, R* cos_t,
-                                                                   R* sp, R* cp) {
+template <class R> struct Direction { R cos_t, sin_t, sp, cp; };
+template <> struct Direction<double> { int64_t cos_t, sin_t, sp, cp; };   // units of 2^-62
+
+// sqrt(v 2^-FRAC) in units of 2^-62, 0 < v 2^-FRAC <= 1: FP64's root of the
+// converted value
+template <int FRAC> __device__ __forceinline__ int64_t fix_sqrt62(uint64_t v) {
+  const double r = sqrt64(__hiloint2double(__double2hiint(__ull2double_rn(v)) - (FRAC << 20), __double2loint(__ull2double_rn(v))));
+  return v ? fix_unsigned62((uint32_t)__double2loint(r), (uint32_t)__double2hiint(r)) : 0;
+}
+
+template <class R> __device__ __forceinline__ Direction<R> draw_direction(uint4 ctr, uint4 rt, const HBParams& hp) {
   using M = Math<R>;
+  Direction<R> d;
   if constexpr (sizeof(R) == 4) {
     const uint32_t c = ((rt.x & 0x1FFu) << 9) | (rt.y & 0x1FFu);
     const uint32_t f = ((rt.z & 0x1FFu) << 9) | (rt.w & 0x1FFu);
-    *cos_t = fmaf((float)(2u * c + 1u), 0x1p-18f, -1.0f);   // exact: 19 significant bits
-    M::sincos2pi(fmaf((float)f, 0x1p-18f, 0x1p-19f), sp, cp);
+    d.cos_t = fmaf((float)(2u * c + 1u), 0x1p-18f, -1.0f);   // exact: 19 significant bits
+    M::sincos2pi(fmaf((float)f, 0x1p-18f, 0x1p-19f), &d.sp, &d.cp);
+    d.sin_t = M::sqrt0(R(1) - d.cos_t * d.cos_t);
   } else {
     ctr.w = 0u;
     const uint4 r = philox(ctr, hp.rk);
-    *cos_t = R(2) * u01<R>(r.x) - R(1);
-    M::sincos2pi(u01<R>(r.y), sp, cp);
+    const uint64_t z = 2 * (uint64_t)r.x + 1;                       // u0 = z 2^-33
+    d.cos_t = (int64_t)(z << 30) - ((int64_t)1 << 62);
+    d.sin_t = fix_sqrt62<64>(z * (((uint64_t)1 << 33) - z));        // sin^2 = 4 u0 (1 - u0)
+    fix_sincos(r.y, &d.sp, &d.cp);
   }
+  return d;
 }
 
 // The accepted link (Section 2, Eqs. 7, 9): X with x0 = a0 and the direction
-// of link_direction, times W = Sigma / k.  rt: the accepting trial's words.
-template <class R>
-__device__ __forceinline__ Quat<R> compose_link(R a0, const Quat<R>& w, uint4 ctr, uint4 rt, const HBParams& hp) {
-  using M = Math<R>;
-  R cos_t, sp, cp;
-  link_direction<R>(ctr, rt, hp, &cos_t, &sp, &cp);
-  const R sin_t = M::sqrt0(R(1) - cos_t * cos_t);
-  const R rad = M::sqrt0(R(1) - a0 * a0);
-  const Quat<R> x = qmake<R>(a0, rad * sin_t * cp, rad * sin_t * sp, rad * cos_t);
+// of draw_direction, times W = Sigma / k.  rt: the accepting trial's words.
+__device__ __forceinline__ Quat<float> compose_from(float a0, const Quat<float>& w, const Direction<float>& d) {
+  const float rad = Math<float>::sqrt0(1.0f - a0 * a0);
+  const Quat<float> x = qmake<float>(a0, rad * d.sin_t * d.cp, rad * d.sin_t * d.sp, rad * d.cos_t);
   return qmul(x, w);
+}
+__device__ __forceinline__ Quat<double> compose_from(int64_t a0, const FixQuat& w, const Direction<double>& d) {
+  // |x|^2 = 1 - a0^2 = (1 - a0) (1 + a0); a0 > -1, and at a0 = 1 the second
+  // factor overflows to 0 like the product
+  constexpr int64_t one = (int64_t)1 << 62;
+  const int64_t rad = fix_sqrt62<62>(fix_umulhi(2 * (uint64_t)(one - a0), 2 * (uint64_t)(one + a0)));
+  const int64_t rs = fix_mulhi(rad, d.sin_t) << 2;
+  const FixQuat x{fix_split(a0 >> 4), fix_split((fix_mulhi(rs, d.cp) + 2) >> 2), fix_split((fix_mulhi(rs, d.sp) + 2) >> 2),
+                  fix_split((fix_mulhi(rad, d.cos_t) + 2) >> 2)};
+  FixSum s = fix_zero();
+  fix_mac(s, x, w);
+  return fix_sum_to_double(s);
+}
+template <class R>
+__device__ __forceinline__ Quat<R> compose_link(A0Of<R> a0, const WOf<R>& w, uint4 ctr, uint4 rt, const HBParams& hp) {
+  return compose_from(a0, w, draw_direction<R>(ctr, rt, hp));
+}
+
+// W = Sigma / k, k = |Sigma|, and alpha = beta k of a staple sum.
+template <class R> struct Frame { WOf<R> w; R alpha; };
+__device__ __forceinline__ Frame<float> staple_frame(const Quat<float>& sig, float beta) {
+  const float k2 = qdot(sig, sig);
+  const float invk = Math<float>::rsqrt(k2);
+  return Frame<float>{qscale(sig, invk), beta * k2 * invk};
+}
+// FP64: from any staple sum, and from one in fixed point (units of 2^-58),
+// which is shifted up to 62 bits first, so that small sums keep their digits:
+// k^2 = k2 2^(-52 - 2 n), W = v (2^26 / sqrt(k2)) in units of 2^-58.
+__device__ __forceinline__ Frame<double> staple_frame(const Quat<double>& sig, double beta) {
+  const double k2 = qdot(sig, sig);
+  const double invk = rsqrt64(k2);
+  const Quat<double> w = qscale(sig, invk);
+  auto fix = [](double v) { return fix_from_any((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v)); };
+  return Frame<double>{FixQuat{fix(w.w), fix(w.x), fix(w.y), fix(w.z)}, __dmul_rn(__dmul_rn(beta, k2), invk)};
+}
+__device__ __forceinline__ Frame<double> staple_frame(const FixSum& s, double beta) {
+  int64_t v[4] = {fix_fold(s.hw, s.mw), fix_fold(s.hx, s.mx), fix_fold(s.hy, s.my), fix_fold(s.hz, s.mz)};
+  const uint64_t top = (uint64_t)((v[0] ^ (v[0] >> 63)) | (v[1] ^ (v[1] >> 63)) | (v[2] ^ (v[2] >> 63)) | (v[3] ^ (v[3] >> 63)));
+  const int n = __clzll((long long)top) - 2;      // |v| < 2^62 after the shift (a sum is below 2^61)
+  Frame<double> f;
+  if (top == 0u) {                                 // a vanishing sum: alpha = 0
+    f.w = fix_one();
+    f.alpha = 0.0;
+    return f;
+  }
+  uint64_t k2 = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = v[i] << n;
+    k2 += (uint64_t)fix_mulhi(v[i], v[i]);         // in [2^58, 2^62]
+  }
+  const double d = __ull2double_rn(k2);
+  const double y = rsqrt64(d);                     // in [2^-31, 2^-29]
+  const uint64_t m = (((uint64_t)(((uint32_t)__double2hiint(y) & 0xFFFFFu) | 0x100000u)) << 32) | (uint32_t)__double2loint(y);
+  const int64_t y90 = (int64_t)(m << ((__double2hiint(y) >> 20) - 1023 + 38));   // y 2^90, below 2^62
+  f.w.w = fix_split(fix_mulhi(v[0], y90));
+  f.w.x = fix_split(fix_mulhi(v[1], y90));
+  f.w.y = fix_split(fix_mulhi(v[2], y90));
+  f.w.z = fix_split(fix_mulhi(v[3], y90));
+  const double k = __dmul_rn(d, y);                // k 2^(26 + n)
+  f.alpha = __dmul_rn(beta, __hiloint2double(__double2hiint(k) - ((26 + n) << 20), __double2loint(k)));
+  return f;
 }
 
 // Full heat-bath draw for one link given its staple sum (Section 2, Eqs. 5-9).
@@ -325,20 +579,17 @@ __device__ __forceinline__ Quat<R> compose_link(R a0, const Quat<R>& w, uint4 ct
 template <class R>
 __device__ __forceinline__ int heatbath_draw(const Quat<R>& sigma, uint4 ctr, const HBParams& hp,
                                              R beta, Quat<R>* out) {
-  using M = Math<R>;
-  const R k2 = qdot(sigma, sigma);
-  const R invk = M::rsqrt(k2);
-  const R alpha = beta * k2 * invk;
-  if (!(alpha >= R(1e-12))) {
+  const Frame<R> f = staple_frame(sigma, beta);
+  if (!(f.alpha >= R(1e-12))) {
     ctr.w = 1u;
     *out = haar_from<R>(philox(ctr, hp.rk));
     return -1;
   }
-  R a0;
+  A0Of<R> a0;
   uint4 rt;
-  const int n = sample_a0_from<R>(1, alpha, trial_inv2a(alpha), trial_e(alpha, hp.sampler), ctr, hp, &a0, &rt);
+  const int n = sample_a0_from<R>(1, f.alpha, trial_inv2a(f.alpha), trial_e(f.alpha, hp.sampler), ctr, hp, &a0, &rt);
   if (n == 0) return 0;
-  *out = compose_link<R>(a0, qscale(sigma, invk), ctr, rt, hp);
+  *out = compose_link<R>(a0, f.w, ctr, rt, hp);
   return n;
 }
 
@@ -375,8 +626,8 @@ template <int CP> struct Links<kF64, CP> {
     if constexpr (CP == kClassPtr) return c[cls];
     else return p + 2 * cls * vh;
   }
-  static __device__ __forceinline__ Quat<double> ldp(const double2* b, uint32_t i) {
-    const double2 a = __ldg(b + 2 * i), d = __ldg(b + 2 * i + 1);
+  template <bool NC> static __device__ __forceinline__ Quat<double> ldp(const double2* b, uint32_t i) {
+    const double2 a = NC ? __ldg(b + 2 * i) : b[2 * i], d = NC ? __ldg(b + 2 * i + 1) : b[2 * i + 1];
     return qmake<double>(a.x, a.y, d.x, d.y);
   }
   __host__ __device__ void set(void* base, int64_t n) {
@@ -429,8 +680,8 @@ template <int CP> struct Links<kF32, CP> {
     if constexpr (CP == kClassPtr) return c[cls];
     else return p + cls * vh;
   }
-  static __device__ __forceinline__ Quat<float> ldp(const float4* b, uint32_t i) {
-    const float4 a = __ldg(b + i);
+  template <bool NC> static __device__ __forceinline__ Quat<float> ldp(const float4* b, uint32_t i) {
+    const float4 a = NC ? __ldg(b + i) : b[i];
     return qmake<float>(a.x, a.y, a.z, a.w);
   }
   __host__ __device__ void set(void* base, int64_t n) {
@@ -478,7 +729,9 @@ template <int CP> struct Links<kF16Q, CP> {
     if constexpr (CP == kClassPtr) return c[cls];
     else return p + cls * vh;
   }
-  static __device__ __forceinline__ Quat<float> ldp(const uint2* b, uint32_t i) { return unpack(__ldg(b + i)); }
+  template <bool NC> static __device__ __forceinline__ Quat<float> ldp(const uint2* b, uint32_t i) {
+    return unpack(NC ? __ldg(b + i) : b[i]);
+  }
   __host__ __device__ void set(void* base, int64_t n) {
     p = static_cast<uint2*>(base);
     vh = n;
@@ -730,6 +983,105 @@ __device__ __forceinline__ Quat<typename Real<P>::T> staple_split(const Links<P,
   if (MU != 3) staple_term<P, MU, 3, NC, CP, MCG>(L, g, x, h, dmu, p, s);
   if (MU == 0) lower = qmake<R>(0, 0, 0, 0);
   return s;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 staples in fixed point (su2_fixed.cuh): the same terms in the same
+// order, each link converted as it is loaded.
+// ---------------------------------------------------------------------------
+// Half-index change of the step x -> x + (up ? 1 : -1) d-hat, d known at run time.
+__device__ __forceinline__ int half_step_rt(const Geom& g, const Site& x, int d, bool up) {
+  const int a = d == 0 ? half_step<0, +1>(g, x) : d == 1 ? half_step<1, +1>(g, x)
+              : d == 2 ? half_step<2, +1>(g, x) : half_step<3, +1>(g, x);
+  const int b = d == 0 ? half_step<0, -1>(g, x) : d == 1 ? half_step<1, -1>(g, x)
+              : d == 2 ? half_step<2, -1>(g, x) : half_step<3, -1>(g, x);
+  return up ? a : b;
+}
+
+// FP64 staples run one code for every direction and parity, a rolled loop over
+// the terms: unrolled and specialised like FP32's, the eight substeps' code
+// (45 KB each) was fetched anew for every launch, which on small lattices cost
+// more than the arithmetic.  Term k: direction nu = k / 2 (skipping mu), the
+// forward path for even k, the backward one for odd k; its three links a b c
+// enter as a b c^dagger (forward) or a^dagger b c.
+struct TermLinks { Quat<double> a, b, c; };
+template <bool NC, bool MCG, int CP>
+__device__ __forceinline__ TermLinks term_links(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h, int dmu,
+                                                int mu, int p, int k) {
+  const int q = p ^ 1, nu = (k >> 1) + ((k >> 1) >= mu);
+  const bool back = k & 1;
+  const int step = half_step_rt(g, x, nu, !back);
+  auto at = [&](int cls, int i, bool mcg) {
+    const double2* e = L.p + 2 * (cls * L.vh + i);
+    const double2 u = mcg ? __ldcg(e) : NC ? __ldg(e) : e[0];
+    const double2 v = mcg ? __ldcg(e + 1) : NC ? __ldg(e + 1) : e[1];
+    return qmake<double>(u.x, u.y, v.x, v.y);
+  };
+  const int hb = h + step, ha = back ? hb : h;
+  TermLinks t;
+  t.a = at(2 * nu + (back ? q : p), ha, false);         // U_nu(x) or U_nu(x-nu)
+  t.b = at(2 * mu + q, hb, MCG);                        // U_mu(x+nu) or U_mu(x-nu)
+  t.c = at(2 * nu + (back ? p : q), ha + dmu, false);   // U_nu(x+mu) or U_nu(x-nu+mu)
+  return t;
+}
+
+__device__ __forceinline__ int half_step_mu(const Geom& g, const Site& x, int mu) { return half_step_rt(g, x, mu, true); }
+
+// The staple sum over nu < nd in FP64 and its partial sum over nu < mu: the
+// path of links outside fix_link's range.
+template <bool NC, bool MCG, int CP>
+__device__ __forceinline__ Quat<double> staple_rolled(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h,
+                                                      int mu, int p, int nd, Quat<double>& lower) {
+  const int dmu = half_step_mu(g, x, mu);
+  Quat<double> s = qmake<double>(0, 0, 0, 0);
+  lower = s;
+#pragma unroll 1
+  for (int k = 0; k < 2 * (nd - 1); ++k) {
+    const TermLinks t = term_links<NC, MCG>(L, g, x, h, dmu, mu, p, k);
+    if (k & 1) qacc_mul(s, qmul_dn(t.a, t.b), t.c);
+    else qacc_mul_nd(s, qmul(t.a, t.b), t.c);
+    if (k + 1 == 2 * mu) lower = s;
+  }
+  return s;
+}
+
+// The same in fixed point, with LOWER also the partial sum.  False if a link is
+// outside fix_link's range; the caller then takes staple_rolled.  A term's
+// links are loaded while the previous term is multiplied.
+template <bool LOWER, bool NC, bool MCG, int CP>
+__device__ __forceinline__ bool staple_fixed(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h, int mu,
+                                             int p, int nd, FixSum& s, Quat<double>& lower) {
+  s = fix_zero();
+  FixBad bad{0u, 0u};
+  const int dmu = half_step_mu(g, x, mu);
+  if (LOWER) lower = qmake<double>(0, 0, 0, 0);
+  TermLinks t = term_links<NC, MCG>(L, g, x, h, dmu, mu, p, 0);
+#pragma unroll 1
+  for (int k = 0; k < 2 * (nd - 1); ++k) {
+    const TermLinks next = term_links<NC, MCG>(L, g, x, h, dmu, mu, p, k + 1 < 2 * (nd - 1) ? k + 1 : k);
+    const int odd = -(k & 1);
+    fix_mac(s, fix_mul(fix_of(t.a, odd, bad), fix_of(t.b, 0, bad)), fix_of(t.c, ~odd, bad));
+    if (LOWER && k + 1 == 2 * mu) lower = fix_sum_to_double(s);
+    t = next;
+  }
+  return fix_ok(bad);
+}
+
+// W, alpha of link (x, mu) and, with MEAS, the staple's partial sum over nu <
+// mu.  FP32 / F16Q: MU and the parity PAR at compile time.
+template <int P, int MU, bool MEAS, bool NC, int CP, bool MCG>
+__device__ __forceinline__ Frame<typename Real<P>::T> link_frame(const Links<P, CP>& L, const Geom& g, const Site& x,
+                                                                 int h, int mu, int p, typename Real<P>::T beta,
+                                                                 Quat<typename Real<P>::T>& lower) {
+  if constexpr (P == kF64) {
+    FixSum s;
+    if (__builtin_expect(staple_fixed<MEAS, NC, MCG>(L, g, x, h, mu, p, 4, s, lower), 1)) return staple_frame(s, beta);
+    return staple_frame(staple_rolled<NC, MCG>(L, g, x, h, mu, p, 4, lower), beta);
+  } else if constexpr (MEAS) {
+    return staple_frame(staple_split<P, MU, NC, CP, MCG>(L, g, x, h, p, lower), beta);
+  } else {
+    return staple_frame(staple<P, MU, 0xF, NC, CP, MCG>(L, g, x, h, p), beta);
+  }
 }
 
 }  // namespace su2

@@ -30,13 +30,13 @@ template <class R> struct PlainAcc {
 // moves in a few wide shared-memory accesses: 64^4 FP32 sweep 1412 -> 1407
 // us, F16Q 1610 -> 1592 us.
 template <class R, bool MEAS> struct __align__(16) Deferred {
-  Quat<R> w;
+  WOf<R> w;
   R alpha;
   int h;
   uint32_t site;
 };
 template <class R> struct __align__(16) Deferred<R, true> {
-  Quat<R> w;
+  WOf<R> w;
   R alpha;
   int h;
   uint32_t site;
@@ -51,7 +51,7 @@ struct HBCount {
 template <class R, bool MEAS>
 __device__ __forceinline__ int finish_deferred(const Deferred<R, MEAS>& d, uint4 ctr, const HBParams& hp,
                                                Quat<R>* out) {
-  R a0;
+  A0Of<R> a0;
   uint4 rt;
   const int n =
       sample_a0_from<R>(2, d.alpha, trial_inv2a(d.alpha), trial_e(d.alpha, hp.sampler), ctr, hp, &a0, &rt);
@@ -59,48 +59,58 @@ __device__ __forceinline__ int finish_deferred(const Deferred<R, MEAS>& d, uint4
   return n;
 }
 
+// Direction and parity of a substep: compile-time for FP32 / F16Q (MU, PAR >= 0,
+// so that every class index is a constant), run-time for FP64 (MU = PAR =
+// kRuntime; see staple_fixed).
+constexpr int kRuntime = -1;
+struct Substep { int mu, p; };
+template <int MU, int PAR> __device__ __forceinline__ Substep substep_of(const Substep& s) {
+  return Substep{MU >= 0 ? MU : s.mu, PAR >= 0 ? PAR : s.p};
+}
+
+// The addressing that goes with it.
+template <int P, int CP> constexpr int hb_addr = P == kF64 ? (int)kFlat : CP;
+// The template arguments of direction MU, parity PAR.
+template <int P, int MU> constexpr int hb_dir = P == kF64 ? kRuntime : MU;
+
 // Update link h of class (MU, PAR).  Rejected first trials go to queue slot
 // atomicAdd(qn, 1) when it is below CAP.  MCG: the staple's loads of the
 // other-parity MU class bypass L1 (the fused pair kernel writes that class
 // earlier in the same launch).  NC: read-only loads; the persistent batched
 // kernel, whose other CTAs write links during the launch, loads coherently.
 template <int P, int MU, bool MEAS, int PAR, bool MCG, int CAP, int CP, bool NC = true>
-__device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, int h, uint32_t tag, uint32_t sweep,
+__device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Substep sub, int h, uint32_t tag, uint32_t sweep,
                                         typename Real<P>::T beta, const HBParams& hp,
                                         Deferred<typename Real<P>::T, MEAS>* queue, int* qn,
                                         PlainAcc<typename Real<P>::T>& plaq, HBCount& cnt) {
-  constexpr int p = PAR;
+  sub = substep_of<MU, PAR>(sub);
+  const int mu = sub.mu, p = sub.p;
   using R = typename Real<P>::T;
-  using M = Math<R>;
   using Def = Deferred<R, MEAS>;
   const Site x = site_from_half(g, (uint32_t)h, p);
   Quat<R> lower;
-  Quat<R> sig;
-  if constexpr (MEAS) sig = staple_split<P, MU, NC, CP, MCG>(L, g, x, h, p, lower);
-  else sig = staple<P, MU, 0xF, NC, CP, MCG>(L, g, x, h, p);
+  const Frame<R> f = link_frame<P, MU, MEAS, NC, CP, MCG>(L, g, x, h, mu, p, beta, lower);
+  const R alpha = f.alpha;
   const uint32_t site = philox_site(g, x);
   const uint4 ctr = make_uint4(site, tag, sweep, 0u);
-  const R k2 = qdot(sig, sig);
-  const R invk = M::rsqrt(k2);
-  const R alpha = beta * k2 * invk;
   if (!(alpha >= R(1e-12))) {
     uint4 c = ctr;
     c.w = 1u;
     const Quat<R> nl = haar_from<R>(philox(c, hp.rk));
-    if constexpr (MEAS) plaq.add(qdot(L.put(2 * MU + p, h, nl), lower));
-    else L.st(2 * MU + p, h, nl);
+    if constexpr (MEAS) plaq.add(qdot(L.put(2 * mu + p, h, nl), lower));
+    else L.st(2 * mu + p, h, nl);
     cnt.haar += 1;
     return;
   }
   const R inv2a = trial_inv2a(alpha);
   const R e = trial_e(alpha, hp.sampler);
-  const Quat<R> w = qscale(sig, invk);
-  R a0;
+  const WOf<R> w = f.w;
+  A0Of<R> a0;
   uint4 rt;
   if (trial_a0<R>(alpha, inv2a, e, ctr, 1, hp, &a0, &rt)) {
     const Quat<R> nl = compose_link<R>(a0, w, ctr, rt, hp);
-    if constexpr (MEAS) plaq.add(qdot(L.put(2 * MU + p, h, nl), lower));
-    else L.st(2 * MU + p, h, nl);
+    if constexpr (MEAS) plaq.add(qdot(L.put(2 * mu + p, h, nl), lower));
+    else L.st(2 * mu + p, h, nl);
     cnt.trials += 1;
   } else if (hp.max_tries > 1) {
     const int slot = atomicAdd(qn, 1);
@@ -115,13 +125,13 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, in
     } else {
       Quat<R> nl;
       const int n = finish_deferred<R, MEAS>(d, ctr, hp, &nl);
-      if constexpr (MEAS) plaq.add(qdot(n ? L.put(2 * MU + p, h, nl) : ldl<P, NC>(L, 2 * MU + p, h), lower));
-      else if (n) L.st(2 * MU + p, h, nl);
+      if constexpr (MEAS) plaq.add(qdot(n ? L.put(2 * mu + p, h, nl) : ldl<P, NC>(L, 2 * mu + p, h), lower));
+      else if (n) L.st(2 * mu + p, h, nl);
       cnt.trials += n ? (unsigned)n : (unsigned)hp.max_tries;
       cnt.capped += n == 0;
     }
   } else {
-    if constexpr (MEAS) plaq.add(qdot(ldl<P, NC>(L, 2 * MU + p, h), lower));
+    if constexpr (MEAS) plaq.add(qdot(ldl<P, NC>(L, 2 * mu + p, h), lower));
     cnt.trials += 1;
     cnt.capped += 1;
   }
@@ -129,17 +139,18 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, in
 
 // Finish the queue entries i = threadIdx.x, threadIdx.x + blockDim.x, ... < n.
 template <int P, int MU, bool MEAS, int PAR, int CP, bool NC = true>
-__device__ __forceinline__ void hb_drain(const Links<P, CP>& L, const Deferred<typename Real<P>::T, MEAS>* queue, int n,
+__device__ __forceinline__ void hb_drain(const Links<P, CP>& L, Substep sub, const Deferred<typename Real<P>::T, MEAS>* queue, int n,
                                          uint32_t tag, uint32_t sweep, const HBParams& hp,
                                          PlainAcc<typename Real<P>::T>& plaq, HBCount& cnt) {
-  constexpr int p = PAR;
+  sub = substep_of<MU, PAR>(sub);
+  const int mu = sub.mu, p = sub.p;
   using R = typename Real<P>::T;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const Deferred<R, MEAS> d = queue[i];
     Quat<R> nl;
     const int t = finish_deferred<R, MEAS>(d, make_uint4(d.site, tag, sweep, 0u), hp, &nl);
-    if constexpr (MEAS) plaq.add(qdot(t ? L.put(2 * MU + p, d.h, nl) : ldl<P, NC>(L, 2 * MU + p, d.h), d.lower));
-    else if (t) L.st(2 * MU + p, d.h, nl);
+    if constexpr (MEAS) plaq.add(qdot(t ? L.put(2 * mu + p, d.h, nl) : ldl<P, NC>(L, 2 * mu + p, d.h), d.lower));
+    else if (t) L.st(2 * mu + p, d.h, nl);
     cnt.trials += t ? (unsigned)t : (unsigned)hp.max_tries;
     cnt.capped += t == 0;
   }
@@ -155,19 +166,37 @@ __device__ __forceinline__ void hb_drain(const Links<P, CP>& L, const Deferred<t
 // near 1e-15 and the update is stored as computed, like the oracle's.  NC:
 // read-only loads (no other block of the launch writes these links).
 template <int P, int MU, int PAR, bool NC, int CP>
-__device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, int h) {
-  constexpr int p = PAR;
+__device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Substep sub, int h) {
+  sub = substep_of<MU, PAR>(sub);
+  const int mu = sub.mu, p = sub.p;
   using R = typename Real<P>::T;
   using M = Math<R>;
   const Site x = site_from_half(g, (uint32_t)h, p);
-  const Quat<R> sig = staple<P, MU, 0xF, NC>(L, g, x, h, p);
+  const Quat<R> u = ldl<P, NC>(L, 2 * mu + p, h);
+  Quat<R> sig;
+  if constexpr (P == kF64) {
+    FixSum s;
+    FixBad bad{0u, 0u};
+    const bool ok = staple_fixed<false, NC, false>(L, g, x, h, mu, p, 4, s, sig);
+    const FixQuat ud = fix_of(u, -1, bad);
+    if (__builtin_expect(ok && fix_ok(bad), 1)) {
+      const Frame<R> f = staple_frame(s, 1.0);
+      if (f.alpha == 0.0) return;
+      s = fix_zero();
+      fix_mac(s, fix_mul(f.w, ud), f.w);
+      L.st(2 * mu + p, h, fix_sum_to_double(s));
+      return;
+    }
+    sig = staple_rolled<NC, false>(L, g, x, h, mu, p, 4, sig);
+  } else {
+    sig = staple<P, MU, 0xF, NC>(L, g, x, h, p);
+  }
   const R k2 = qdot(sig, sig);
   if (!(k2 >= M::kTiny)) return;
   const Quat<R> w = qscale(sig, M::rsqrt(k2));
-  const Quat<R> u = ldl<P, NC>(L, 2 * MU + p, h);
   Quat<R> v = qmul(qmul_nd(w, u), w);
   if constexpr (P != kF64) v = qscale(v, M::rsqrt(qdot(v, v)));
-  L.st(2 * MU + p, h, v);
+  L.st(2 * mu + p, h, v);
 }
 
 }  // namespace su2

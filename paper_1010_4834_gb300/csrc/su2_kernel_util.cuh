@@ -21,6 +21,41 @@ static int grid_for(K kernel, int64_t work, int smem = 0, int block = kThreads) 
   return (int)(g < 1 ? 1 : g);
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_pdl may start
+// while its predecessor in the stream still runs; pdl_wait() waits for the
+// predecessor to complete and its writes to be visible (a hardware wait), and
+// the kernel reads nothing that a predecessor writes before it.  pdl_trigger()
+// lets the next grid start (where it fits beside this one); it always comes
+// after pdl_wait(), so that when a grid starts, everything before its direct
+// predecessor is complete.  A kernel that can start beside a running
+// predecessor reads links by plain loads: a read-only load (ld.global.nc) is
+// for data that does not change while the kernel runs, and the compiler moves
+// it across the wait.  pdl_wait() returns a zero it cannot see through, which
+// goes into the kernel's indices.
+__device__ __forceinline__ int pdl_wait() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
+  return zero;
+}
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Whether a lattice's kernels overlap so.
+static inline bool overlaps(const LatticeView&) { return false; }
+
+template <class... KP, class... A>
+static cudaError_t launch_pdl(bool overlap, void (*kernel)(KP...), dim3 grid, int threads, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;   // else an ordinary launch, in which pdl_wait() returns at once
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ---------------------------------------------------------------------------
 // Reduction helpers
 // ---------------------------------------------------------------------------
@@ -50,11 +85,11 @@ template <class T> __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// Block-sum NV doubles into partials[block*NV + k]; returns true in the last
-// block to finish (all partials then visible to it).
+// Block-sum NV doubles into partials[slot*NV + k]; returns true in the last of
+// the nblocks blocks to finish (all partials then visible to it).
 template <int NV>
-__device__ __forceinline__ bool block_partial(double (&v)[NV], double* partials,
-                                              unsigned int* counter) {
+__device__ __forceinline__ bool block_partial(double (&v)[NV], double* partials, unsigned int* counter, int slot,
+                                              int nblocks) {
   __shared__ double sh[kThreads / 32][NV];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -70,12 +105,12 @@ __device__ __forceinline__ bool block_partial(double (&v)[NV], double* partials,
     for (int k = 0; k < NV; ++k) {
       double t = lane < kThreads / 32 ? sh[lane][k] : 0.0;
       t = warp_sum(t);
-      if (lane == 0) partials[(size_t)blockIdx.x * NV + k] = t;
+      if (lane == 0) partials[(size_t)slot * NV + k] = t;
     }
     if (lane == 0) {
       __threadfence();
       const unsigned int ticket = atomicAdd(counter, 1u);
-      last = (ticket == gridDim.x - 1);
+      last = (ticket == (unsigned int)nblocks - 1u);
     }
   }
   __syncthreads();
@@ -142,7 +177,7 @@ __device__ __forceinline__ void plaquette_from_block_sums(const double* meas, in
 #define SU2_HB_MINB 4
 #endif
 template <int P> struct Occ { static constexpr int hb = SU2_HB_MINB; };
-template <> struct Occ<kF64> { static constexpr int hb = 2; };
+template <> struct Occ<kF64> { static constexpr int hb = 3; };
 
 template <int P, int CP = kFlat> static Links<P, CP> links_of(void* base, int64_t vh) {
   Links<P, CP> L;

@@ -19,6 +19,7 @@
 #include "su2_hb_link.cuh"
 #include "su2_internal.h"
 #include "su2_kernel_util.cuh"
+#include "su2_measure.cuh"
 
 namespace su2 {
 
@@ -103,9 +104,10 @@ __global__ void __launch_bounds__(kThreads) k_init(Links<P> L, Geom g, int start
 // every link of direction MU and parity PAR.
 // ---------------------------------------------------------------------------
 template <int P, int MU, int PAR>
-__global__ void __launch_bounds__(kThreads, Occ<P>::hb) k_overrelax(Links<P, kClassPtr> L, Geom g) {
+__global__ void __launch_bounds__(kThreads, Occ<P>::hb)
+    k_overrelax(Links<P, hb_addr<P, kClassPtr>> L, Geom g, Substep sub) {
   const int stride = gridDim.x * blockDim.x;
-  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.vh; h += stride) or_link<P, MU, PAR, true>(L, g, h);
+  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.vh; h += stride) or_link<P, MU, PAR, true>(L, g, sub, h);
 }
 
 // ---------------------------------------------------------------------------
@@ -115,79 +117,21 @@ __global__ void __launch_bounds__(kThreads, Occ<P>::hb) k_overrelax(Links<P, kCl
 // out[0] all, out[1] spatial, out[2] space-time means.
 // ---------------------------------------------------------------------------
 template <int P>
-__device__ __forceinline__ typename Real<P>::T plaq(const Links<P>& L, int q, const Quat<typename Real<P>::T>& umu,
-                                                   const Quat<typename Real<P>::T>& unu, int mu, int nu,
-                                                   int h_pmu, int h_pnu) {
-  using R = typename Real<P>::T;
-  const Quat<R> a = qmul(umu, L.ld(2 * nu + q, h_pmu));
-  const Quat<R> b = qmul(unu, L.ld(2 * mu + q, h_pnu));
-  return qdot(a, b);
-}
-
-// The sixteen links one site's six plaquettes use: its own four and, for each
-// direction mu, the three U_nu(x + mu) with nu != mu.
-template <int P> struct PlaqLinks { Quat<typename Real<P>::T> u[4], n[4][3]; };
-
-template <int P>
-__device__ __forceinline__ void plaq_load(const Links<P>& L, const Geom& g, int s, PlaqLinks<P>& k, int& p) {
-  const Site x = site_from_index(g, (uint32_t)s);
-  p = parity(x);
-  const int q = p ^ 1;
-  const int h = s >> 1;
-  const int hm[4] = {hidx(g, shifted<0, +1>(g, x)), hidx(g, shifted<1, +1>(g, x)), hidx(g, shifted<2, +1>(g, x)),
-                     hidx(g, shifted<3, +1>(g, x))};
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) k.u[mu] = L.ld(2 * mu + p, h);
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int nu = j < mu ? j : j + 1;
-      k.n[mu][j] = L.ld(2 * nu + q, hm[mu]);
-    }
-  }
-}
-
-// U_nu(x + mu) among the loaded links.
-template <int P>
-__device__ __forceinline__ const Quat<typename Real<P>::T>& plaq_nb(const PlaqLinks<P>& k, int mu, int nu) {
-  return k.n[mu][nu < mu ? nu : nu - 1];
-}
-
-template <int P>
-__device__ __forceinline__ void plaq_sums(const PlaqLinks<P>& k, typename Real<P>::T& ss, typename Real<P>::T& ts) {
-  using R = typename Real<P>::T;
-  ss = R(0);
-  ts = R(0);
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-#pragma unroll
-    for (int nu = mu + 1; nu < 4; ++nu) {
-      const R v = qdot(qmul(k.u[mu], plaq_nb<P>(k, mu, nu)), qmul(k.u[nu], plaq_nb<P>(k, nu, mu)));
-      if (nu == 3) ts += v; else ss += v;
-    }
-  }
-}
-
-template <int P>
-__global__ void __launch_bounds__(kThreads) k_plaquette(Links<P> L, Geom g, int64_t s0, int64_t V,
-                                                        double* partials, unsigned int* counter, double* out) {
+__device__ __forceinline__ void plaquette_sum(const Links<P>& L, const Geom& g, int64_t s0, int64_t V, double* partials,
+                                              unsigned int* counter, double* out) {
   using R = typename Real<P>::T;
   Acc<R> sp, tm;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   // the plaquettes of the V sites from s0 on (all sites: s0 = 0, V = volume);
   // 64-bit loop index: V may come within one stride of 2^31
   for (int64_t s = s0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < s0 + V; s += stride) {
-    PlaqLinks<P> k0;
-    int p0;
-    plaq_load<P>(L, g, (int)s, k0, p0);
     R ss0, ts0;
-    plaq_sums<P>(k0, ss0, ts0);
+    plaq_site(L, g, (int)s, ss0, ts0);
     sp.add(ss0);
     tm.add(ts0);
   }
   double v[2] = {sp.value(), tm.value()};
-  if (block_partial<2>(v, partials, counter)) {
+  if (block_partial<2>(v, partials, counter, blockIdx.x, gridDim.x)) {
     double tot[2];
     final_sum<2>(partials, gridDim.x, tot);
     if (threadIdx.x == 0) {
@@ -198,6 +142,19 @@ __global__ void __launch_bounds__(kThreads) k_plaquette(Links<P> L, Geom g, int6
       *counter = 0;
     }
   }
+}
+
+template <int P>
+__global__ void __launch_bounds__(kThreads) k_plaquette(Links<P> L, Geom g, int64_t s0, int64_t V,
+                                                        double* partials, unsigned int* counter, double* out) {
+  plaquette_sum<P>(L, g, s0, V, partials, counter, out);
+}
+
+// FP64 at 128 registers a thread, two blocks an SM.
+template <>
+__global__ void __launch_bounds__(kThreads, 2) k_plaquette<kF64>(Links<kF64> L, Geom g, int64_t s0, int64_t V,
+                                                                 double* partials, unsigned int* counter, double* out) {
+  plaquette_sum<kF64>(L, g, s0, V, partials, counter, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -221,13 +178,12 @@ __global__ void __launch_bounds__(kThreads) k_plaquette(Links<P> L, Geom g, int6
 template <int P> struct PolyMinBlocks { static constexpr int value = 4; };
 template <> struct PolyMinBlocks<kF64> { static constexpr int value = 2; };
 
-template <int P>
+template <int P, bool NC>
 __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
     k_polyakov(Links<P, kClassPtr> L, Geom g, int lg, double* partials, unsigned int* counter, double* out,
-               SweepEpilogue ep) {
+               SweepEpilogue ep, int early) {
   using R = typename Real<P>::T;
   using LT = Links<P, kClassPtr>;
-  constexpr int C = 8;
   __shared__ Quat<R> seg_prod[kThreads];
   Acc<R> acc;
   const int nsig = g.n[0] * g.n[1] * g.n[2];
@@ -238,7 +194,9 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
   const int q = threadIdx.x / lines;
   const int l = threadIdx.x - q * lines;
   const int t0 = q * seg;
-  for (int first = blockIdx.x * lines; first < nsig; first += gridDim.x * lines) {
+  const int zero = pdl_wait();
+  if (early) pdl_trigger();
+  for (int first = blockIdx.x * lines + zero; first < nsig; first += gridDim.x * lines) {
     const int xs = first + l;
     Quat<R> pr = qone<R>();
     if (xs < nsig) {
@@ -250,15 +208,7 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
       const typename LT::E* b0 = swap ? L.cls_base(7) : L.cls_base(6);
       const typename LT::E* b1 = swap ? L.cls_base(6) : L.cls_base(7);
       const uint32_t e0 = hh + nsig_h * (uint32_t)t0;
-      int t = 0;
-      for (; t + C <= seg; t += C) {
-        Quat<R> u[C];
-#pragma unroll
-        for (int j = 0; j < C; ++j) u[j] = LT::ldp((j & 1) ? b1 : b0, e0 + nsig_h * (uint32_t)(t + j));
-#pragma unroll
-        for (int j = 0; j < C; ++j) pr = qmul(pr, u[j]);
-      }
-      for (; t < seg; ++t) pr = qmul(pr, LT::ldp((t & 1) ? b1 : b0, e0 + nsig_h * (uint32_t)t));
+      pr = time_line<P, kClassPtr, NC>(b0, b1, e0, nsig_h, seg);
     }
     if (G > 1) {
       seg_prod[threadIdx.x] = pr;
@@ -271,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
     if (q == 0 && xs < nsig) acc.add(pr.w);
   }
   double v[1] = {acc.value()};
-  if (block_partial<1>(v, partials, counter)) {
+  if (block_partial<1>(v, partials, counter, blockIdx.x, gridDim.x)) {
     double tot[1];
     final_sum<1>(partials, gridDim.x, tot);
     // every thread reads the counter here; thread 0 advances it only after
@@ -301,24 +251,25 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
 // three.  Each link's staple terms are added nu ascending, forward then
 // backward.  blockIdx.y = parity.
 // ---------------------------------------------------------------------------
-template <int P, int MU, int NU>
+template <int P, int MU, int NU, bool NC>
 __device__ __forceinline__ void ape_pair(const Links<P, kClassPtr>& L, int h, int p, const int (&dp)[3], const int (&dm)[3],
                                          const Quat<typename Real<P>::T>& umu, const Quat<typename Real<P>::T>& unu,
                                          Quat<typename Real<P>::T>& smu, Quat<typename Real<P>::T>& snu) {
   using R = typename Real<P>::T;
   const int q = p ^ 1;
-  const Quat<R> a = qmul_nd(L.ld(2 * NU + q, h + dp[MU]), L.ld(2 * MU + q, h + dp[NU]));
+  auto link = [&](int cls, int i) { return ldl<P, NC>(L, cls, i); };
+  const Quat<R> a = qmul_nd(link(2 * NU + q, h + dp[MU]), link(2 * MU + q, h + dp[NU]));
   const int hn = h + dm[NU], hm = h + dm[MU];  // x - nu, x - mu
   // link mu, term nu: forward U_nu(x) A^dag, backward U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
   qacc_mul_nd(smu, unu, a);
-  qacc_mul(smu, qmul_dn(L.ld(2 * NU + q, hn), L.ld(2 * MU + q, hn)), L.ld(2 * NU + p, hn + dp[MU]));
+  qacc_mul(smu, qmul_dn(link(2 * NU + q, hn), link(2 * MU + q, hn)), link(2 * NU + p, hn + dp[MU]));
   // link nu, term mu: forward U_mu(x) A, backward U_mu(x-mu)^dag U_nu(x-mu) U_mu(x-mu+nu)
   qacc_mul(snu, umu, a);
-  qacc_mul(snu, qmul_dn(L.ld(2 * MU + q, hm), L.ld(2 * NU + q, hm)), L.ld(2 * MU + p, hm + dp[NU]));
+  qacc_mul(snu, qmul_dn(link(2 * MU + q, hm), link(2 * NU + q, hm)), link(2 * MU + p, hm + dp[NU]));
 }
 
-template <int P>
-__device__ __forceinline__ void ape_store(const Links<P, kClassPtr>& dst, int cls, int h, const Quat<typename Real<P>::T>& u,
+template <int P, int CP>
+__device__ __forceinline__ void ape_store(const Links<P, CP>& dst, int cls, int h, const Quat<typename Real<P>::T>& u,
                                           const Quat<typename Real<P>::T>& sig, typename Real<P>::T c0,
                                           typename Real<P>::T c1) {
   using R = typename Real<P>::T;
@@ -333,38 +284,65 @@ __device__ __forceinline__ void ape_store(const Links<P, kClassPtr>& dst, int cl
 #endif
 // The sites of parity PAR (a template parameter, so every class index is a
 // compile-time constant for the per-class base pointers).
-template <int P, int PAR>
+template <int P, int PAR, bool NC>
 __device__ __forceinline__ void ape_sites(const Links<P, kClassPtr>& src, const Links<P, kClassPtr>& dst, const Geom& g,
-                                          typename Real<P>::T c0, typename Real<P>::T c1) {
+                                          typename Real<P>::T c0, typename Real<P>::T c1, int zero) {
   using R = typename Real<P>::T;
   constexpr int p = PAR;
   const int vh = (int)g.vh;
   const int stride = gridDim.x * blockDim.x;
-  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < vh; h += stride) {
+  for (int h = blockIdx.x * blockDim.x + threadIdx.x + zero; h < vh; h += stride) {
     const Site x = site_from_half(g, (uint32_t)h, p);
     // half-index steps to the six spatial neighbours; the index of x + a + b
     // is h + step(a) + step(b) for steps in different directions
     const int dp[3] = {half_step<0, +1>(g, x), half_step<1, +1>(g, x), half_step<2, +1>(g, x)};
     const int dm[3] = {half_step<0, -1>(g, x), half_step<1, -1>(g, x), half_step<2, -1>(g, x)};
-    const Quat<R> u0 = src.ld(0 + p, h), u1 = src.ld(2 + p, h), u2 = src.ld(4 + p, h);
+    const Quat<R> u0 = ldl<P, NC>(src, 0 + p, h), u1 = ldl<P, NC>(src, 2 + p, h), u2 = ldl<P, NC>(src, 4 + p, h);
     Quat<R> s0 = qmake<R>(0, 0, 0, 0), s1 = s0, s2 = s0;
-    ape_pair<P, 0, 1>(src, h, p, dp, dm, u0, u1, s0, s1);
-    ape_pair<P, 0, 2>(src, h, p, dp, dm, u0, u2, s0, s2);
-    ape_pair<P, 1, 2>(src, h, p, dp, dm, u1, u2, s1, s2);
+    ape_pair<P, 0, 1, NC>(src, h, p, dp, dm, u0, u1, s0, s1);
+    ape_pair<P, 0, 2, NC>(src, h, p, dp, dm, u0, u2, s0, s2);
+    ape_pair<P, 1, 2, NC>(src, h, p, dp, dm, u1, u2, s1, s2);
     ape_store<P>(dst, 0 + p, h, u0, s0, c0, c1);
     ape_store<P>(dst, 2 + p, h, u1, s1, c0, c1);
     ape_store<P>(dst, 4 + p, h, u2, s2, c0, c1);
   }
 }
 
-template <int P>
+// FP64: one link a thread, its four staples in fixed point (su2_fixed.cuh).
+// Sharing the forward products among a site's three links as above keeps three
+// sums of 16 registers and spilled 2 KB a thread; the nine further loads and
+// conversions cost less.
+template <bool NC>
+__device__ __forceinline__ void ape_links_fixed(const Links<kF64>& src, const Links<kF64>& dst, const Geom& g, int mu,
+                                                int p, double c0, double c1) {
+  const int vh = (int)g.vh;
+  const int stride = gridDim.x * blockDim.x;
+  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < vh; h += stride) {
+    const Site x = site_from_half(g, (uint32_t)h, p);
+    FixSum s;
+    Quat<double> sig;
+    if (__builtin_expect(staple_fixed<false, NC, false>(src, g, x, h, mu, p, 3, s, sig), 1))
+      sig = fix_sum_to_double(s);
+    else
+      sig = staple_rolled<NC, false>(src, g, x, h, mu, p, 3, sig);
+    ape_store<kF64>(dst, 2 * mu + p, h, ldl<kF64, NC>(src, 2 * mu + p, h), sig, c0, c1);
+  }
+}
+
+template <int P, bool NC>
 __global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : SU2_APE3_MINB)
-    k_ape(Links<P, kClassPtr> src, Links<P, kClassPtr> dst, Geom g, double alpha_d) {
+    k_ape(Links<P, hb_addr<P, kClassPtr>> src, Links<P, hb_addr<P, kClassPtr>> dst, Geom g, double alpha_d, int early) {
   using R = typename Real<P>::T;
+  const int zero = pdl_wait();
+  if (early) pdl_trigger();
   const R alpha = (R)alpha_d;
   const R c0 = R(1) - alpha, c1 = R(0.25) * alpha;
-  if (blockIdx.y == 0) ape_sites<P, 0>(src, dst, g, c0, c1);
-  else ape_sites<P, 1>(src, dst, g, c0, c1);
+  if constexpr (P == kF64) {
+    ape_links_fixed<NC>(src, dst, g, (int)(blockIdx.y >> 1) + zero, (int)(blockIdx.y & 1), c0, c1);
+  } else {
+    if (blockIdx.y == 0) ape_sites<P, 0, NC>(src, dst, g, c0, c1, zero);
+    else ape_sites<P, 1, NC>(src, dst, g, c0, c1, zero);
+  }
 }
 
 template <int P>
@@ -688,9 +666,11 @@ __global__ void __launch_bounds__(NTH, 1) k_wilson_rt(Links<P> Ls, Links<P> Lt, 
 
 // out[(R-1) tmax + (T-1)] from k_wilson_rt's per-block sums: one block per
 // output adds the gx blocks of its (R chunk, T chunk) in a fixed order.
+// excess: the sum of the time links' |U|^2 - 1 over all 1/inv terms in units of
+// 2^-58 (k_wilson_tg in FP64), or NULL.
 template <int RC>
 __global__ void __launch_bounds__(kThreads) k_wilson_rt_final(const double* partials, int gx, int ntc, int tmax,
-                                                              double inv, double* out) {
+                                                              double inv, const long long* excess, double* out) {
   const int o = blockIdx.x;
   const int r = o / tmax, t = o % tmax;
   const int y = (r / RC) * ntc + t / kWrtT;
@@ -698,7 +678,10 @@ __global__ void __launch_bounds__(kThreads) k_wilson_rt_final(const double* part
   double a = 0.0;
   for (int bx = threadIdx.x; bx < gx; bx += blockDim.x) a += __ldcg(partials + ((size_t)y * gx + bx) * (RC * kWrtT) + slot);
   const double tot = block_sum(a);
-  if (threadIdx.x == 0) out[o] = tot * inv;
+  if (threadIdx.x == 0) {
+    const double w = tot * inv;
+    out[o] = excess ? w + w * ((double)(t + 1) * ((double)*excess * 0x1p-58 * inv)) : w;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -744,29 +727,82 @@ constexpr int kTgT = 16;                 // T values in registers; also the rows
 constexpr int kTgChunks = 8;             // row chunks of a column (lanes per column)
 constexpr int kTgCols = 32 / kTgChunks;  // columns of a warp
 constexpr int kTgExt = kTgT / kTgChunks; // extended rows a lane owns
-// block size limit (the register budget): planes of up to 64 columns in
-// FP32 / F16Q, 32 in FP64
-template <int P> struct TgThreads { static constexpr int value = P == kF64 ? 256 : 512; };
+constexpr int kTgThreads = 512;          // planes of up to 64 columns
 
-template <class R> __device__ __forceinline__ Quat<R> qunit(const Quat<R>& q) {
-  return qscale(q, Math<R>::rsqrt(qdot(q, q)));
+// q / |q|.  Near |q| = 1 as q + q d, d = (1 - |q|^2) / 2 + ...: a scale factor is
+// itself rounded, to 2^-24 below 1 and 2^-23 above, and the approximate root's
+// error near 1 has one sign, which came back four times in every loop (16^4 FP32,
+// W to 8 x 8, off FP64: 7.8e-7 with the root, 4.1e-7 with a Newton step on it).
+__device__ __forceinline__ Quat<float> qunit(const Quat<float>& q) {
+  const float e = fmaf(-q.w, q.w, fmaf(-q.x, q.x, fmaf(-q.y, q.y, fmaf(-q.z, q.z, 1.0f))));
+  if (fabsf(e) > 0x1p-10f) return qscale(q, rsqrtf(qdot(q, q)));   // links set from outside
+  const float d = e * fmaf(0.375f, e, 0.5f);
+  return qmake<float>(fmaf(q.w, d, q.w), fmaf(q.x, d, q.x), fmaf(q.y, d, q.y), fmaf(q.z, d, q.z));
 }
 
-// Site (column a, slice t) of the plane (mu, c1, c2).
-__device__ __forceinline__ Site plane_site(const Geom& g, int mu, int a, int c1, int c2, int t) {
+// The kernel's arithmetic: FP32 quaternions with FP32 sums, or (FP64) the
+// 58-bit fixed point of su2_fixed.cuh with 64-bit sums in units of 2^-52 (one
+// plane's sum of one (R, T) and warp is below 2^60).  In fixed point a link
+// must be a unit quaternion to 2^-29 (`bad` is raised otherwise).  The gauge
+// transform normalises the time lines, whose links are unit quaternions only to
+// FP64 rounding (together about 1e-16 a link below one in a typical store, 1e-15
+// on a loop of T = 12); FP64 sums the time links' |U|^2 - 1 on the way (`excess`),
+// and the loops of extent T get the factor 1 + T <|U|^2 - 1> back.
+template <int P> struct TgMath {
+  using E = Quat<float>;
+  using A = float;
+  static __device__ __forceinline__ E load(const Links<P>& L, int cls, int h, bool&) { return L.ld(cls, h); }
+  static __device__ __forceinline__ int64_t excess(const E&) { return 0; }
+  static __device__ __forceinline__ E one() { return qone<float>(); }
+  static __device__ __forceinline__ E mul(const E& a, const E& b) { return qmul(a, b); }
+  static __device__ __forceinline__ E mul_nd(const E& a, const E& b) { return qmul_nd(a, b); }
+  static __device__ __forceinline__ E unit(const E& q) { return qunit(q); }
+  static __device__ __forceinline__ A dot(const E& a, const E& b, A s) {
+    return fma(a.w, b.w, fma(a.x, b.x, fma(a.y, b.y, fma(a.z, b.z, s))));
+  }
+  static __device__ __forceinline__ double value(A s) { return (double)s; }
+};
+
+template <> struct TgMath<kF64> {
+  using E = FixQuat;
+  using A = int64_t;
+  static __device__ __forceinline__ E load(const Links<kF64>& L, int cls, int h, bool& bad) {
+    return fix_unit_link(L.ld(cls, h), bad);
+  }
+  // |q|^2 - 1 in units of 2^-58
+  static __device__ __forceinline__ int64_t excess(const E& q) { return fix_dot(q, q, -((int64_t)1 << kFixFrac)); }
+  static __device__ __forceinline__ E one() { return fix_one(); }
+  static __device__ __forceinline__ E mul(const E& a, const E& b) { return fix_mul(a, b); }
+  static __device__ __forceinline__ E mul_nd(const E& a, const E& b) {
+    return fix_mul(a, fix_conj(b));
+  }
+  // q (3 - |q|^2) / 2: one Newton step, enough while |q|^2 is within 2^-26 of one
+  static __device__ __forceinline__ Fix scaled(const Fix& a, int e) {
+    return fix_split(fix_value(a) + (((int64_t)a.h * e) >> kFixLow));
+  }
+  static __device__ __forceinline__ E unit(const E& q) {
+    const int e = (int)(-fix_dot(q, q, -((int64_t)1 << kFixFrac)) >> 1);
+    return E{scaled(q.w, e), scaled(q.x, e), scaled(q.y, e), scaled(q.z, e)};
+  }
+  static __device__ __forceinline__ A dot(const E& a, const E& b, A s) { return s + (fix_dot(a, b, 32) >> 6); }
+  static __device__ __forceinline__ double value(A s) { return fix_to_double<52>(s); }
+};
+
+// Site (column a, slice 0) of the plane (mu, c1, c2).
+__device__ __forceinline__ Site plane_site(const Geom& g, int mu, int a, int c1, int c2) {
   Site y;
   y.x0 = mu == 0 ? a : c1;
   y.x1 = mu == 0 ? c1 : (mu == 1 ? a : c2);
   y.x2 = mu == 2 ? a : c2;
-  y.x3 = t;
-  y.row = y.x1 + g.n[1] * (y.x2 + g.n[2] * y.x3);
+  y.x3 = 0;
+  y.row = y.x1 + g.n[1] * y.x2;
   return y;
 }
 
 // Row layout of a staged plane, chunks of RO rows.  Eight lanes of a 16-byte
 // shared access are two chunks of four columns, so rows c RO + i and
 // (c+1) RO + i must start 4 mod 8 quaternions apart (16 banks), and so must
-// the extended rows Nt + 2c + e and Nt + 2c + 2 + e.  The latter needs a
+// the extended rows 2c + e and 2c + 2 + e.  The latter needs a
 // row stride S = 2 mod 4; the former then holds for RO = 2 mod 4 and, with
 // the origin rows of odd chunks shifted by tg_skew_unit quaternions, for RO
 // = 0 mod 4 (shift 4) and RO odd (S = 2 mod 8, shift 2).  S leaves room for
@@ -777,25 +813,39 @@ template <int RO> __host__ __device__ __forceinline__ int tg_stride(int cols) {
   const int lo = cols + tg_skew_unit<RO>();
   return lo + ((2 - lo % m) + m) % m;
 }
-template <int RO> __device__ __forceinline__ int tg_row(int r, int nt, int stride) {
-  return r * stride + (r < nt ? tg_skew_unit<RO>() * ((r / RO) & 1) : 0);
+// row r of the staged plane: kTgChunks RO origin rows, then the extended ones
+template <int RO> __device__ __forceinline__ int tg_row(int r, int stride) {
+  return r * stride + (r < kTgChunks * RO ? tg_skew_unit<RO>() * ((r / RO) & 1) : 0);
 }
 
-template <int P, int RO>
-__global__ void __launch_bounds__(TgThreads<P>::value, 1)
-    k_wilson_tg(Links<P> Ls, Links<P> Lt, Geom g, int rmax, int tmax, double* partials) {
-  using R = typename Real<P>::T;
-  constexpr int NTH = TgThreads<P>::value;
+// EXACT: Nt is a multiple of eight (every origin row starts loops), compiled
+// without the tests.
+template <int P, int RO, bool EXACT>
+__global__ void __launch_bounds__(kTgThreads, 1)
+    k_wilson_tg(Links<P> Ls, Links<P> Lt, Geom g, int rmax, int tmax, double* partials, double* flag,
+                unsigned long long* excess) {
+  using M = TgMath<P>;
+  using E = typename M::E;
+  using A = typename M::A;
+  constexpr int NO = kTgChunks * RO;               // origin rows, at least Nt
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double acc64[16 * kTgT];              // block totals; slot (R-1) kTgT + T-1
-  __shared__ R wsum[16][NTH / 32][kTgT];           // per R and warp
+  __shared__ A wsum[16][kTgThreads / 32][kTgT];    // per R and warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nt = g.n[3], nr = nt + kTgT;           // nt = kTgChunks RO
+  const int nt = g.n[3];
   const int hts = g.n0h * g.st[3];
   for (int i = threadIdx.x; i < 16 * kTgT; i += blockDim.x) acc64[i] = 0.0;
   const int ntr0 = g.n[1] * g.n[2], ntr1 = g.n[0] * g.n[2], ntr2 = g.n[0] * g.n[1];
   const int nunits = ntr0 + ntr1 + ntr2;
   const int c = lane / kTgCols, r0 = c * RO;
+  bool bad = false;
+  int64_t over = 0;
+  // slice of row r: rows past the last slice repeat the first ones
+  auto slice = [&](int r) {
+    if constexpr (EXACT) return r < nt ? r : (r - NO) % nt;
+    while (r >= nt) r -= nt;
+    return r;
+  };
   for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
     const int mu = u < ntr0 ? 0 : (u < ntr0 + ntr1 ? 1 : 2);
     const int tr = u - (mu == 0 ? 0 : (mu == 1 ? ntr0 : ntr0 + ntr1));
@@ -804,74 +854,69 @@ __global__ void __launch_bounds__(TgThreads<P>::value, 1)
     const int c1 = tr % n1st, c2 = tr / n1st;
     const int W = nm + rmax - 1;       // columns of the staged plane (column cc is plane column cc mod nm)
     const int SU = tg_stride<RO>(W), SS = tg_stride<RO>(nm);
-    Quat<R>* Ue = reinterpret_cast<Quat<R>*>(smem_raw);  // Ue[tg_row(r, SU) + cc] = U'(cc, r), r < nr
-    Quat<R>* Sb = Ue + nr * SU + 4;                      // Sb[tg_row(r, SS) + a]: G(a, r), then S'_R(a, r)
-    Quat<R>* Ct = Sb + nr * SS + 4;                      // Ct[k nm + a]: product of scan chunk k
-    Quat<R>* Pb = Ct + kTgChunks * nm;                   // Pb[a] = P(a)
+    E* Ue = reinterpret_cast<E*>(smem_raw);      // Ue[tg_row(r, SU) + cc] = U'(cc, r), r < NO + kTgT
+    E* Sb = Ue + (NO + kTgT) * SU + 4;           // Sb[tg_row(r, SS) + a]: G(a, r), then S'_R(a, r)
+    E* Ct = Sb + (NO + kTgT) * SS + 4;           // Ct[k nm + a]: product of scan chunk k
+    E* Pb = Ct + kTgChunks * nm;                 // Pb[a] = P(a)
     const int a = kTgCols * warp + lane % kTgCols;
     const bool active = a < nm;
     __syncthreads();  // the previous plane's readers are done
     // (1) this lane's links, loaded together: the time and spatial links of
-    // its origin rows (one site each) and the spatial links of the slices
-    // 2c, 2c + 1 that its extended rows repeat; then the time links'
-    // products within the chunk
-    Quat<R> us[RO + kTgExt];
+    // its origin rows and the spatial links that its extended rows repeat;
+    // then the time links' products within the chunk
+    E us[RO + kTgExt];
     if (active) {
-      Quat<R> ut[RO];
-      const Site y = plane_site(g, mu, a, c1, c2, r0);
-      int h = hidx(g, y), par = parity(y);
+      E ut[RO];
+      const Site y = plane_site(g, mu, a, c1, c2);
+      const int h0 = hidx(g, y), par0 = parity(y);
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
-        ut[i] = Lt.ld(6 + par, h);
-        us[i] = Ls.ld(2 * mu + par, h);
-        h += hts;
-        par ^= 1;
+        const int t = slice(r0 + i), h = h0 + hts * t, par = (par0 ^ t) & 1;
+        ut[i] = EXACT || r0 + i < nt ? M::load(Lt, 6 + par, h, bad) : M::one();
+        over += M::excess(ut[i]);
+        us[i] = M::load(Ls, 2 * mu + par, h, bad);
       }
 #pragma unroll
       for (int e = 0; e < kTgExt; ++e) {
-        const Site ye = plane_site(g, mu, a, c1, c2, (kTgExt * c + e) % nt);
-        us[RO + e] = Ls.ld(2 * mu + parity(ye), hidx(g, ye));
+        const int t = slice(NO + kTgExt * c + e), h = h0 + hts * t, par = (par0 ^ t) & 1;
+        us[RO + e] = M::load(Ls, 2 * mu + par, h, bad);
       }
-      Quat<R> L = qone<R>();
+      E L = M::one();
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
-        Sb[tg_row<RO>(r0 + i, nt, SS) + a] = L;
-        L = qunit(qmul(L, ut[i]));
+        Sb[tg_row<RO>(r0 + i, SS) + a] = L;
+        L = M::unit(M::mul(L, ut[i]));
       }
       Ct[c * nm + a] = L;
     }
     __syncthreads();
     // (2) prefix over the chunks: G(a, r) for the thread's rows, P(a) = G(a, Nt)
     if (active) {
-      Quat<R> Q = qone<R>();
-      for (int k = 0; k < c; ++k) Q = qunit(qmul(Q, Ct[k * nm + a]));
+      E Q = M::one();
+      for (int k = 0; k < c; ++k) Q = M::unit(M::mul(Q, Ct[k * nm + a]));
       if (c > 0) {
 #pragma unroll
         for (int i = 0; i < RO; ++i) {
-          Quat<R>* p = Sb + tg_row<RO>(r0 + i, nt, SS) + a;
-          *p = qunit(qmul(Q, *p));
+          E* p = Sb + tg_row<RO>(r0 + i, SS) + a;
+          *p = M::unit(M::mul(Q, *p));
         }
       }
-      if (c == kTgChunks - 1) Pb[a] = qunit(qmul(Q, Ct[c * nm + a]));
+      if (c == kTgChunks - 1) Pb[a] = M::unit(M::mul(Q, Ct[c * nm + a]));
     }
     __syncthreads();
     // (3) U'(a, r) = G(a, t) U_mu(a, t) G(a+1, t)^dag for the lane's rows,
-    // conjugated by P on its extended rows; column a + nm (a < rmax - 1)
-    // repeats column a
+    // conjugated by P on the rows past the last slice; column a + nm (a <
+    // rmax - 1) repeats column a
     if (active) {
       const int an = a + 1 == nm ? 0 : a + 1;
-      const bool dup = a < rmax - 1;
 #pragma unroll
       for (int i = 0; i < RO + kTgExt; ++i) {
-        const bool ext = i >= RO;
-        const int t = ext ? (kTgExt * c + (i - RO)) % nt : r0 + i;
-        const int r = ext ? nt + kTgExt * c + (i - RO) : r0 + i;
-        const int gt = tg_row<RO>(t, nt, SS);
-        Quat<R> v = qmul_nd(qmul(Sb[gt + a], us[i]), Sb[gt + an]);
-        if (ext) v = qmul_nd(qmul(Pb[a], v), Pb[an]);
-        const int ru = tg_row<RO>(r, nt, SU);
-        Ue[ru + a] = v;
-        if (dup) Ue[ru + a + nm] = v;
+        const int r = i < RO ? r0 + i : NO + kTgExt * c + (i - RO);
+        const int gt = tg_row<RO>(slice(r), SS);
+        E v = M::mul_nd(M::mul(Sb[gt + a], us[i]), Sb[gt + an]);
+        if (EXACT ? i >= RO : r >= nt) v = M::mul_nd(M::mul(Pb[a], v), Pb[an]);
+        const int ru = tg_row<RO>(r, SU);
+        for (int cc = a; cc < W; cc += nm) Ue[ru + cc] = v;
       }
     }
     __syncthreads();  // Sb now holds lines
@@ -880,51 +925,52 @@ __global__ void __launch_bounds__(TgThreads<P>::value, 1)
     constexpr int unit = tg_skew_unit<RO>();
     const int sk = unit * (c & 1);
     const int bu = r0 * SU + sk + a, bs = r0 * SS + sk + a;
-    const int bue = (nt + kTgExt * c) * SU + a, bse = (nt + kTgExt * c) * SS + a;
-    Quat<R> own[RO];  // the origin rows' lines; the extended rows' stay in Sb
-    R acc[kTgT];
+    const int bue = (NO + kTgExt * c) * SU + a, bse = (NO + kTgExt * c) * SS + a;
+    const int rows = nt - r0;  // loops start from the first `rows` of the lane's origin rows
+    E own[RO];  // the origin rows' lines; the extended rows' stay in Sb
+    A acc[kTgT];
 #pragma unroll
-    for (int k = 0; k < kTgT; ++k) acc[k] = R(0);
+    for (int k = 0; k < kTgT; ++k) acc[k] = A(0);
     for (int Rl = 1; Rl <= rmax; ++Rl) {
       if (active) {
 #pragma unroll
         for (int i = 0; i < RO; ++i) {
-          const Quat<R> v = Ue[bu + i * SU + Rl - 1];
-          own[i] = Rl == 1 ? v : qmul(own[i], v);
+          const E v = Ue[bu + i * SU + Rl - 1];
+          own[i] = Rl == 1 ? v : M::mul(own[i], v);
           Sb[bs + i * SS] = own[i];
         }
 #pragma unroll
         for (int e = 0; e < kTgExt; ++e) {
-          const Quat<R> v = Ue[bue + e * SU + Rl - 1];
-          Quat<R>* p = Sb + bse + e * SS;
-          *p = Rl == 1 ? v : qmul(*p, v);
+          const E v = Ue[bue + e * SU + Rl - 1];
+          E* p = Sb + bse + e * SS;
+          *p = Rl == 1 ? v : M::mul(*p, v);
         }
       }
       __syncwarp();
       if (active) {
         // origin rows r0 + i, i < RO, against rows r0 + j, j = i + T; the
-        // benchmark's T range (all sixteen) takes a copy without the T test
+        // common case, all sixteen T and Nt a multiple of eight, takes a copy
+        // without the tests
         auto dots = [&](auto full_c) {
           constexpr bool FULL = decltype(full_c)::value;
 #pragma unroll
           for (int j = 1; j < RO + kTgT; ++j) {
-            Quat<R> w;
+            if (!FULL && j >= RO + tmax) break;
+            E w;
             if (j < RO) {
               w = own[j < RO ? j : 0];
             } else {
-              const int rr = r0 + j;  // chunk c + j / RO while below Nt
-              w = Sb[rr * SS + (rr < nt ? unit * ((c + j / RO) & 1) : 0) + a];
+              const int rr = r0 + j;  // chunk c + j / RO while an origin row
+              w = Sb[rr * SS + (rr < NO ? unit * ((c + j / RO) & 1) : 0) + a];
             }
 #pragma unroll
             for (int i = 0; i < RO; ++i) {
               const int T = j - i;
-              if (T >= 1 && T <= kTgT && (FULL || T <= tmax))
-                acc[T - 1] =
-                    fma(own[i].w, w.w, fma(own[i].x, w.x, fma(own[i].y, w.y, fma(own[i].z, w.z, acc[T - 1]))));
+              if (T >= 1 && T <= kTgT && (FULL || (T <= tmax && (EXACT || i < rows)))) acc[T - 1] = M::dot(own[i], w, acc[T - 1]);
             }
           }
         };
-        if (tmax == kTgT) dots(std::true_type{});
+        if (EXACT && tmax == kTgT) dots(std::true_type{});
         else dots(std::false_type{});
       }
       __syncwarp();  // the lines are read before the next R overwrites them
@@ -938,8 +984,8 @@ __global__ void __launch_bounds__(TgThreads<P>::value, 1)
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
           if (m < half) {
-            const R send = upper ? acc[m] : acc[m + half];
-            const R keep = upper ? acc[m + half] : acc[m];
+            const A send = upper ? acc[m] : acc[m + half];
+            const A keep = upper ? acc[m + half] : acc[m];
             acc[m] = keep + __shfl_xor_sync(0xffffffffu, send, off);
           }
         }
@@ -948,16 +994,21 @@ __global__ void __launch_bounds__(TgThreads<P>::value, 1)
       acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
       if ((lane & 1) == 0) wsum[Rl - 1][warp][lo] = acc[0];
 #pragma unroll
-      for (int k = 0; k < kTgT; ++k) acc[k] = R(0);
+      for (int k = 0; k < kTgT; ++k) acc[k] = A(0);
     }
     __syncthreads();
     // the plane's sums, warps in a fixed order
     const int nw = (int)(blockDim.x >> 5);
     for (int s = threadIdx.x; s < rmax * kTgT; s += blockDim.x) {
       double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += (double)wsum[s / kTgT][w][s % kTgT];
+      for (int w = 0; w < nw; ++w) t += M::value(wsum[s / kTgT][w][s % kTgT]);
       acc64[s] += t;
     }
+  }
+  if (bad) *flag = 1.0;
+  if constexpr (P == kF64) {
+    over = warp_sum(over);
+    if (lane == 0) atomicAdd(excess, (unsigned long long)over);   // exact in any order
   }
   __syncthreads();
   for (int i = threadIdx.x; i < 16 * kTgT; i += blockDim.x) partials[(size_t)blockIdx.x * 16 * kTgT + i] = acc64[i];
@@ -1032,14 +1083,12 @@ cudaError_t launch_init(const LatticeView& v, int start, PhiloxKey key, uint32_t
 
 cudaError_t launch_overrelax(const LatticeView& v, int mu, int parity, cudaStream_t st) {
   SU2_DISPATCH(v.prec, SU2_DISPATCH_MU(mu, {
-    auto L = links_of<P, kClassPtr>(v.links, v.g.vh);
-    if (parity == 0) {
-      const int gr = grid_for(k_overrelax<P, MU, 0>, v.g.vh);
-      k_overrelax<P, MU, 0><<<gr, kThreads, 0, st>>>(L, v.g);
-    } else {
-      const int gr = grid_for(k_overrelax<P, MU, 1>, v.g.vh);
-      k_overrelax<P, MU, 1><<<gr, kThreads, 0, st>>>(L, v.g);
-    }
+    auto L = links_of<P, hb_addr<P, kClassPtr>>(v.links, v.g.vh);
+    auto launch = [&](auto kernel) {
+      kernel<<<grid_for(kernel, v.g.vh), kThreads, 0, st>>>(L, v.g, Substep{mu, parity});
+    };
+    if (parity == 0) launch(k_overrelax<P, hb_dir<P, MU>, hb_dir<P, 0>>);
+    else launch(k_overrelax<P, hb_dir<P, MU>, hb_dir<P, 1>>);
   }));
   count_launches(1);
   return cudaGetLastError();
@@ -1101,8 +1150,12 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
     // and leaves segments of at least 8 links
     int lg = 0;
     while (lg < 3 && v.g.n[3] % (2 << lg) == 0 && v.g.n[3] / (2 << lg) >= 8) ++lg;
-    const int gr = grid_for(k_polyakov<P>, nsig << lg);
-    k_polyakov<P><<<gr, kThreads, 0, st>>>(L, v.g, lg, s.partials, s.counter, s.out, e);
+    auto launch = [&](auto kernel) {
+      const int gr = grid_for(kernel, nsig << lg);
+      return launch_pdl(overlaps(v), kernel, dim3(gr), kThreads, st, L, v.g, lg, s.partials, s.counter, s.out, e, (int)overlaps(v));
+    };
+    const cudaError_t err = overlaps(v) ? launch(k_polyakov<P, false>) : launch(k_polyakov<P, true>);
+    if (err != cudaSuccess) return err;
   });
   count_launches(1);
   return cudaGetLastError();
@@ -1110,12 +1163,17 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
 
 cudaError_t launch_ape(const LatticeView& src, void* dst, double alpha, cudaStream_t st) {
   SU2_DISPATCH(src.prec, {
-    auto S = links_of<P, kClassPtr>(src.links, src.g.vh);
-    auto D = links_of<P, kClassPtr>(dst, src.g.vh);
-    // two y-slices (one per parity) share the machine
-    int gx = grid_for(k_ape<P>, 2 * src.g.vh) / 2;
-    if (gx < 1) gx = 1;
-    k_ape<P><<<dim3(gx, 2), kThreads, 0, st>>>(S, D, src.g, alpha);
+    auto S = links_of<P, hb_addr<P, kClassPtr>>(src.links, src.g.vh);
+    auto D = links_of<P, hb_addr<P, kClassPtr>>(dst, src.g.vh);
+    // the y-slices (parities; in FP64 link classes) share the machine
+    const int slices = P == kF64 ? 6 : 2;
+    auto launch = [&](auto kernel) {
+      int gx = grid_for(kernel, slices * src.g.vh) / slices;
+      if (gx < 1) gx = 1;
+      return launch_pdl(overlaps(src), kernel, dim3(gx, slices), kThreads, st, S, D, src.g, alpha, (int)overlaps(src));
+    };
+    const cudaError_t e = overlaps(src) ? launch(k_ape<P, false>) : launch(k_ape<P, true>);
+    if (e != cudaSuccess) return e;
   });
   count_launches(1);
   return cudaGetLastError();
@@ -1180,7 +1238,7 @@ static cudaError_t launch_wilson_rt_rc(const LatticeView& v, const void* spatial
   count_launches(1);
   const int64_t V = 2 * v.g.vh;
   k_wilson_rt_final<RC><<<rmax * tmax, kThreads, 0, st>>>(s.partials, (int)gx, ntc, tmax, 1.0 / (3.0 * (double)V),
-                                                          s.out);
+                                                          nullptr, s.out);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1216,30 +1274,28 @@ static cudaError_t launch_wilson_rt(const LatticeView& v, const void* spatial, i
   return cudaErrorInvalidValue;
 }
 
-// The temporal-gauge kernel when R and T are at most 16, Nt is a multiple of
-// 8 with Nt / 8 in {1, 2, 4, 6, 8}, one block holds four columns a warp of
-// the widest plane, and the staged plane fits in shared memory; *used =
-// false otherwise.
-template <int P, int RO>
+// The temporal-gauge kernel when R and T are at most 16, Nt is at most 64, one
+// block holds four columns a warp of the widest plane, and the staged plane
+// fits in shared memory; *used = false otherwise.
+template <int P, int RO, bool EXACT>
 static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                                         const Scratch& s, cudaStream_t st, bool* used) {
-  using R = typename Real<P>::T;
-  constexpr int kMaxThreads = TgThreads<P>::value;
+                                         const Scratch& s, double* flag, cudaStream_t st, bool* used) {
+  using E = typename TgMath<P>::E;
   *used = false;
   const int nmax = std::max(v.g.n[0], std::max(v.g.n[1], v.g.n[2]));
-  const int nt = v.g.n[3], nr = nt + kTgT;
+  const int nr = kTgChunks * RO + kTgT;
   const int nth = (nmax + kTgCols - 1) / kTgCols * 32;
-  if (nth > kMaxThreads) return cudaSuccess;
+  if (nth > kTgThreads) return cudaSuccess;
   int dev = 0;
   cudaGetDevice(&dev);
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, k_wilson_tg<P, RO>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, k_wilson_tg<P, RO, EXACT>);
   if (e != cudaSuccess) return e;
   const int64_t smem = ((int64_t)nr * tg_stride<RO>(nmax + rmax - 1) + 4 + (int64_t)nr * tg_stride<RO>(nmax) + 4 +
                         (int64_t)kTgChunks * nmax + nmax) *
-                       (int64_t)sizeof(Quat<R>);
+                       (int64_t)sizeof(E);
   const int64_t dyn_max = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
   if (smem > dyn_max) return cudaSuccess;
   // raised once per device, as for the time-outer kernel
@@ -1248,12 +1304,12 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   if (dev >= 0 && dev < 64) {
     const int lim = (int)dyn_max;
     std::call_once(attr_once[dev], [dev, lim]() {
-      attr_err[dev] = cudaFuncSetAttribute(k_wilson_tg<P, RO>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      attr_err[dev] = cudaFuncSetAttribute(k_wilson_tg<P, RO, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     });
     if (attr_err[dev] != cudaSuccess) return attr_err[dev];
   }
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wilson_tg<P, RO>, nth, (size_t)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wilson_tg<P, RO, EXACT>, nth, (size_t)smem);
   if (per_sm < 1) per_sm = 1;
   const int64_t nunits = (int64_t)v.g.n[1] * v.g.n[2] + (int64_t)v.g.n[0] * v.g.n[2] + (int64_t)v.g.n[0] * v.g.n[1];
   int64_t gx = (int64_t)device_info().sms * per_sm;
@@ -1263,39 +1319,51 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   *used = true;
   auto Lt = links_of<P>(v.links, v.g.vh);
   auto Ls = links_of<P>(const_cast<void*>(spatial), v.g.vh);
-  k_wilson_tg<P, RO><<<(unsigned)gx, nth, (size_t)smem, st>>>(Ls, Lt, v.g, rmax, tmax, s.partials);
+  // a word of the counters' 256 bytes, away from the reductions' own
+  unsigned long long* excess = P == kF64 ? reinterpret_cast<unsigned long long*>(s.counter + 32) : nullptr;
+  if (excess) e = cudaMemsetAsync(excess, 0, sizeof *excess, st);
+  if (e != cudaSuccess) return e;
+  k_wilson_tg<P, RO, EXACT><<<(unsigned)gx, nth, (size_t)smem, st>>>(Ls, Lt, v.g, rmax, tmax, s.partials, flag, excess);
   count_launches(1);
   const int64_t V = 2 * v.g.vh;
   k_wilson_rt_final<16><<<rmax * tmax, kThreads, 0, st>>>(s.partials, (int)gx, 1, tmax, 1.0 / (3.0 * (double)V),
-                                                          s.out);
+                                                          reinterpret_cast<const long long*>(excess), s.out);
   count_launches(1);
   return cudaGetLastError();
 }
 
 template <int P>
 static cudaError_t launch_wilson_tg(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                                    const Scratch& s, cudaStream_t st, bool* used) {
+                                    const Scratch& s, double* flag, cudaStream_t st, bool* used) {
   *used = false;
-  const int nt = v.g.n[3];
-  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || nt % kTgChunks != 0) return cudaSuccess;
-  switch (nt / kTgChunks) {
-    case 1: return launch_wilson_tg_rows<P, 1>(v, spatial, rmax, tmax, s, st, used);
-    case 2: return launch_wilson_tg_rows<P, 2>(v, spatial, rmax, tmax, s, st, used);
-    case 4: return launch_wilson_tg_rows<P, 4>(v, spatial, rmax, tmax, s, st, used);
-    case 6: return launch_wilson_tg_rows<P, 6>(v, spatial, rmax, tmax, s, st, used);
-    case 8: return launch_wilson_tg_rows<P, 8>(v, spatial, rmax, tmax, s, st, used);
+  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || (P == kF64 && !flag)) return cudaSuccess;
+  auto launch = [&](auto rows) -> cudaError_t {
+    constexpr int RO = decltype(rows)::value;
+    if (P != kF64 && v.g.n[3] == kTgChunks * RO)
+      return launch_wilson_tg_rows<P, RO, P != kF64>(v, spatial, rmax, tmax, s, flag, st, used);
+    return launch_wilson_tg_rows<P, RO, false>(v, spatial, rmax, tmax, s, flag, st, used);
+  };
+  switch ((v.g.n[3] + kTgChunks - 1) / kTgChunks) {
+    case 1: return launch(std::integral_constant<int, 1>{});
+    case 2: return launch(std::integral_constant<int, 2>{});
+    case 3: return launch(std::integral_constant<int, 3>{});
+    case 4: return launch(std::integral_constant<int, 4>{});
+    case 5: return launch(std::integral_constant<int, 5>{});
+    case 6: return launch(std::integral_constant<int, 6>{});
+    case 7: return launch(std::integral_constant<int, 7>{});
+    case 8: return launch(std::integral_constant<int, 8>{});
     default: return cudaSuccess;
   }
 }
 
 cudaError_t launch_wilson(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                          const Scratch& s, cudaStream_t st) {
+                          const Scratch& s, double* flag, cudaStream_t st) {
   if (rmax < 1 || rmax > kWilsonMaxR || tmax < 1) return cudaErrorInvalidValue;
   {
     bool used = false;
     cudaError_t e = cudaSuccess;
     SU2_DISPATCH(v.prec, {
-      e = launch_wilson_tg<P>(v, spatial, rmax, tmax, s, st, &used);
+      e = launch_wilson_tg<P>(v, spatial, rmax, tmax, s, flag, st, &used);
       if (e == cudaSuccess && !used) e = launch_wilson_rt<P>(v, spatial, rmax, tmax, s, st, &used);
     });
     if (e != cudaSuccess || used) return e;

@@ -195,20 +195,20 @@ __global__ void __launch_bounds__(kPairThreads, kPairBlocksPerSM)
 #pragma unroll
       for (int k = 0; k < kPairLinksPerThread; ++k) {
         const int h = h0 + k * BS + (int)threadIdx.x;
-        if (h < h1) hb_link<P, MU, false, 0, false, CAP>(L, g, h, tag, sweep, beta, hp,
+        if (h < h1) hb_link<P, MU, false, 0, false, CAP>(L, g, Substep{MU, 0}, h, tag, sweep, beta, hp,
                                                          reinterpret_cast<Deferred<R, false>*>(queue), &qn, plaq, cnt);
       }
       __syncthreads();
-      hb_drain<P, MU, false, 0>(L, reinterpret_cast<Deferred<R, false>*>(queue), min(qn, CAP), tag, sweep, hp, plaq,
+      hb_drain<P, MU, false, 0>(L, Substep{MU, 0}, reinterpret_cast<Deferred<R, false>*>(queue), min(qn, CAP), tag, sweep, hp, plaq,
                                 cnt);
     } else {
 #pragma unroll
       for (int k = 0; k < kPairLinksPerThread; ++k) {
         const int h = h0 + k * BS + (int)threadIdx.x;
-        if (h < h1) hb_link<P, MU, MEAS, 1, true, CAP>(L, g, h, tag, sweep, beta, hp, queue, &qn, plaq, cnt);
+        if (h < h1) hb_link<P, MU, MEAS, 1, true, CAP>(L, g, Substep{MU, 1}, h, tag, sweep, beta, hp, queue, &qn, plaq, cnt);
       }
       __syncthreads();
-      hb_drain<P, MU, MEAS, 1>(L, queue, min(qn, CAP), tag, sweep, hp, plaq, cnt);
+      hb_drain<P, MU, MEAS, 1>(L, Substep{MU, 1}, queue, min(qn, CAP), tag, sweep, hp, plaq, cnt);
     }
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -1,0 +1,91 @@
+"""The FP64 kernels in fixed point, and their FP64 path for links outside the
+fixed-point range; the small-lattice substep at the edges of its range; the
+temporal-gauge Wilson kernel on time extents of every remainder.  FP64 against
+the oracle at 1e-12 (values up to 6 and about a hundred operations of 2^-53
+each leave 1e-14; loops up to W = |U|^64 on scaled links are compared relative to
+their size)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1010_4834_gb300 import Batch, Lattice, inputs
+from test_gpu_parity import MTOL, as_stored, substep_compare
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (4, 6, 8, 4)
+
+
+def _field(kind, dims=DIMS, seed=3):
+    """Links in and out of the fixed-point range (components 0 or below 2^-31,
+    norms off one), everywhere or on some links only."""
+    U = inputs.random_field(dims, seed)
+    rng = np.random.default_rng(seed)
+    some = rng.random(U.shape[:2]) < 0.1
+    if kind == "abelian":
+        return inputs.abelian_field(inputs.abelian_angles(dims, seed))
+    if kind == "cold":
+        return np.broadcast_to(np.array([1.0, 0.0, 0.0, 0.0]), U.shape).copy()
+    if kind == "tiny":                    # one component below the range, of either sign
+        U[some, 1] = rng.choice([-1, 1], some.sum()) * np.exp2(rng.uniform(-60, -30, some.sum()))
+        return U / np.linalg.norm(U, axis=-1, keepdims=True)
+    if kind == "edge":                    # norms at the edge of the range
+        return U * (1 + 0.06 * rng.uniform(-1, 1, U.shape[:2]))[..., None]
+    if kind == "scaled":
+        U[some] *= 1.3
+    return U
+
+
+KINDS = ["random", "abelian", "cold", "tiny", "edge", "scaled"]
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_fp64_substep_on_any_links(kind):
+    U = _field(kind)
+    for mu, p in ((0, 0), (1, 1), (2, 0), (3, 1)):
+        lat = Lattice(DIMS, 2.3, seed=7, prec="f64")
+        lat.set_links(U)
+        lat.substep(mu, p, 5)
+        ref = U.copy()
+        oracle.substep(list(DIMS), ref, oracle.chain(2.3, seed=7), 5, mu, p)
+        assert (ref != U).any()
+        np.testing.assert_allclose(lat.get_links(), ref, atol=1e-12, rtol=0)
+
+
+@pytest.mark.parametrize("beta,sampler,tries", [(0.02, "kp", 64), (0.3, "kp", 64), (0.08, "kp", 2), (0.3, "creutz", 64),
+                                                (2.4, "creutz", 3), (2.4, "kp", 1), (40.0, "kp", 64), (300.0, "kp", 3)])
+def test_fp64_draws_over_couplings(beta, sampler, tries):
+    # small beta: alpha on both sides of the value below which a trial runs in FP64
+    substep_compare(DIMS, "f64", beta, _field("random"), 1, 0, sweep=2, sampler=sampler, max_tries=tries)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_fp64_overrelaxation_smearing_and_measurements_on_any_links(kind):
+    U = _field(kind)
+    d = list(DIMS)
+    lat = Lattice(DIMS, 2.0, prec="f64")
+    lat.set_links(U)
+    np.testing.assert_allclose(lat.plaquette(), oracle.plaquette(d, U), atol=2e-12, rtol=0)
+    assert abs(lat.polyakov() - oracle.polyakov(d, U)) < 2e-12
+    np.testing.assert_allclose(lat.wilson_loops(4, 4), oracle.wilson_loops(d, U, 4, 4), atol=2e-12, rtol=1e-11)
+    lat.ape_smear(0.6, 2)
+    S = oracle.ape_smear(d, U.copy(), 0.6, 2)
+    np.testing.assert_allclose(lat.wilson_loops(4, 4, smeared=True), oracle.wilson_loops(d, S, 4, 4), atol=2e-12, rtol=1e-11)
+    lat.overrelax(1)
+    for mu in range(4):
+        for p in range(2):
+            oracle.overrelax_substep(d, U, mu, p)
+    # U' = W U^+ W keeps |U|; a staple sum that all but vanishes has no direction
+    np.testing.assert_allclose(lat.get_links(), U, atol=1e-11, rtol=0)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("nt", [2, 4, 6, 10, 12, 14, 18, 20, 24, 28, 36, 40, 46, 56, 62])
+def test_wilson_loops_on_every_remainder_of_the_time_extent(nt, prec):
+    dims = (6, 4, 6, nt)
+    U = inputs.random_field(dims, 31)
+    ref = oracle.wilson_loops(list(dims), as_stored(U, prec), 4, min(nt, 16))
+    lat = Lattice(dims, 2.0, prec=prec)
+    lat.set_links(U)
+    for rmax, tmax in ((4, min(nt, 16)), (3, min(nt, 5)), (1, 1)):
+        np.testing.assert_allclose(lat.wilson_loops(rmax, tmax), ref[:rmax, :tmax], atol=MTOL[prec] * 5, rtol=0)
