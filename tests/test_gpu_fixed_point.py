@@ -79,6 +79,37 @@ def test_fp64_overrelaxation_smearing_and_measurements_on_any_links(kind):
     np.testing.assert_allclose(lat.get_links(), U, atol=1e-11, rtol=0)
 
 
+@pytest.mark.parametrize("prec,dims", [("f64", (32, 16, 38, 4)), ("f64", (34, 16, 38, 4)), ("f64", (2, 2, 2, 2)),
+                                       ("f64", (6, 2, 2, 10)), ("f64", (8, 8, 8, 18)), ("f64", (8, 8, 8, 20)),
+                                       ("f64", (16, 16, 8, 18)), ("f64", (16, 16, 16, 10)), ("f32", (32, 32, 38, 4)), ("f32", (34, 32, 38, 4)),
+                                       ("f32", (2, 2, 2, 2)), ("f32", (6, 10, 2, 14)), ("f16q", (32, 32, 38, 4)),
+                                       ("f16q", (10, 6, 2, 4))])
+@pytest.mark.parametrize("sampler,tries,nor", [("kp", 64, 0), ("creutz", 64, 1), ("kp", 2, 2)])
+def test_small_lattice_substeps_leave_the_batched_kernel_s_links(prec, dims, sampler, tries, nor):
+    # at and just past the largest lattice of the small kernel (152 SMs) and of
+    # its FP64 forms with eight and two lanes a link, and at volumes that do not
+    # fill a block or a warp: direct launches, replayed graphs and measured
+    # sweeps, against the batched kernel
+    a = Lattice(dims, 2.2, seed=9, start="hot", prec=prec)
+    m = Lattice(dims, 2.2, seed=9, start="hot", prec=prec)
+    b = Batch([dims], [2.2], seed=9, start="hot", prec=prec)
+    for x in (a, m, b):
+        x.set_options(tries, sampler)
+        x.set_overrelax(nor)
+    a.sweep(3)
+    a.sweep(16)
+    m.sweep_measure(2)
+    hist = m.sweep_measure(17)
+    b.sweep(19)
+    got = a.get_links()
+    assert np.array_equal(got, b.get_links(0))
+    assert np.array_equal(got, m.get_links())
+    np.testing.assert_allclose(hist[-1, :3], a.plaquette(), atol=MTOL[prec], rtol=0)
+    assert abs(hist[-1, 3] - a.polyakov()) < 1e-12
+    np.testing.assert_allclose(b.plaquette()[0], a.plaquette(), atol=1e-9 if prec != "f64" else 1e-13, rtol=0)
+    np.testing.assert_allclose(b.polyakov()[0], a.polyakov(), atol=1e-9 if prec != "f64" else 1e-13, rtol=0)
+
+
 @pytest.mark.parametrize("prec", ["f64", "f32"])
 @pytest.mark.parametrize("nt", [2, 4, 6, 10, 12, 14, 18, 20, 24, 28, 36, 40, 46, 56, 62])
 def test_wilson_loops_on_every_remainder_of_the_time_extent(nt, prec):
