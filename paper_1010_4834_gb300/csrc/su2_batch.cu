@@ -34,6 +34,8 @@ struct su2_batch {
   uint32_t* d_sweep;
   Scratch scratch;
   double* d_results;
+  BatchBlock4* d_mblocks;  // the blocks of a measurement of every lattice
+  int n_mblocks;
   double* h_results;
   double* d_mpart;  // measured sweeps: four partial-sum slots per CTA
   cudaStream_t stream;
@@ -95,6 +97,21 @@ void drop_graph(su2_batch* b) {
   if (b->graph) cudaGraphExecDestroy(b->graph);
   b->graph = nullptr;
   b->graph_n = 0;
+}
+
+// The blocks of a measurement of every lattice: shares of about equal size,
+// four a multiprocessor in all, at least two sites a thread and one block a
+// lattice.
+std::vector<BatchBlock4> measure_blocks(const su2_batch* b) {
+  int64_t total = 0;
+  for (const BatchLattice& d : b->desc) total += 2 * d.g.vh;
+  const int64_t share = std::max<int64_t>(2 * 256, total / (4 * device_info().sms) + 1);
+  std::vector<BatchBlock4> blocks;
+  for (int i = 0; i < b->n; ++i) {
+    const int count = (int)((2 * b->desc[i].g.vh + share - 1) / share);
+    for (int k = 0; k < count; ++k) blocks.push_back(BatchBlock4{i, k, count, 0});
+  }
+  return blocks;
 }
 
 // Deal the lattices to G groups, largest first, each to the group with the
@@ -280,9 +297,12 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   const size_t o_ctl = o; o = align256(o + sizeof(BatchCtl));
   const size_t o_sweep = o; o = align256(o + 64);
   const size_t o_part = o; o = align256(o + kScratchPartials * sizeof(double));
-  const size_t o_cnt = o; o = align256(o + 64 * sizeof(unsigned int));
+  const size_t o_cnt = o; o = align256(o + (size_t)n * sizeof(unsigned int));
   const size_t o_out = o; o = align256(o + kScratchOut * sizeof(double));
   const size_t o_res = o; o = align256(o + 3 * (size_t)n * sizeof(double));
+  const std::vector<BatchBlock4> mblocks = measure_blocks(b);
+  b->n_mblocks = (int)mblocks.size();
+  const size_t o_mblk = o; o = align256(o + mblocks.size() * sizeof(BatchBlock4));
   const size_t o_mpart = o; o = align256(o + 4 * (size_t)kMaxCtas * sizeof(double));
   cudaError_t e = cudaMalloc(&b->base, o);
   if (e != cudaSuccess) {
@@ -303,6 +323,7 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   b->scratch.counter = (unsigned int*)(base + o_cnt);
   b->scratch.out = (double*)(base + o_out);
   b->d_results = (double*)(base + o_res);
+  b->d_mblocks = (BatchBlock4*)(base + o_mblk);
   b->d_mpart = (double*)(base + o_mpart);
   if (cuda_stream) {
     b->stream = (cudaStream_t)cuda_stream;
@@ -313,6 +334,8 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   SU2_CU_CLEAN(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMallocHost(&b->h_results, 3 * (size_t)n * sizeof(double)), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMemcpyAsync(b->d_desc, b->desc.data(), n * sizeof(BatchLattice), cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
+  SU2_CU_CLEAN(cudaMemcpyAsync(b->d_mblocks, mblocks.data(), mblocks.size() * sizeof(BatchBlock4),
+                               cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMemsetAsync(b->d_bars, 0, kMaxGroups * sizeof(GroupBarrier), b->stream), su2_batch_destroy(b));
   BatchCtl ctl;
   std::memset(&ctl, 0, sizeof ctl);
@@ -328,7 +351,7 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   }
   SU2_CU_CLEAN(cudaMemcpyAsync(b->d_ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMemsetAsync(b->d_sweep, 0, 64, b->stream), su2_batch_destroy(b));
-  SU2_CU_CLEAN(cudaMemsetAsync(b->scratch.counter, 0, 64 * sizeof(unsigned int), b->stream), su2_batch_destroy(b));
+  SU2_CU_CLEAN(cudaMemsetAsync(b->scratch.counter, 0, (size_t)n * sizeof(unsigned int), b->stream), su2_batch_destroy(b));
   const PhiloxKey key = batch_key(b);
   for (int i = 0; i < n; ++i)
     SU2_CU_CLEAN(launch_init(lview(b, i), start, key, (uint32_t)i << 2, b->stream), su2_batch_destroy(b));
@@ -553,11 +576,8 @@ static int batch_measure(su2_batch* b, int which, double* out) {
   if (!b || !out) return fail(SU2_EINVAL, "NULL argument");
   DeviceGuard dg(b->device);
   const int k = which == 0 ? 3 : 1;
-  for (int i = 0; i < b->n; ++i) {
-    if (which == 0) SU2_CU(launch_plaquette(lview(b, i), b->scratch, b->stream));
-    else SU2_CU(launch_polyakov(lview(b, i), b->scratch, b->stream));
-    SU2_CU(cudaMemcpyAsync(b->d_results + (size_t)k * i, b->scratch.out, k * sizeof(double), cudaMemcpyDeviceToDevice, b->stream));
-  }
+  SU2_CU(launch_batch_measure(b->prec, which != 0, b->d_desc, b->d_mblocks, b->n_mblocks, b->scratch.partials,
+                              b->scratch.counter, b->d_results, b->stream));
   SU2_CU(cudaMemcpyAsync(b->h_results, b->d_results, (size_t)k * b->n * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
   SU2_CU(cudaStreamSynchronize(b->stream));
   std::memcpy(out, b->h_results, (size_t)k * b->n * sizeof(double));

@@ -27,6 +27,16 @@ struct BatchCtl {
 // searched by su2_batch_tune).
 constexpr int kBatchThreads = 256;  // default
 
+// A block of a batched measurement: block `rank` of the `count` that share a
+// lattice (consecutive blocks).
+struct BatchBlock4 {
+  int lattice, rank, count, pad;
+};
+// Plaquette means (3 doubles a lattice) or Polyakov loops (1) of every lattice;
+// counters: one zero word a lattice, left zero.
+cudaError_t launch_batch_measure(int prec, bool polyakov, const BatchLattice* desc, const BatchBlock4* blocks,
+                                 int nblocks, double* partials, unsigned int* counters, double* out, cudaStream_t st);
+
 // One launch's arguments (see k_batch_groups).
 struct BatchArgs {
   const BatchLattice* desc;

@@ -16,6 +16,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "su2_batch.h"
 #include "su2_hb_link.cuh"
 #include "su2_internal.h"
 #include "su2_kernel_util.cuh"
@@ -234,6 +235,62 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
     if (ep.meas) {
       plaquette_from_block_sums(ep.meas, kMeasStride, ep.nb, ep.volume, row);
       if (threadIdx.x == 0) *ep.sweep += 1u;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Plaquette or Polyakov loop of every lattice of a batch in one launch: block b
+// takes a share of one lattice (blocks[b]) and the last block of a lattice
+// adds its blocks' sums in a fixed order.  (64 lattices of 8^4 to 24^3 x 6, one
+// launch and one device copy per lattice before: see launch_batch_measure.)
+// ---------------------------------------------------------------------------
+template <int P, bool POLY>
+__global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : 3)
+    k_batch_measure(const BatchLattice* __restrict__ desc, const BatchBlock4* __restrict__ blocks, double* partials,
+                    unsigned int* counters, double* out) {
+  using R = typename Real<P>::T;
+  const BatchBlock4 b = blocks[blockIdx.x];
+  const Geom& g = desc[b.lattice].g;
+  Links<P> L;
+  L.set(desc[b.lattice].links, g.vh);
+  const int first = b.rank * kThreads + (int)threadIdx.x, stride = b.count * kThreads;
+  constexpr int NV = POLY ? 1 : 2;
+  double v[NV];
+  if constexpr (POLY) {
+    Acc<R> acc;
+    const int nsig = g.n[0] * g.n[1] * g.n[2];
+    for (int xs = first; xs < nsig; xs += stride) {
+      const int odd = parity(site_from_index(g, (uint32_t)xs));   // of (xs, t = 0)
+      acc.add(time_line<P, kFlat, true>(L.cls_base(6 + odd), L.cls_base(7 - odd), (uint32_t)(xs >> 1), (uint32_t)(nsig / 2),
+                                  g.n[3]).w);
+    }
+    v[0] = acc.value();
+  } else {
+    Acc<R> sp, tm;
+    for (int s = first; s < (int)(2 * g.vh); s += stride) {
+      R ss, ts;
+      plaq_site(L, g, s, ss, ts);
+      sp.add(ss);
+      tm.add(ts);
+    }
+    v[0] = sp.value();
+    v[NV - 1] = tm.value();
+  }
+  if (block_partial<NV>(v, partials, counters + b.lattice, blockIdx.x, b.count)) {
+    double tot[NV];
+    final_sum<NV>(partials + (size_t)(blockIdx.x - b.rank) * NV, b.count, tot);
+    if (threadIdx.x == 0) {
+      if constexpr (POLY) {
+        out[b.lattice] = tot[0] / (double)(g.n[0] * g.n[1] * g.n[2]);
+      } else {
+        const double n3 = 3.0 * (double)(2 * g.vh);
+        double* o = out + 3 * (size_t)b.lattice;
+        o[0] = (tot[0] + tot[NV - 1]) / (2.0 * n3);
+        o[1] = tot[0] / n3;
+        o[2] = tot[NV - 1] / n3;
+      }
+      counters[b.lattice] = 0;
     }
   }
 }
@@ -1156,6 +1213,17 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
     };
     const cudaError_t err = overlaps(v) ? launch(k_polyakov<P, false>) : launch(k_polyakov<P, true>);
     if (err != cudaSuccess) return err;
+  });
+  count_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_measure(int prec, bool polyakov, const BatchLattice* desc, const BatchBlock4* blocks,
+                                 int nblocks, double* partials, unsigned int* counters, double* out,
+                                 cudaStream_t st) {
+  SU2_DISPATCH(prec, {
+    if (polyakov) k_batch_measure<P, true><<<nblocks, kThreads, 0, st>>>(desc, blocks, partials, counters, out);
+    else k_batch_measure<P, false><<<nblocks, kThreads, 0, st>>>(desc, blocks, partials, counters, out);
   });
   count_launches(1);
   return cudaGetLastError();

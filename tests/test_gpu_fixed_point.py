@@ -120,3 +120,18 @@ def test_wilson_loops_on_every_remainder_of_the_time_extent(nt, prec):
     lat.set_links(U)
     for rmax, tmax in ((4, min(nt, 16)), (3, min(nt, 5)), (1, 1)):
         np.testing.assert_allclose(lat.wilson_loops(rmax, tmax), ref[:rmax, :tmax], atol=MTOL[prec] * 5, rtol=0)
+
+
+def test_batched_measurements_of_uneven_lattices():
+    dims = [(4, 4, 4, 4), (16, 8, 12, 6), (2, 2, 2, 2), (6, 10, 4, 14), (8, 8, 8, 8)]
+    for prec in ("f64", "f32", "f16q"):
+        b = Batch(dims, [2.0] * len(dims), seed=1, start="cold", prec=prec)
+        fields = [inputs.random_field(d, 50 + i) for i, d in enumerate(dims)]
+        for i, U in enumerate(fields):
+            b.set_links(i, U)
+        for _ in range(2):                # the second call finds the counters at zero
+            plaq, poly = b.plaquette(), b.polyakov()
+            for i, (d, U) in enumerate(zip(dims, fields)):
+                ref = as_stored(U, prec)
+                np.testing.assert_allclose(plaq[i], oracle.plaquette(list(d), ref), atol=MTOL[prec], rtol=0)
+                assert abs(poly[i] - oracle.polyakov(list(d), ref)) < MTOL[prec]
