@@ -904,6 +904,15 @@ template <int D, int S> __device__ __forceinline__ int half_step(const Geom& g, 
   return xd == 0 ? g.hwr[D] : -g.hst[D];
 }
 
+// s += v / |v|
+__device__ __forceinline__ void qacc_unit(Quat<float>& s, const Quat<float>& v) {
+  const float n = rsqrtf(qdot(v, v));
+  s.w = fmaf(v.w, n, s.w);
+  s.x = fmaf(v.x, n, s.x);
+  s.y = fmaf(v.y, n, s.y);
+  s.z = fmaf(v.z, n, s.z);
+}
+
 // F16Q staple loads without the per-link re-normalisation: staple_term
 // scales each product of three links once instead (see there).
 template <int P, bool NC, bool MCG, int CP>
@@ -924,19 +933,19 @@ __device__ __forceinline__ void staple_term(const Links<P, CP>& L, const Geom& g
   const int q = p ^ 1;
   const int h_mnu = h + half_step<NU, -1>(g, x);
   if constexpr (P == kF16Q) {
-    // binary16 links re-normalised per term: a product of quaternions has the
-    // product of their norms, so each term of three stored links is scaled
-    // once by 1 / (|a| |b| |c|) (one rsqrt where per-link re-normalisation
-    // takes three); equal to the staple of the re-normalised links up to
-    // FP32 rounding
+    // binary16 links re-normalised per term: each product of three stored
+    // links is scaled to unit norm by its own (4 multiply-adds, one rsqrt and
+    // the scaled sum, where the three links' norms took 12 and 2 more; 64^4
+    // substep: see k_heatbath); equal to the staple of the re-normalised links
+    // up to FP32 rounding
     const Quat<R> a = ld_raw<P, NC, false>(L, 2 * NU + p, h);
     const Quat<R> b = ld_raw<P, NC, MCG>(L, 2 * MU + q, h + half_step<NU, +1>(g, x));
     const Quat<R> c = ld_raw<P, NC, false>(L, 2 * NU + q, h + dmu);
     const Quat<R> d = ld_raw<P, NC, false>(L, 2 * NU + q, h_mnu);
     const Quat<R> e = ld_raw<P, NC, MCG>(L, 2 * MU + q, h_mnu);
     const Quat<R> f = ld_raw<P, NC, false>(L, 2 * NU + p, h_mnu + dmu);
-    qacc_mul_nd(s, qscale(qmul(a, b), rsqrtf(qdot(a, a) * qdot(b, b) * qdot(c, c))), c);
-    qacc_mul(s, qscale(qmul_dn(d, e), rsqrtf(qdot(d, d) * qdot(e, e) * qdot(f, f))), f);
+    qacc_unit(s, qmul_nd(qmul(a, b), c));
+    qacc_unit(s, qmul(qmul_dn(d, e), f));
   } else {
     const Quat<R> a = ldl<P, NC>(L, 2 * NU + p, h);                                // U_nu(x)
     const Quat<R> b = ldmu<P, NC, MCG>(L, 2 * MU + q, h + half_step<NU, +1>(g, x)); // U_mu(x+nu)

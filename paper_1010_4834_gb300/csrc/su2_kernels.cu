@@ -308,21 +308,38 @@ __global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : 3)
 // three.  Each link's staple terms are added nu ascending, forward then
 // backward.  blockIdx.y = parity.
 // ---------------------------------------------------------------------------
+// binary16 links enter as stored and each product of three is scaled to unit
+// norm (qacc_unit), as in the heat bath's staples.
+template <int P, bool NC>
+__device__ __forceinline__ Quat<typename Real<P>::T> ape_link(const Links<P, kClassPtr>& L, int cls, int h) {
+  if constexpr (P == kF16Q) return ld_raw<P, NC, false>(L, cls, h);
+  else return ldl<P, NC>(L, cls, h);
+}
+// s += a b^dagger, s += a b
+template <int P, class Q> __device__ __forceinline__ void ape_acc_nd(Q& s, const Q& a, const Q& b) {
+  if constexpr (P == kF16Q) qacc_unit(s, qmul_nd(a, b));
+  else qacc_mul_nd(s, a, b);
+}
+template <int P, class Q> __device__ __forceinline__ void ape_acc(Q& s, const Q& a, const Q& b) {
+  if constexpr (P == kF16Q) qacc_unit(s, qmul(a, b));
+  else qacc_mul(s, a, b);
+}
+
 template <int P, int MU, int NU, bool NC>
 __device__ __forceinline__ void ape_pair(const Links<P, kClassPtr>& L, int h, int p, const int (&dp)[3], const int (&dm)[3],
                                          const Quat<typename Real<P>::T>& umu, const Quat<typename Real<P>::T>& unu,
                                          Quat<typename Real<P>::T>& smu, Quat<typename Real<P>::T>& snu) {
   using R = typename Real<P>::T;
   const int q = p ^ 1;
-  auto link = [&](int cls, int i) { return ldl<P, NC>(L, cls, i); };
+  auto link = [&](int cls, int i) { return ape_link<P, NC>(L, cls, i); };
   const Quat<R> a = qmul_nd(link(2 * NU + q, h + dp[MU]), link(2 * MU + q, h + dp[NU]));
   const int hn = h + dm[NU], hm = h + dm[MU];  // x - nu, x - mu
   // link mu, term nu: forward U_nu(x) A^dag, backward U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu)
-  qacc_mul_nd(smu, unu, a);
-  qacc_mul(smu, qmul_dn(link(2 * NU + q, hn), link(2 * MU + q, hn)), link(2 * NU + p, hn + dp[MU]));
+  ape_acc_nd<P>(smu, unu, a);
+  ape_acc<P>(smu, qmul_dn(link(2 * NU + q, hn), link(2 * MU + q, hn)), link(2 * NU + p, hn + dp[MU]));
   // link nu, term mu: forward U_mu(x) A, backward U_mu(x-mu)^dag U_nu(x-mu) U_mu(x-mu+nu)
-  qacc_mul(snu, umu, a);
-  qacc_mul(snu, qmul_dn(link(2 * MU + q, hm), link(2 * NU + q, hm)), link(2 * MU + p, hm + dp[NU]));
+  ape_acc<P>(snu, umu, a);
+  ape_acc<P>(snu, qmul_dn(link(2 * MU + q, hm), link(2 * NU + q, hm)), link(2 * MU + p, hm + dp[NU]));
 }
 
 template <int P, int CP>
@@ -354,11 +371,16 @@ __device__ __forceinline__ void ape_sites(const Links<P, kClassPtr>& src, const 
     // is h + step(a) + step(b) for steps in different directions
     const int dp[3] = {half_step<0, +1>(g, x), half_step<1, +1>(g, x), half_step<2, +1>(g, x)};
     const int dm[3] = {half_step<0, -1>(g, x), half_step<1, -1>(g, x), half_step<2, -1>(g, x)};
-    const Quat<R> u0 = ldl<P, NC>(src, 0 + p, h), u1 = ldl<P, NC>(src, 2 + p, h), u2 = ldl<P, NC>(src, 4 + p, h);
+    Quat<R> u0 = ape_link<P, NC>(src, 0 + p, h), u1 = ape_link<P, NC>(src, 2 + p, h), u2 = ape_link<P, NC>(src, 4 + p, h);
     Quat<R> s0 = qmake<R>(0, 0, 0, 0), s1 = s0, s2 = s0;
     ape_pair<P, 0, 1, NC>(src, h, p, dp, dm, u0, u1, s0, s1);
     ape_pair<P, 0, 2, NC>(src, h, p, dp, dm, u0, u2, s0, s2);
     ape_pair<P, 1, 2, NC>(src, h, p, dp, dm, u1, u2, s1, s2);
+    if constexpr (P == kF16Q) {
+      u0 = qscale(u0, rsqrtf(qdot(u0, u0)));
+      u1 = qscale(u1, rsqrtf(qdot(u1, u1)));
+      u2 = qscale(u2, rsqrtf(qdot(u2, u2)));
+    }
     ape_store<P>(dst, 0 + p, h, u0, s0, c0, c1);
     ape_store<P>(dst, 2 + p, h, u1, s1, c0, c1);
     ape_store<P>(dst, 4 + p, h, u2, s2, c0, c1);
