@@ -186,8 +186,8 @@ int su2_restart(su2_lattice* h, int start);
  * The Monte Carlo production loop: n >= 0 times (one heat-bath sweep, then
  * su2_plaquette and su2_polyakov of the new configuration).  hist[4*i + k]
  * receives, for sweep i of this call, the three plaquette means (k = 0..2)
- * and the Polyakov loop (k = 3).  Results stay on the device until the end
- * of the call (one synchronisation per 1024 sweeps).  Advances the sweep
+ * and the Polyakov loop (k = 3).  Results are read at the end of the call
+ * (one synchronisation per 1024 sweeps).  Advances the sweep
  * counter by n.  The plaquette is summed inside the sweep (in the
  * odd-parity substeps of mu = 1, 2, 3, from their staples), so it equals
  * su2_plaquette of the new configuration up to the order of summation (a

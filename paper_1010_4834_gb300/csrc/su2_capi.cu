@@ -58,7 +58,8 @@ struct su2_lattice {
   double* d_hist;
   double* staging;
   int64_t staging_sites;
-  double* h_out;  // pinned host results
+  double* h_out;   // pinned host memory that the kernels write results to (kScratchOut doubles),
+  double* h_hist;  // and the history ring behind it (kHistRing rows of 4)
   // streams and the cached sweep graph
   cudaStream_t stream;
   bool own_stream;
@@ -82,7 +83,7 @@ constexpr int kGraphSweeps = 8;
 constexpr int64_t kStagingSites = (int64_t)1 << 18;
 
 struct Layout {
-  size_t links, ape0, ape1, partials, counter, out, state, hist, pair, staging, total;
+  size_t links, ape0, ape1, partials, counter, state, pair, staging, total;
 };
 
 
@@ -98,9 +99,7 @@ Layout layout_for(const int dims[4], int prec) {
   L.ape1 = o; o = align256(o + 3 * (size_t)V * lb);
   L.partials = o; o = align256(o + kScratchPartials * sizeof(double));
   L.counter = o; o = align256(o + 64 * sizeof(unsigned int));
-  L.out = o; o = align256(o + kScratchOut * sizeof(double));
   L.state = o; o = align256(o + 256);
-  L.hist = o; o = align256(o + (size_t)kHistRing * 4 * sizeof(double));
   L.pair = o; o = align256(o + sizeof(PairCtl) + (size_t)dims[3] * sizeof(unsigned int));
   const int64_t st = V < kStagingSites ? V : kStagingSites;
   L.staging = o; o = align256(o + (size_t)st * 16 * sizeof(double));
@@ -211,10 +210,8 @@ static int init_common(su2_lattice** out, const int dims[4], double beta, uint64
   h->ape[1] = b + L.ape1;
   h->scratch.partials = (double*)(b + L.partials);
   h->scratch.counter = (unsigned int*)(b + L.counter);
-  h->scratch.out = (double*)(b + L.out);
   h->d_sweep = (uint32_t*)(b + L.state);
   h->d_stats = (unsigned long long*)(b + L.state + 64);
-  h->d_hist = (double*)(b + L.hist);
   h->d_pair = (PairCtl*)(b + L.pair);
   h->d_done0 = (unsigned int*)(b + L.pair + sizeof(PairCtl));
   h->schedule = SU2_SCHED_AUTO;
@@ -230,8 +227,16 @@ static int init_common(su2_lattice** out, const int dims[4], double beta, uint64
     h->own_stream = true;
   }
   SU2_CU_CLEAN(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking), su2_destroy(h));
-  SU2_CU_CLEAN(cudaMallocHost(&h->h_out, kScratchOut * sizeof(double)), su2_destroy(h));
-  SU2_CU_CLEAN(cudaMemsetAsync(b + L.counter, 0, L.out - L.counter, h->stream), su2_destroy(h));
+  // Results go straight to the host: the last block of a reduction (or the
+  // block of an output) writes them over the host link, and the call reads
+  // them after its stream synchronisation, without a device-to-host copy
+  // (16^4 FP32 analysis, seven results: 224 -> 206 us; 8 measured sweeps of
+  // 32^3x4 with over-relaxation: 484 -> 475 us).
+  SU2_CU_CLEAN(cudaHostAlloc(&h->h_out, (kScratchOut + 4 * kHistRing) * sizeof(double), cudaHostAllocMapped), su2_destroy(h));
+  h->h_hist = h->h_out + kScratchOut;
+  SU2_CU_CLEAN(cudaHostGetDevicePointer((void**)&h->scratch.out, h->h_out, 0), su2_destroy(h));
+  h->d_hist = h->scratch.out + kScratchOut;
+  SU2_CU_CLEAN(cudaMemsetAsync(b + L.counter, 0, L.state - L.counter, h->stream), su2_destroy(h));
   SU2_CU_CLEAN(cudaMemsetAsync(b + L.state, 0, 256, h->stream), su2_destroy(h));
   SU2_CU_CLEAN(cudaMemsetAsync(b + L.pair, 0, L.staging - L.pair, h->stream), su2_destroy(h));
   SU2_CU_CLEAN(launch_init(view(h), start, philox_key(h->seed), 0u, h->stream), su2_destroy(h));
@@ -522,12 +527,9 @@ extern "C" int su2_sweep_measure(su2_lattice* h, int n, double* hist) {
     // kHistRing: at most two contiguous pieces
     const int r0 = (int)((h->sweep + (uint64_t)c0) % (uint64_t)kHistRing);
     const int first = m < kHistRing - r0 ? m : kHistRing - r0;
-    SU2_CU(cudaMemcpyAsync(hist + 4 * (size_t)c0, h->d_hist + 4 * (size_t)r0, (size_t)first * 4 * sizeof(double),
-                           cudaMemcpyDeviceToHost, h->stream));
-    if (m > first)
-      SU2_CU(cudaMemcpyAsync(hist + 4 * (size_t)(c0 + first), h->d_hist, (size_t)(m - first) * 4 * sizeof(double),
-                             cudaMemcpyDeviceToHost, h->stream));
     SU2_CU(cudaStreamSynchronize(h->stream));
+    std::memcpy(hist + 4 * (size_t)c0, h->h_hist + 4 * (size_t)r0, (size_t)first * 4 * sizeof(double));
+    std::memcpy(hist + 4 * (size_t)(c0 + first), h->h_hist, (size_t)(m - first) * 4 * sizeof(double));
   }
   h->sweep += (uint64_t)n;
   if (n) h->smeared = 0;
@@ -647,7 +649,6 @@ extern "C" int su2_overrelax_sweep(su2_lattice* h, int n) {
 }
 
 static int fetch_out(su2_lattice* h, int count, double* dst) {
-  SU2_CU(cudaMemcpyAsync(h->h_out, h->scratch.out, count * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   SU2_CU(cudaStreamSynchronize(h->stream));
   int rc = check_pair(h);
   if (rc) return rc;
@@ -748,9 +749,8 @@ extern "C" int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smea
   // FP64: the fixed-point kernel reports links that are not unit quaternions
   // (a store filled from outside) in the word behind the results; the loops are
   // then multiplied out in FP64
-  double* flag = h->scratch.out + n;
-  SU2_CU(cudaMemsetAsync(flag, 0, sizeof *flag, h->stream));
-  SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, flag, h->stream));
+  h->h_out[n] = 0.0;  // every call that writes results has waited for them
+  SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, h->scratch.out + n, h->stream));
   double got[32 * 32 + 1];
   int rc = fetch_out(h, n + 1, got);
   if (rc) return rc;
