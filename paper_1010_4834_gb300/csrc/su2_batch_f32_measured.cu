@@ -1,3 +1,4 @@
+#define SU2_COMPILER_FUSES
 #include "su2_batch_kernel.cuh"
 
 namespace su2 {

@@ -90,27 +90,8 @@ template <class R> __device__ __forceinline__ R qdot(const Quat<R>& a, const Qua
 
 // Products with every rounding spelled out: a sum of two products leaves the
 // compiler the choice which of them it fuses, and kernels that must agree bit
-// for bit (plain, measured and small-lattice substeps, batches, time slabs) did
-// differ.  FP32 fuses as the kernels were compiled before: the first product of
-// each sum, or the first positive one.
-template <> __device__ __forceinline__ float qdot<float>(const Quat<float>& a, const Quat<float>& b) {
-  return fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x))));
-}
-template <> __device__ __forceinline__ Quat<float> qmul<float>(const Quat<float>& a, const Quat<float>& b) {
-  return qmake<float>(fmaf(-a.z, b.z, fmaf(-a.y, b.y, fmaf(a.w, b.w, __fmul_rn(-a.x, b.x)))),
-                      fmaf(a.z, b.y, fmaf(-a.y, b.z, fmaf(a.w, b.x, __fmul_rn(a.x, b.w)))),
-                      fmaf(a.x, b.z, fmaf(-a.z, b.x, fmaf(a.w, b.y, __fmul_rn(a.y, b.w)))),
-                      fmaf(a.y, b.x, fmaf(-a.x, b.y, fmaf(a.w, b.z, __fmul_rn(a.z, b.w)))));
-}
-template <> __device__ __forceinline__ Quat<float> qmul_nd<float>(const Quat<float>& a, const Quat<float>& b) {
-  return qmake<float>(fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x)))),
-                      fmaf(-a.z, b.y, fmaf(a.y, b.z, fmaf(a.x, b.w, __fmul_rn(-a.w, b.x)))),
-                      fmaf(-a.x, b.z, fmaf(a.z, b.x, fmaf(a.y, b.w, __fmul_rn(-a.w, b.y)))),
-                      fmaf(-a.y, b.x, fmaf(a.x, b.y, fmaf(a.z, b.w, __fmul_rn(-a.w, b.z)))));
-}
-template <> __device__ __forceinline__ Quat<float> qmul_dn<float>(const Quat<float>& a, const Quat<float>& b) {
-  return qmul<float>(qmake<float>(a.w, -a.x, -a.y, -a.z), b);
-}
+// for bit (plain, measured and small-lattice substeps, pairs, time slabs) did
+// differ.
 template <> __device__ __forceinline__ double qdot<double>(const Quat<double>& a, const Quat<double>& b) {
   return __fma_rn(a.z, b.z, __fma_rn(a.y, b.y, __fma_rn(a.x, b.x, __dmul_rn(a.w, b.w))));
 }
@@ -127,6 +108,48 @@ template <> __device__ __forceinline__ Quat<double> qmul_nd<double>(const Quat<d
 }
 template <> __device__ __forceinline__ Quat<double> qmul_dn<double>(const Quat<double>& a, const Quat<double>& b) {
   return qmul<double>(qmake<double>(a.w, -a.x, -a.y, -a.z), b);
+}
+
+// The updates' products.  In the heat-bath substeps' files FP32 fuses the first
+// product of each sum, or the first positive one, as those kernels were compiled
+// before.  Files whose kernels need no such agreement define SU2_COMPILER_FUSES:
+// FP32 batches, whose links stay those of earlier versions so, and measurements
+// and over-relaxation, which schedule better (64^4: plaquette 344 us, 366 spelled
+// out, FP32; over-relaxation 1376 us a sweep and 1411, F16Q).
+#ifdef SU2_COMPILER_FUSES
+constexpr bool kCompilerFuses = true;
+#else
+constexpr bool kCompilerFuses = false;
+#endif
+template <class R> __device__ __forceinline__ R qdot_rn(const Quat<R>& a, const Quat<R>& b) {
+  if constexpr (kCompilerFuses || sizeof(R) == 8)
+    return qdot(a, b);
+  else
+    return fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x))));
+}
+template <class R> __device__ __forceinline__ Quat<R> qmul_rn(const Quat<R>& a, const Quat<R>& b) {
+  if constexpr (kCompilerFuses || sizeof(R) == 8)
+    return qmul(a, b);
+  else
+    return qmake<R>(fmaf(-a.z, b.z, fmaf(-a.y, b.y, fmaf(a.w, b.w, __fmul_rn(-a.x, b.x)))),
+                    fmaf(a.z, b.y, fmaf(-a.y, b.z, fmaf(a.w, b.x, __fmul_rn(a.x, b.w)))),
+                    fmaf(a.x, b.z, fmaf(-a.z, b.x, fmaf(a.w, b.y, __fmul_rn(a.y, b.w)))),
+                    fmaf(a.y, b.x, fmaf(-a.x, b.y, fmaf(a.w, b.z, __fmul_rn(a.z, b.w)))));
+}
+template <class R> __device__ __forceinline__ Quat<R> qmul_nd_rn(const Quat<R>& a, const Quat<R>& b) {
+  if constexpr (kCompilerFuses || sizeof(R) == 8)
+    return qmul_nd(a, b);
+  else
+    return qmake<R>(fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.w, b.w, __fmul_rn(a.x, b.x)))),
+                    fmaf(-a.z, b.y, fmaf(a.y, b.z, fmaf(a.x, b.w, __fmul_rn(-a.w, b.x)))),
+                    fmaf(-a.x, b.z, fmaf(a.z, b.x, fmaf(a.y, b.w, __fmul_rn(-a.w, b.y)))),
+                    fmaf(-a.y, b.x, fmaf(a.x, b.y, fmaf(a.z, b.w, __fmul_rn(-a.w, b.z)))));
+}
+template <class R> __device__ __forceinline__ Quat<R> qmul_dn_rn(const Quat<R>& a, const Quat<R>& b) {
+  if constexpr (kCompilerFuses)
+    return qmul_dn(a, b);
+  else
+    return qmul_rn(qmake<R>(a.w, -a.x, -a.y, -a.z), b);
 }
 
 template <class R> __device__ __forceinline__ void qacc(Quat<R>& a, const Quat<R>& b) {
@@ -507,7 +530,7 @@ template <class R> __device__ __forceinline__ Direction<R> draw_direction(uint4 
 __device__ __forceinline__ Quat<float> compose_from(float a0, const Quat<float>& w, const Direction<float>& d) {
   const float rad = Math<float>::sqrt0(1.0f - a0 * a0);
   const Quat<float> x = qmake<float>(a0, rad * d.sin_t * d.cp, rad * d.sin_t * d.sp, rad * d.cos_t);
-  return qmul(x, w);
+  return qmul_rn(x, w);
 }
 __device__ __forceinline__ Quat<double> compose_from(int64_t a0, const FixQuat& w, const Direction<double>& d) {
   // |x|^2 = 1 - a0^2 = (1 - a0) (1 + a0); a0 > -1, and at a0 = 1 the second
@@ -529,7 +552,7 @@ __device__ __forceinline__ Quat<R> compose_link(A0Of<R> a0, const WOf<R>& w, uin
 // W = Sigma / k, k = |Sigma|, and alpha = beta k of a staple sum.
 template <class R> struct Frame { WOf<R> w; R alpha; };
 __device__ __forceinline__ Frame<float> staple_frame(const Quat<float>& sig, float beta) {
-  const float k2 = qdot(sig, sig);
+  const float k2 = qdot_rn(sig, sig);
   const float invk = Math<float>::rsqrt(k2);
   return Frame<float>{qscale(sig, invk), beta * k2 * invk};
 }
@@ -756,7 +779,7 @@ template <int CP> struct Links<kF16Q, CP> {
   }
   static __device__ __forceinline__ Quat<float> unpack(const uint2 a) {
     const Quat<float> q = unpack_raw(a);
-    return qscale(q, rsqrtf(qdot(q, q)));
+    return qscale(q, rsqrtf(qdot_rn(q, q)));
   }
   __device__ __forceinline__ Quat<float> ld_raw(int cls, int i) const { return unpack_raw(__ldg(at(cls, i))); }
   __device__ __forceinline__ Quat<float> ldc_raw(int cls, int i) const { return unpack_raw(*at(cls, i)); }
@@ -906,7 +929,7 @@ template <int D, int S> __device__ __forceinline__ int half_step(const Geom& g, 
 
 // s += v / |v|
 __device__ __forceinline__ void qacc_unit(Quat<float>& s, const Quat<float>& v) {
-  const float n = rsqrtf(qdot(v, v));
+  const float n = rsqrtf(qdot_rn(v, v));
   s.w = fmaf(v.w, n, s.w);
   s.x = fmaf(v.x, n, s.x);
   s.y = fmaf(v.y, n, s.y);
@@ -936,7 +959,7 @@ __device__ __forceinline__ void staple_term(const Links<P, CP>& L, const Geom& g
     // binary16 links re-normalised per term: each product of three stored
     // links is scaled to unit norm by its own (4 multiply-adds, one rsqrt and
     // the scaled sum, where the three links' norms took 12 and 2 more; 64^4
-    // substep: see k_heatbath); equal to the staple of the re-normalised links
+    // sweep 1535 -> 1414 us); equal to the staple of the re-normalised links
     // up to FP32 rounding
     const Quat<R> a = ld_raw<P, NC, false>(L, 2 * NU + p, h);
     const Quat<R> b = ld_raw<P, NC, MCG>(L, 2 * MU + q, h + half_step<NU, +1>(g, x));
@@ -944,8 +967,8 @@ __device__ __forceinline__ void staple_term(const Links<P, CP>& L, const Geom& g
     const Quat<R> d = ld_raw<P, NC, false>(L, 2 * NU + q, h_mnu);
     const Quat<R> e = ld_raw<P, NC, MCG>(L, 2 * MU + q, h_mnu);
     const Quat<R> f = ld_raw<P, NC, false>(L, 2 * NU + p, h_mnu + dmu);
-    qacc_unit(s, qmul_nd(qmul(a, b), c));
-    qacc_unit(s, qmul(qmul_dn(d, e), f));
+    qacc_unit(s, qmul_nd_rn(qmul_rn(a, b), c));
+    qacc_unit(s, qmul_rn(qmul_dn_rn(d, e), f));
   } else {
     const Quat<R> a = ldl<P, NC>(L, 2 * NU + p, h);                                // U_nu(x)
     const Quat<R> b = ldmu<P, NC, MCG>(L, 2 * MU + q, h + half_step<NU, +1>(g, x)); // U_mu(x+nu)
@@ -953,8 +976,8 @@ __device__ __forceinline__ void staple_term(const Links<P, CP>& L, const Geom& g
     const Quat<R> d = ldl<P, NC>(L, 2 * NU + q, h_mnu);                            // U_nu(x-nu)
     const Quat<R> e = ldmu<P, NC, MCG>(L, 2 * MU + q, h_mnu);                      // U_mu(x-nu)
     const Quat<R> f = ldl<P, NC>(L, 2 * NU + p, h_mnu + dmu);                      // U_nu(x-nu+mu)
-    qacc_mul_nd(s, qmul(a, b), c);
-    qacc_mul(s, qmul_dn(d, e), f);
+    qacc_mul_nd(s, qmul_rn(a, b), c);
+    qacc_mul(s, qmul_dn_rn(d, e), f);
   }
 }
 

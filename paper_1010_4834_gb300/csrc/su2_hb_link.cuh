@@ -97,7 +97,7 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
     uint4 c = ctr;
     c.w = 1u;
     const Quat<R> nl = haar_from<R>(philox(c, hp.rk));
-    if constexpr (MEAS) plaq.add(qdot(L.put(2 * mu + p, h, nl), lower));
+    if constexpr (MEAS) plaq.add(qdot_rn(L.put(2 * mu + p, h, nl), lower));
     else L.st(2 * mu + p, h, nl);
     cnt.haar += 1;
     return;
@@ -109,7 +109,7 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
   uint4 rt;
   if (trial_a0<R>(alpha, inv2a, e, ctr, 1, hp, &a0, &rt)) {
     const Quat<R> nl = compose_link<R>(a0, w, ctr, rt, hp);
-    if constexpr (MEAS) plaq.add(qdot(L.put(2 * mu + p, h, nl), lower));
+    if constexpr (MEAS) plaq.add(qdot_rn(L.put(2 * mu + p, h, nl), lower));
     else L.st(2 * mu + p, h, nl);
     cnt.trials += 1;
   } else if (hp.max_tries > 1) {
@@ -125,13 +125,13 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
     } else {
       Quat<R> nl;
       const int n = finish_deferred<R, MEAS>(d, ctr, hp, &nl);
-      if constexpr (MEAS) plaq.add(qdot(n ? L.put(2 * mu + p, h, nl) : ldl<P, NC>(L, 2 * mu + p, h), lower));
+      if constexpr (MEAS) plaq.add(qdot_rn(n ? L.put(2 * mu + p, h, nl) : ldl<P, NC>(L, 2 * mu + p, h), lower));
       else if (n) L.st(2 * mu + p, h, nl);
       cnt.trials += n ? (unsigned)n : (unsigned)hp.max_tries;
       cnt.capped += n == 0;
     }
   } else {
-    if constexpr (MEAS) plaq.add(qdot(ldl<P, NC>(L, 2 * mu + p, h), lower));
+    if constexpr (MEAS) plaq.add(qdot_rn(ldl<P, NC>(L, 2 * mu + p, h), lower));
     cnt.trials += 1;
     cnt.capped += 1;
   }
@@ -149,7 +149,7 @@ __device__ __forceinline__ void hb_drain(const Links<P, CP>& L, Substep sub, con
     const Deferred<R, MEAS> d = queue[i];
     Quat<R> nl;
     const int t = finish_deferred<R, MEAS>(d, make_uint4(d.site, tag, sweep, 0u), hp, &nl);
-    if constexpr (MEAS) plaq.add(qdot(t ? L.put(2 * mu + p, d.h, nl) : ldl<P, NC>(L, 2 * mu + p, d.h), d.lower));
+    if constexpr (MEAS) plaq.add(qdot_rn(t ? L.put(2 * mu + p, d.h, nl) : ldl<P, NC>(L, 2 * mu + p, d.h), d.lower));
     else if (t) L.st(2 * mu + p, d.h, nl);
     cnt.trials += t ? (unsigned)t : (unsigned)hp.max_tries;
     cnt.capped += t == 0;
@@ -172,9 +172,9 @@ __device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Su
   using R = typename Real<P>::T;
   using M = Math<R>;
   const Site x = site_from_half(g, (uint32_t)h, p);
-  const Quat<R> u = ldl<P, NC>(L, 2 * mu + p, h);
-  Quat<R> sig;
+  Quat<R> sig, u;
   if constexpr (P == kF64) {
+    u = ldl<P, NC>(L, 2 * mu + p, h);
     FixSum s;
     FixBad bad{0u, 0u};
     const bool ok = staple_fixed<false, NC, false>(L, g, x, h, mu, p, 4, s, sig);
@@ -191,11 +191,12 @@ __device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Su
   } else {
     sig = staple<P, MU, 0xF, NC>(L, g, x, h, p);
   }
-  const R k2 = qdot(sig, sig);
+  const R k2 = qdot_rn(sig, sig);
   if (!(k2 >= M::kTiny)) return;
   const Quat<R> w = qscale(sig, M::rsqrt(k2));
-  Quat<R> v = qmul(qmul_nd(w, u), w);
-  if constexpr (P != kF64) v = qscale(v, M::rsqrt(qdot(v, v)));
+  if constexpr (P != kF64) u = ldl<P, NC>(L, 2 * mu + p, h);   // the staple's registers are free
+  Quat<R> v = qmul_rn(qmul_nd_rn(w, u), w);
+  if constexpr (P != kF64) v = qscale(v, M::rsqrt(qdot_rn(v, v)));
   L.st(2 * mu + p, h, v);
 }
 

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(BS, 2 * SmallPerSM<P>::value / BS)
   }
   R plaq = R(0);
   if (valid) {
-    if constexpr (MEAS) plaq = qdot(found ? L.put(2 * mu + p, h, nl) : L.ldc(2 * mu + p, h), lower);
+    if constexpr (MEAS) plaq = qdot_rn(found ? L.put(2 * mu + p, h, nl) : L.ldc(2 * mu + p, h), lower);
     else if (found) L.st(2 * mu + p, h, nl);
   }
   if constexpr (MEAS) {
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(64, 8)
   const bool writes = valid && j == 0;
   double plaq = 0.0;
   if (writes) {
-    if constexpr (MEAS) plaq = qdot(found ? L.put(2 * mu + p, h, nl) : L.ldc(2 * mu + p, h), lower);
+    if constexpr (MEAS) plaq = qdot_rn(found ? L.put(2 * mu + p, h, nl) : L.ldc(2 * mu + p, h), lower);
     else if (found) L.st(2 * mu + p, h, nl);
   }
   if constexpr (MEAS) {

@@ -42,8 +42,7 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // Whether a lattice's kernels overlap so: while one substep's threads fit twice,
 // at the heat bath's registers (the small-lattice kernels).  Larger lattices'
 // kernels do not trigger and use read-only loads (64^4 FP32, plain against
-// read-only: plaquette 348 and 317 us, Polyakov loop 58 and 50, APE step 349 and
-// 345).
+// read-only: APE step 350 and 344 us, Polyakov loop the same).
 template <int P> struct SmallPerSM { static constexpr int value = P == kF64 ? 256 : 512; };
 static inline bool overlaps(const LatticeView& v) {
   return v.g.vh <= (int64_t)(v.prec == kF64 ? SmallPerSM<kF64>::value : SmallPerSM<kF32>::value) * device_info().sms;

@@ -10,6 +10,7 @@
 // kernels: per-thread sums (compensated when the arithmetic is FP32), FP64
 // warp shuffles, one partial per block and a last-block finisher that adds
 // the partials in a fixed order, so a result is reproducible run to run.
+#define SU2_COMPILER_FUSES
 #include <algorithm>
 #include <atomic>
 #include <cfloat>
