@@ -226,8 +226,8 @@ SU2_HD int64_t fix_mulhi(int64_t a, int64_t b) {
 // Table of -ln u: the leading 7 fraction bits i of the significand m select
 // a 16-bit reciprocal I of the interval's centre 1 + (i + 1/2)/128, and
 // t = ln(I 2^-16) in units of 2^-58 (Tang's table-driven logarithm, ACM TOMS
-// 16, 1990).
-struct FixLog { int64_t t; int64_t inv; };
+// 16, 1990).  Aligned for the 16-byte load of an entry.
+struct alignas(16) FixLog { int64_t t; int64_t inv; };
 #define SU2_FIX_LOG_TABLE                                                                                     \
   {-1123689413616504ll, 65281}, {-3357597927618363ll, 64777}, {-5573081980516173ll, 64281}, {-7774097633284494ll, 63792}, \
   {-9960179792198405ll, 63310}, {-12126270533003689ll, 62836}, {-14276411659491797ll, 62369}, {-16410121222244478ll, 61909}, \
@@ -281,6 +281,7 @@ SU2_HD int64_t fix_neg_log(uint32_t x) {
   const uint64_t zn = z << lz;
   const uint32_t i = (uint32_t)(zn >> 56) & 127u;
 #ifdef __CUDA_ARCH__
+  static_assert(sizeof(FixLog) == sizeof(longlong2) && alignof(FixLog) >= alignof(longlong2), "one load an entry");
   const longlong2 e = __ldg(reinterpret_cast<const longlong2*>(fix_log_table) + i);
   const int64_t t = e.x;
   const uint32_t inv = (uint32_t)e.y;

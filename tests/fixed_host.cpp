@@ -14,6 +14,8 @@ static FixQuat link(const double* v, int conj, FixBad& bad) {
 
 extern "C" {
 int fixed_frac() { return kFixFrac; }
+int fixed_log_entry_alignment() { return (int)alignof(FixLog); }
+int fixed_log_entry_size() { return (int)sizeof(FixLog); }
 // out[4]: the converted components, v = h 2^29 + l; returns fix_ok
 int fixed_link(const double* v, int conj, int64_t* out) {
   FixBad bad{0, 0};

@@ -123,6 +123,12 @@ def test_sums_of_products_are_closer_than_fp64(lib):
     assert np.sqrt(np.mean(np.square(off))) < 0.25 * np.sqrt(np.mean(np.square(off64)))
 
 
+def test_log_table_entries_are_aligned_for_their_16_byte_load(lib):
+    # the device reads an entry (two 8-byte words) by one 16-byte load
+    assert lib.fixed_log_entry_size() == 16
+    assert lib.fixed_log_entry_alignment() == 16
+
+
 def _draws():
     rng = np.random.default_rng(4)
     edge = [0, 1, 2, 3, (1 << 32) - 1, (1 << 32) - 2, (1 << 31) - 1, 1 << 31, (1 << 30) - 1, 1 << 30, 3 << 30, (3 << 30) - 1,
