@@ -327,7 +327,7 @@ int su2_ape_smear(su2_lattice* h, double alpha, int n);
  * su2_ape_smear (SU2_ESTATE if there is none since the last sweep or
  * set_links); temporal links are always the chain's.  For Rmax, Tmax <= 16,
  * N3 <= 64 and planes that fit a multiprocessor's shared memory (spatial extents
- * to 64; FP64: unit quaternions only) the loops are evaluated in temporal gauge
+ * to 64; unit quaternions only) the loops are evaluated in temporal gauge
  * (the loop is gauge invariant: after the transform each is one dot
  * product of two spatial lines), which equals the direct product up to
  * rounding; other shapes multiply the loops out.  Synchronises.

@@ -742,13 +742,9 @@ extern "C" int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smea
   DeviceGuard dg(h->device);
   const void* spatial = use_smeared ? h->ape[h->smeared - 1] : h->links;
   const int n = Rmax * Tmax;
-  if (h->prec != SU2_F64) {
-    SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, nullptr, h->stream));
-    return fetch_out(h, n, out);
-  }
-  // FP64: the fixed-point kernel reports links that are not unit quaternions
-  // (a store filled from outside) in the word behind the results; the loops are
-  // then multiplied out in FP64
+  // the temporal-gauge kernel reports links that are not unit quaternions (a
+  // store filled from outside) in the word behind the results; the loops are
+  // then multiplied out
   h->h_out[n] = 0.0;  // every call that writes results has waited for them
   SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, h->scratch.out + n, h->stream));
   double got[32 * 32 + 1];

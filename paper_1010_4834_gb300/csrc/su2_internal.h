@@ -107,9 +107,9 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
 cudaError_t launch_ape(const LatticeView& src, void* dst, double alpha, cudaStream_t st);
 cudaError_t launch_copy_spatial(const LatticeView& src, void* dst, cudaStream_t st);
 // Wilson loops: spatial links from `spatial` (6 classes), time links from v.
-// FP64: *flag (device, zero before) is set to 1 if the kernel met links that are
-// not unit quaternions and its result is void; with flag = nullptr the kernels
-// that take any links run.
+// *flag (device, zero before) is set to 1 if the kernel met links that are not
+// unit quaternions and its result is void; with flag = nullptr the kernels that
+// take any links run.
 cudaError_t launch_wilson(const LatticeView& v, const void* spatial, int rmax, int tmax,
                           const Scratch& s, double* flag, cudaStream_t st);
 // Canonical FP64 host layout <-> device store, for sites [s0, s0 + ns).

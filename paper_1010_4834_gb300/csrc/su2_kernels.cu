@@ -810,21 +810,24 @@ constexpr int kTgCols = 32 / kTgChunks;  // columns of a warp
 constexpr int kTgExt = kTgT / kTgChunks; // extended rows a lane owns
 constexpr int kTgThreads = 512;          // planes of up to 64 columns
 
-// q / |q|.  Near |q| = 1 as q + q d, d = (1 - |q|^2) / 2 + ...: a scale factor is
+// q / |q| for |q| near one, as q + q d, d = (1 - |q|^2) / 2: a scale factor is
 // itself rounded, to 2^-24 below 1 and 2^-23 above, and the approximate root's
 // error near 1 has one sign, which came back four times in every loop (16^4 FP32,
 // W to 8 x 8, off FP64: 7.8e-7 with the root, 4.1e-7 with a Newton step on it).
-__device__ __forceinline__ Quat<float> qunit(const Quat<float>& q) {
+// `bad` is raised from |q|^2 off one by 2^-18 on (the links of FP32 chains stay
+// within 1.1e-6 = 2^-19.8): the kernel drops the time links' norms, which up to
+// there changes a loop by less than 1e-6.
+__device__ __forceinline__ Quat<float> qunit(const Quat<float>& q, bool& bad) {
   const float e = fmaf(-q.w, q.w, fmaf(-q.x, q.x, fmaf(-q.y, q.y, fmaf(-q.z, q.z, 1.0f))));
-  if (fabsf(e) > 0x1p-10f) return qscale(q, rsqrtf(qdot(q, q)));   // links set from outside
-  const float d = e * fmaf(0.375f, e, 0.5f);
+  bad |= !(fabsf(e) <= 0x1p-18f);
+  const float d = 0.5f * e;
   return qmake<float>(fmaf(q.w, d, q.w), fmaf(q.x, d, q.x), fmaf(q.y, d, q.y), fmaf(q.z, d, q.z));
 }
 
 // The kernel's arithmetic: FP32 quaternions with FP32 sums, or (FP64) the
 // 58-bit fixed point of su2_fixed.cuh with 64-bit sums in units of 2^-52 (one
-// plane's sum of one (R, T) and warp is below 2^60).  In fixed point a link
-// must be a unit quaternion to 2^-29 (`bad` is raised otherwise).  The gauge
+// plane's sum of one (R, T) and warp is below 2^60).  The time links must be unit
+// quaternions, in fixed point all links to 2^-29 (`bad` is raised otherwise).  The gauge
 // transform normalises the time lines, whose links are unit quaternions only to
 // FP64 rounding (together about 1e-16 a link below one in a typical store, 1e-15
 // on a loop of T = 12); FP64 sums the time links' |U|^2 - 1 on the way (`excess`),
@@ -837,7 +840,7 @@ template <int P> struct TgMath {
   static __device__ __forceinline__ E one() { return qone<float>(); }
   static __device__ __forceinline__ E mul(const E& a, const E& b) { return qmul(a, b); }
   static __device__ __forceinline__ E mul_nd(const E& a, const E& b) { return qmul_nd(a, b); }
-  static __device__ __forceinline__ E unit(const E& q) { return qunit(q); }
+  static __device__ __forceinline__ E unit(const E& q, bool& bad) { return qunit(q, bad); }
   static __device__ __forceinline__ A dot(const E& a, const E& b, A s) {
     return fma(a.w, b.w, fma(a.x, b.x, fma(a.y, b.y, fma(a.z, b.z, s))));
   }
@@ -861,7 +864,7 @@ template <> struct TgMath<kF64> {
   static __device__ __forceinline__ Fix scaled(const Fix& a, int e) {
     return fix_split(fix_value(a) + (((int64_t)a.h * e) >> kFixLow));
   }
-  static __device__ __forceinline__ E unit(const E& q) {
+  static __device__ __forceinline__ E unit(const E& q, bool&) {
     const int e = (int)(-fix_dot(q, q, -((int64_t)1 << kFixFrac)) >> 1);
     return E{scaled(q.w, e), scaled(q.x, e), scaled(q.y, e), scaled(q.z, e)};
   }
@@ -966,7 +969,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
         Sb[tg_row<RO>(r0 + i, SS) + a] = L;
-        L = M::unit(M::mul(L, ut[i]));
+        L = M::unit(M::mul(L, ut[i]), bad);
       }
       Ct[c * nm + a] = L;
     }
@@ -974,15 +977,15 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     // (2) prefix over the chunks: G(a, r) for the thread's rows, P(a) = G(a, Nt)
     if (active) {
       E Q = M::one();
-      for (int k = 0; k < c; ++k) Q = M::unit(M::mul(Q, Ct[k * nm + a]));
+      for (int k = 0; k < c; ++k) Q = M::unit(M::mul(Q, Ct[k * nm + a]), bad);
       if (c > 0) {
 #pragma unroll
         for (int i = 0; i < RO; ++i) {
           E* p = Sb + tg_row<RO>(r0 + i, SS) + a;
-          *p = M::unit(M::mul(Q, *p));
+          *p = M::unit(M::mul(Q, *p), bad);
         }
       }
-      if (c == kTgChunks - 1) Pb[a] = M::unit(M::mul(Q, Ct[c * nm + a]));
+      if (c == kTgChunks - 1) Pb[a] = M::unit(M::mul(Q, Ct[c * nm + a]), bad);
     }
     __syncthreads();
     // (3) U'(a, r) = G(a, t) U_mu(a, t) G(a+1, t)^dag for the lane's rows,
@@ -1438,7 +1441,7 @@ template <int P>
 static cudaError_t launch_wilson_tg(const LatticeView& v, const void* spatial, int rmax, int tmax,
                                     const Scratch& s, double* flag, cudaStream_t st, bool* used) {
   *used = false;
-  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || (P == kF64 && !flag)) return cudaSuccess;
+  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || !flag) return cudaSuccess;
   auto launch = [&](auto rows) -> cudaError_t {
     constexpr int RO = decltype(rows)::value;
     if (P != kF64 && v.g.n[3] == kTgChunks * RO)
