@@ -330,7 +330,9 @@ int su2_ape_smear(su2_lattice* h, double alpha, int n);
  * to 64; unit quaternions only) the loops are evaluated in temporal gauge
  * (the loop is gauge invariant: after the transform each is one dot
  * product of two spatial lines), which equals the direct product up to
- * rounding; other shapes multiply the loops out.  Synchronises.
+ * rounding; other shapes, and links further from unit norm than a chain
+ * leaves them (|U|^2 off one by 4e-6 in FP32, 7e-15 in FP64), multiply
+ * the loops out.  Synchronises.
  */
 int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smeared, double* out);
 

@@ -831,12 +831,16 @@ __device__ __forceinline__ Quat<float> qunit(const Quat<float>& q, bool& bad) {
 // transform normalises the time lines, whose links are unit quaternions only to
 // FP64 rounding (together about 1e-16 a link below one in a typical store, 1e-15
 // on a loop of T = 12); FP64 sums the time links' |U|^2 - 1 on the way (`excess`),
-// and the loops of extent T get the factor 1 + T <|U|^2 - 1> back.
+// and the loops of extent T get the factor 1 + T <|U|^2 - 1> back.  That gives back
+// the mean norm, not a loop's own: FP64 raises `bad` where a time link's |U|^2 is
+// off one by 2^-47 (7e-15; heat-bath links stay within 7e-16), below which the
+// difference is within FP64's rounding of the loop (norms 1e-9 up in half of the
+// lattice and down in the other half: 2.5e-10 at T = 12).
 template <int P> struct TgMath {
   using E = Quat<float>;
   using A = float;
   static __device__ __forceinline__ E load(const Links<P>& L, int cls, int h, bool&) { return L.ld(cls, h); }
-  static __device__ __forceinline__ int64_t excess(const E&) { return 0; }
+  static __device__ __forceinline__ int64_t excess(const E&, bool&) { return 0; }
   static __device__ __forceinline__ E one() { return qone<float>(); }
   static __device__ __forceinline__ E mul(const E& a, const E& b) { return qmul(a, b); }
   static __device__ __forceinline__ E mul_nd(const E& a, const E& b) { return qmul_nd(a, b); }
@@ -853,8 +857,13 @@ template <> struct TgMath<kF64> {
   static __device__ __forceinline__ E load(const Links<kF64>& L, int cls, int h, bool& bad) {
     return fix_unit_link(L.ld(cls, h), bad);
   }
-  // |q|^2 - 1 in units of 2^-58
-  static __device__ __forceinline__ int64_t excess(const E& q) { return fix_dot(q, q, -((int64_t)1 << kFixFrac)); }
+  // a time link's |q|^2 - 1 in units of 2^-58
+  static __device__ __forceinline__ int64_t excess(const E& q, bool& bad) {
+    constexpr int64_t most = (int64_t)1 << (kFixFrac - 47);
+    const int64_t x = fix_dot(q, q, -((int64_t)1 << kFixFrac));
+    bad |= x < -most || x > most;
+    return x;
+  }
   static __device__ __forceinline__ E one() { return fix_one(); }
   static __device__ __forceinline__ E mul(const E& a, const E& b) { return fix_mul(a, b); }
   static __device__ __forceinline__ E mul_nd(const E& a, const E& b) {
@@ -957,7 +966,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
       for (int i = 0; i < RO; ++i) {
         const int t = slice(r0 + i), h = h0 + hts * t, par = (par0 ^ t) & 1;
         ut[i] = EXACT || r0 + i < nt ? M::load(Lt, 6 + par, h, bad) : M::one();
-        over += M::excess(ut[i]);
+        over += M::excess(ut[i], bad);
         us[i] = M::load(Ls, 2 * mu + par, h, bad);
       }
 #pragma unroll
