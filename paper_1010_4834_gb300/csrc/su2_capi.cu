@@ -743,16 +743,17 @@ extern "C" int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smea
   const void* spatial = use_smeared ? h->ape[h->smeared - 1] : h->links;
   const int n = Rmax * Tmax;
   // the temporal-gauge kernel reports links that are not unit quaternions (a
-  // store filled from outside) in the word behind the results; the loops are
-  // then multiplied out
-  h->h_out[n] = 0.0;  // every call that writes results has waited for them
-  SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, h->scratch.out + n, h->stream));
+  // store filled from outside) in the word behind the results; then its form that
+  // keeps norms runs (FP64), and if they are too far off that, the kernels that
+  // multiply the loops out
   double got[32 * 32 + 1];
-  int rc = fetch_out(h, n + 1, got);
-  if (rc) return rc;
-  if (got[n] != 0.0) {
-    SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, nullptr, h->stream));
-    return fetch_out(h, n, out);
+  for (WilsonLinks links : {kWilsonUnit, kWilsonNear, kWilsonAny}) {
+    if (links == kWilsonNear && h->prec != SU2_F64) continue;
+    h->h_out[n] = 0.0;  // every call that writes results has waited for them
+    SU2_CU(launch_wilson(view(h), spatial, Rmax, Tmax, h->scratch, links, h->scratch.out + n, h->stream));
+    int rc = fetch_out(h, n + 1, got);
+    if (rc) return rc;
+    if (got[n] == 0.0) break;
   }
   std::memcpy(out, got, n * sizeof(double));
   return SU2_OK;

@@ -350,18 +350,19 @@ __device__ __forceinline__ Quat<double> fix_sum_to_double(const FixSum& s) {
                        fix_to_double(fix_fold(s.hy, s.my)), fix_to_double(fix_fold(s.hz, s.mz)));
 }
 
-// A link that must be a unit quaternion to 2^-29, whatever its components
+// A link whose |q|^2 must be within 2^-BITS of one, whatever its components
 // (zero, tiny); `bad` is raised otherwise.
+template <int BITS = 28>
 __device__ __forceinline__ FixQuat fix_unit_link(const Quat<double>& q, bool& bad) {
   FixQuat f;
   f.w = fix_from_any((uint32_t)__double2loint(q.w), (uint32_t)__double2hiint(q.w));
   f.x = fix_from_any((uint32_t)__double2loint(q.x), (uint32_t)__double2hiint(q.x));
   f.y = fix_from_any((uint32_t)__double2loint(q.y), (uint32_t)__double2hiint(q.y));
   f.z = fix_from_any((uint32_t)__double2loint(q.z), (uint32_t)__double2hiint(q.z));
-  // components below 2 (the conversion's range) and |q|^2 within 2^-28 of one
+  // components below 2 (the conversion's range)
   const uint32_t top = (uint32_t)(__double2hiint(q.w) | __double2hiint(q.x) | __double2hiint(q.y) | __double2hiint(q.z));
-  const int64_t off = fix_dot(f, f, -((int64_t)1 << kFixFrac)) + ((int64_t)1 << (kFixFrac - 28));
-  bad |= (top & 0x40000000u) != 0u || (uint64_t)off >> (kFixFrac - 27) != 0u;
+  const int64_t off = fix_dot(f, f, -((int64_t)1 << kFixFrac)) + ((int64_t)1 << (kFixFrac - BITS));
+  bad |= (top & 0x40000000u) != 0u || (uint64_t)off >> (kFixFrac - BITS + 1) != 0u;
   return f;
 }
 

@@ -107,11 +107,16 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
 cudaError_t launch_ape(const LatticeView& src, void* dst, double alpha, cudaStream_t st);
 cudaError_t launch_copy_spatial(const LatticeView& src, void* dst, cudaStream_t st);
 // Wilson loops: spatial links from `spatial` (6 classes), time links from v.
-// *flag (device, zero before) is set to 1 if the kernel met links that are not
-// unit quaternions and its result is void; with flag = nullptr the kernels that
-// take any links run.
+// links: what the kernel may take them for.  *flag (device, zero before) is set to
+// 1 if they are not that, and the result is void.  Shapes that the temporal-gauge
+// kernel does not take run the kernels that take any links.
+enum WilsonLinks {
+  kWilsonUnit,   // unit quaternions, up to the rounding of a chain
+  kWilsonNear,   // FP64: |U|^2 within 2^-16 of one
+  kWilsonAny
+};
 cudaError_t launch_wilson(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                          const Scratch& s, double* flag, cudaStream_t st);
+                          const Scratch& s, WilsonLinks links, double* flag, cudaStream_t st);
 // Canonical FP64 host layout <-> device store, for sites [s0, s0 + ns).
 cudaError_t launch_to_canonical(const LatticeView& v, double* canon, int64_t s0, int64_t ns,
                                 cudaStream_t st);

@@ -827,8 +827,8 @@ __device__ __forceinline__ Quat<float> qunit(const Quat<float>& q, bool& bad) {
 // The kernel's arithmetic: FP32 quaternions with FP32 sums, or (FP64) the
 // 58-bit fixed point of su2_fixed.cuh with 64-bit sums in units of 2^-52 (one
 // plane's sum of one (R, T) and warp is below 2^60).  The time links must be unit
-// quaternions, in fixed point all links to 2^-29 (`bad` is raised otherwise).  The gauge
-// transform normalises the time lines, whose links are unit quaternions only to
+// quaternions, in fixed point all links to 2^-29 (`bad` is raised otherwise; NORMS,
+// below, takes more).  The gauge transform normalises the time lines, whose links are unit quaternions only to
 // FP64 rounding (together about 1e-16 a link below one in a typical store, 1e-15
 // on a loop of T = 12); FP64 sums the time links' |U|^2 - 1 on the way (`excess`),
 // and the loops of extent T get the factor 1 + T <|U|^2 - 1> back.  That gives back
@@ -839,7 +839,9 @@ __device__ __forceinline__ Quat<float> qunit(const Quat<float>& q, bool& bad) {
 template <int P> struct TgMath {
   using E = Quat<float>;
   using A = float;
-  static __device__ __forceinline__ E load(const Links<P>& L, int cls, int h, bool&) { return L.ld(cls, h); }
+  template <bool> static __device__ __forceinline__ E load(const Links<P>& L, int cls, int h, bool&) {
+    return L.ld(cls, h);
+  }
   static __device__ __forceinline__ int64_t excess(const E&, bool&) { return 0; }
   static __device__ __forceinline__ E one() { return qone<float>(); }
   static __device__ __forceinline__ E mul(const E& a, const E& b) { return qmul(a, b); }
@@ -854,8 +856,8 @@ template <int P> struct TgMath {
 template <> struct TgMath<kF64> {
   using E = FixQuat;
   using A = int64_t;
-  static __device__ __forceinline__ E load(const Links<kF64>& L, int cls, int h, bool& bad) {
-    return fix_unit_link(L.ld(cls, h), bad);
+  template <bool NORMS> static __device__ __forceinline__ E load(const Links<kF64>& L, int cls, int h, bool& bad) {
+    return fix_unit_link<NORMS ? 16 : 28>(L.ld(cls, h), bad);
   }
   // a time link's |q|^2 - 1 in units of 2^-58
   static __device__ __forceinline__ int64_t excess(const E& q, bool& bad) {
@@ -880,6 +882,30 @@ template <> struct TgMath<kF64> {
   static __device__ __forceinline__ A dot(const E& a, const E& b, A s) { return s + (fix_dot(a, b, 32) >> 6); }
   static __device__ __forceinline__ double value(A s) { return fix_to_double<52>(s); }
 };
+
+// A factor near one: its excess over one and that of its inverse, units of 2^-58.
+struct TgNorm { int64_t d, i; };
+__device__ __forceinline__ int64_t tg_times(int64_t x, int64_t y) { return x + y + fix_mulhi(x, y * 64); }
+__device__ __forceinline__ TgNorm tg_times(const TgNorm& a, const TgNorm& b) {
+  return TgNorm{tg_times(a.d, b.d), tg_times(a.i, b.i)};
+}
+__device__ __forceinline__ Fix tg_scaled(const Fix& a, int64_t x) {
+  const int64_t v = fix_value(a);
+  return fix_split(v + fix_mulhi(v, x * 64));
+}
+__device__ __forceinline__ FixQuat tg_scaled(const FixQuat& q, int64_t x) {
+  return FixQuat{tg_scaled(q.w, x), tg_scaled(q.x, x), tg_scaled(q.y, x), tg_scaled(q.z, x)};
+}
+// |q|; q becomes q / |q|.  With e = |q|^2 - 1, |e| <= 2^-16: the square root's and
+// its inverse's binomial series to e^3 (e^4 is below 2^-63).
+__device__ __forceinline__ TgNorm tg_take_norm(FixQuat& q) {
+  const int64_t e = fix_dot(q, q, -((int64_t)1 << kFixFrac));
+  const int64_t x = (int64_t)((uint64_t)e << 20);                  // 2^-78
+  const int64_t e2 = fix_mulhi(x, x), e3 = fix_mulhi(e2, x);       // 2^-92, 2^-106
+  const TgNorm n{(e >> 1) - (e2 >> 37) + (e3 >> 52), ((3 * e2) >> 37) - (e >> 1) - ((5 * e3) >> 52)};
+  q = tg_scaled(q, n.i);
+  return n;
+}
 
 // Site (column a, slice 0) of the plane (mu, c1, c2).
 __device__ __forceinline__ Site plane_site(const Geom& g, int mu, int a, int c1, int c2) {
@@ -913,7 +939,15 @@ template <int RO> __device__ __forceinline__ int tg_row(int r, int stride) {
 
 // EXACT: Nt is a multiple of eight (every origin row starts loops), compiled
 // without the tests.
-template <int P, int RO, bool EXACT>
+// NORMS (FP64): links up to 2^-16 off unit norm (in |U|^2; a configuration stored
+// in FP32, say).  A loop carries the product of its time links' norms, N(a, r + T)
+// N(a + R, r + T) / (N(a, r) N(a + R, r)) with N(a, r) the norms' product along
+// column a up to row r: the lines published to the other lanes get the factor N N
+// of their two columns, the lines that loops start from its inverse.
+// 32^4, links rounded to FP32, W(16,16): 82 ms multiplied out by the time-outer
+// kernel, here 4.7, after the 3.4 of the kernel without NORMS that found them.
+// Compiled for even RO.
+template <int P, int RO, bool EXACT, bool NORMS>
 __global__ void __launch_bounds__(kTgThreads, 1)
     k_wilson_tg(Links<P> Ls, Links<P> Lt, Geom g, int rmax, int tmax, double* partials, double* flag,
                 unsigned long long* excess) {
@@ -951,6 +985,9 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     E* Sb = Ue + (NO + kTgT) * SU + 4;           // Sb[tg_row(r, SS) + a]: G(a, r), then S'_R(a, r)
     E* Ct = Sb + (NO + kTgT) * SS + 4;           // Ct[k nm + a]: product of scan chunk k
     E* Pb = Ct + kTgChunks * nm;                 // Pb[a] = P(a)
+    TgNorm* Nb = reinterpret_cast<TgNorm*>(Pb + nm);   // NORMS: Nb[r nm + a] = N(a, r), r < NO
+    TgNorm* Nc = Nb + NO * nm;                   // norms of the scan chunks
+    TgNorm* Np = Nc + kTgChunks * nm;            // Np[a] = N(a, Nt)
     const int a = kTgCols * warp + lane % kTgCols;
     const bool active = a < nm;
     __syncthreads();  // the previous plane's readers are done
@@ -965,14 +1002,23 @@ __global__ void __launch_bounds__(kTgThreads, 1)
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
         const int t = slice(r0 + i), h = h0 + hts * t, par = (par0 ^ t) & 1;
-        ut[i] = EXACT || r0 + i < nt ? M::load(Lt, 6 + par, h, bad) : M::one();
-        over += M::excess(ut[i], bad);
-        us[i] = M::load(Ls, 2 * mu + par, h, bad);
+        ut[i] = EXACT || r0 + i < nt ? M::template load<NORMS>(Lt, 6 + par, h, bad) : M::one();
+        if constexpr (!NORMS) over += M::excess(ut[i], bad);
+        us[i] = M::template load<NORMS>(Ls, 2 * mu + par, h, bad);
       }
 #pragma unroll
       for (int e = 0; e < kTgExt; ++e) {
         const int t = slice(NO + kTgExt * c + e), h = h0 + hts * t, par = (par0 ^ t) & 1;
-        us[RO + e] = M::load(Ls, 2 * mu + par, h, bad);
+        us[RO + e] = M::template load<NORMS>(Ls, 2 * mu + par, h, bad);
+      }
+      if constexpr (NORMS) {
+        TgNorm n{0, 0};
+#pragma unroll
+        for (int i = 0; i < RO; ++i) {
+          Nb[(r0 + i) * nm + a] = n;
+          n = tg_times(n, tg_take_norm(ut[i]));
+        }
+        Nc[c * nm + a] = n;
       }
       E L = M::one();
 #pragma unroll
@@ -995,6 +1041,12 @@ __global__ void __launch_bounds__(kTgThreads, 1)
         }
       }
       if (c == kTgChunks - 1) Pb[a] = M::unit(M::mul(Q, Ct[c * nm + a]), bad);
+      if constexpr (NORMS) {
+        TgNorm n{0, 0};
+        for (int k = 0; k < c; ++k) n = tg_times(n, Nc[k * nm + a]);
+        for (int i = 0; i < RO; ++i) Nb[(r0 + i) * nm + a] = tg_times(n, Nb[(r0 + i) * nm + a]);
+        if (c == kTgChunks - 1) Np[a] = tg_times(n, Nc[c * nm + a]);
+      }
     }
     __syncthreads();
     // (3) U'(a, r) = G(a, t) U_mu(a, t) G(a+1, t)^dag for the lane's rows,
@@ -1020,7 +1072,16 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     const int bu = r0 * SU + sk + a, bs = r0 * SS + sk + a;
     const int bue = (NO + kTgExt * c) * SU + a, bse = (NO + kTgExt * c) * SS + a;
     const int rows = nt - r0;  // loops start from the first `rows` of the lane's origin rows
-    E own[RO];  // the origin rows' lines; the extended rows' stay in Sb
+    E own[RO];  // the origin rows' lines; the extended rows' stay in Sb (NORMS: in ext)
+    E from[NORMS ? RO : 1], ext[NORMS ? kTgExt : 1];   // NORMS: the lines that loops start from
+    auto norms = [&](int r, int b) {   // N(a, r) N(b, r)
+      TgNorm n{0, 0};
+      for (int col : {a, b}) {
+        const TgNorm m = Nb[slice(r) * nm + col];
+        n = tg_times(n, r < nt ? m : tg_times(m, Np[col]));
+      }
+      return n;
+    };
     A acc[kTgT];
 #pragma unroll
     for (int k = 0; k < kTgT; ++k) acc[k] = A(0);
@@ -1030,13 +1091,24 @@ __global__ void __launch_bounds__(kTgThreads, 1)
         for (int i = 0; i < RO; ++i) {
           const E v = Ue[bu + i * SU + Rl - 1];
           own[i] = Rl == 1 ? v : M::mul(own[i], v);
-          Sb[bs + i * SS] = own[i];
+          if constexpr (NORMS) {
+            const TgNorm n = norms(r0 + i, a + Rl < nm ? a + Rl : a + Rl - nm);
+            Sb[bs + i * SS] = tg_scaled(own[i], n.d);
+            from[i] = tg_scaled(own[i], n.i);
+          } else {
+            Sb[bs + i * SS] = own[i];
+          }
         }
 #pragma unroll
         for (int e = 0; e < kTgExt; ++e) {
           const E v = Ue[bue + e * SU + Rl - 1];
           E* p = Sb + bse + e * SS;
-          *p = Rl == 1 ? v : M::mul(*p, v);
+          if constexpr (NORMS) {
+            ext[e] = Rl == 1 ? v : M::mul(ext[e], v);
+            *p = tg_scaled(ext[e], norms(NO + kTgExt * c + e, a + Rl < nm ? a + Rl : a + Rl - nm).d);
+          } else {
+            *p = Rl == 1 ? v : M::mul(*p, v);
+          }
         }
       }
       __syncwarp();
@@ -1050,7 +1122,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
           for (int j = 1; j < RO + kTgT; ++j) {
             if (!FULL && j >= RO + tmax) break;
             E w;
-            if (j < RO) {
+            if (!NORMS && j < RO) {
               w = own[j < RO ? j : 0];
             } else {
               const int rr = r0 + j;  // chunk c + j / RO while an origin row
@@ -1059,7 +1131,8 @@ __global__ void __launch_bounds__(kTgThreads, 1)
 #pragma unroll
             for (int i = 0; i < RO; ++i) {
               const int T = j - i;
-              if (T >= 1 && T <= kTgT && (FULL || (T <= tmax && (EXACT || i < rows)))) acc[T - 1] = M::dot(own[i], w, acc[T - 1]);
+              if (T >= 1 && T <= kTgT && (FULL || (T <= tmax && (EXACT || i < rows))))
+                acc[T - 1] = M::dot(NORMS ? from[NORMS ? i : 0] : own[i], w, acc[T - 1]);
             }
           }
         };
@@ -1099,7 +1172,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     }
   }
   if (bad) *flag = 1.0;
-  if constexpr (P == kF64) {
+  if constexpr (P == kF64 && !NORMS) {
     over = warp_sum(over);
     if (lane == 0) atomicAdd(excess, (unsigned long long)over);   // exact in any order
   }
@@ -1391,7 +1464,7 @@ static cudaError_t launch_wilson_rt(const LatticeView& v, const void* spatial, i
 // The temporal-gauge kernel when R and T are at most 16, Nt is at most 64, one
 // block holds four columns a warp of the widest plane, and the staged plane
 // fits in shared memory; *used = false otherwise.
-template <int P, int RO, bool EXACT>
+template <int P, int RO, bool EXACT, bool NORMS>
 static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spatial, int rmax, int tmax,
                                          const Scratch& s, double* flag, cudaStream_t st, bool* used) {
   using E = typename TgMath<P>::E;
@@ -1405,11 +1478,12 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, k_wilson_tg<P, RO, EXACT>);
+  cudaError_t e = cudaFuncGetAttributes(&fa, k_wilson_tg<P, RO, EXACT, NORMS>);
   if (e != cudaSuccess) return e;
   const int64_t smem = ((int64_t)nr * tg_stride<RO>(nmax + rmax - 1) + 4 + (int64_t)nr * tg_stride<RO>(nmax) + 4 +
                         (int64_t)kTgChunks * nmax + nmax) *
-                       (int64_t)sizeof(E);
+                       (int64_t)sizeof(E) +
+                       (NORMS ? (int64_t)(kTgChunks * RO + kTgChunks + 1) * nmax * (int64_t)sizeof(TgNorm) : 0);
   const int64_t dyn_max = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
   if (smem > dyn_max) return cudaSuccess;
   // raised once per device, as for the time-outer kernel
@@ -1418,12 +1492,12 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   if (dev >= 0 && dev < 64) {
     const int lim = (int)dyn_max;
     std::call_once(attr_once[dev], [dev, lim]() {
-      attr_err[dev] = cudaFuncSetAttribute(k_wilson_tg<P, RO, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      attr_err[dev] = cudaFuncSetAttribute(k_wilson_tg<P, RO, EXACT, NORMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     });
     if (attr_err[dev] != cudaSuccess) return attr_err[dev];
   }
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wilson_tg<P, RO, EXACT>, nth, (size_t)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_wilson_tg<P, RO, EXACT, NORMS>, nth, (size_t)smem);
   if (per_sm < 1) per_sm = 1;
   const int64_t nunits = (int64_t)v.g.n[1] * v.g.n[2] + (int64_t)v.g.n[0] * v.g.n[2] + (int64_t)v.g.n[0] * v.g.n[1];
   int64_t gx = (int64_t)device_info().sms * per_sm;
@@ -1434,10 +1508,10 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   auto Lt = links_of<P>(v.links, v.g.vh);
   auto Ls = links_of<P>(const_cast<void*>(spatial), v.g.vh);
   // a word of the counters' 256 bytes, away from the reductions' own
-  unsigned long long* excess = P == kF64 ? reinterpret_cast<unsigned long long*>(s.counter + 32) : nullptr;
+  unsigned long long* excess = P == kF64 && !NORMS ? reinterpret_cast<unsigned long long*>(s.counter + 32) : nullptr;
   if (excess) e = cudaMemsetAsync(excess, 0, sizeof *excess, st);
   if (e != cudaSuccess) return e;
-  k_wilson_tg<P, RO, EXACT><<<(unsigned)gx, nth, (size_t)smem, st>>>(Ls, Lt, v.g, rmax, tmax, s.partials, flag, excess);
+  k_wilson_tg<P, RO, EXACT, NORMS><<<(unsigned)gx, nth, (size_t)smem, st>>>(Ls, Lt, v.g, rmax, tmax, s.partials, flag, excess);
   count_launches(1);
   const int64_t V = 2 * v.g.vh;
   k_wilson_rt_final<16><<<rmax * tmax, kThreads, 0, st>>>(s.partials, (int)gx, 1, tmax, 1.0 / (3.0 * (double)V),
@@ -1448,14 +1522,18 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
 
 template <int P>
 static cudaError_t launch_wilson_tg(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                                    const Scratch& s, double* flag, cudaStream_t st, bool* used) {
+                                    const Scratch& s, WilsonLinks links, double* flag, cudaStream_t st, bool* used) {
   *used = false;
-  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || !flag) return cudaSuccess;
+  if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || links == kWilsonAny) return cudaSuccess;
   auto launch = [&](auto rows) -> cudaError_t {
     constexpr int RO = decltype(rows)::value;
-    if (P != kF64 && v.g.n[3] == kTgChunks * RO)
-      return launch_wilson_tg_rows<P, RO, P != kF64>(v, spatial, rmax, tmax, s, flag, st, used);
-    return launch_wilson_tg_rows<P, RO, false>(v, spatial, rmax, tmax, s, flag, st, used);
+    if constexpr (P == kF64) {
+      if (links == kWilsonNear)
+        return launch_wilson_tg_rows<P, (RO + 1) / 2 * 2, false, true>(v, spatial, rmax, tmax, s, flag, st, used);
+    } else if (v.g.n[3] == kTgChunks * RO) {
+      return launch_wilson_tg_rows<P, RO, true, false>(v, spatial, rmax, tmax, s, flag, st, used);
+    }
+    return launch_wilson_tg_rows<P, RO, false, false>(v, spatial, rmax, tmax, s, flag, st, used);
   };
   switch ((v.g.n[3] + kTgChunks - 1) / kTgChunks) {
     case 1: return launch(std::integral_constant<int, 1>{});
@@ -1471,13 +1549,13 @@ static cudaError_t launch_wilson_tg(const LatticeView& v, const void* spatial, i
 }
 
 cudaError_t launch_wilson(const LatticeView& v, const void* spatial, int rmax, int tmax,
-                          const Scratch& s, double* flag, cudaStream_t st) {
+                          const Scratch& s, WilsonLinks links, double* flag, cudaStream_t st) {
   if (rmax < 1 || rmax > kWilsonMaxR || tmax < 1) return cudaErrorInvalidValue;
   {
     bool used = false;
     cudaError_t e = cudaSuccess;
     SU2_DISPATCH(v.prec, {
-      e = launch_wilson_tg<P>(v, spatial, rmax, tmax, s, flag, st, &used);
+      e = launch_wilson_tg<P>(v, spatial, rmax, tmax, s, links, flag, st, &used);
       if (e == cudaSuccess && !used) e = launch_wilson_rt<P>(v, spatial, rmax, tmax, s, st, &used);
     });
     if (e != cudaSuccess || used) return e;

@@ -4,6 +4,8 @@ temporal-gauge Wilson kernel on time extents of every remainder.  FP64 against
 the oracle at 1e-12 (values up to 6 and about a hundred operations of 2^-53
 each leave 1e-14; loops up to W = |U|^64 on scaled links are compared relative to
 their size)."""
+import time
+
 import numpy as np
 import pytest
 
@@ -166,6 +168,24 @@ def test_fp64_wilson_loops_on_links_off_unit_norm(nt, off, halves):
     ref = oracle.wilson_loops(list(dims), U, 4, 12)
     for _ in range(2):
         np.testing.assert_allclose(lat.wilson_loops(4, 12), ref, atol=1e-14, rtol=0)
+
+
+def _seconds(call, n=10):
+    times = []
+    for _ in range(n):
+        t0 = time.perf_counter()
+        call()
+        times.append(time.perf_counter() - t0)
+    return min(times)
+
+
+def test_fp64_wilson_loops_of_a_store_rounded_to_fp32_stay_in_temporal_gauge():
+    # 2.5 times a chain's links' time; 17 times where the loops are multiplied out
+    dims = (16, 16, 16, 16)
+    lat = Lattice(dims, 2.4, seed=1, start="hot", prec="f64")
+    unit = _seconds(lambda: lat.wilson_loops(8, 8))
+    lat.set_links(as_stored(lat.get_links(), "f32"))
+    assert _seconds(lambda: lat.wilson_loops(8, 8)) < 6 * unit
 
 
 def test_batched_measurements_of_uneven_lattices():
