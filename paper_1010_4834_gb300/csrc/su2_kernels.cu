@@ -957,8 +957,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
   constexpr int NO = kTgChunks * RO;               // origin rows, at least Nt
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double acc64[16 * kTgT];              // block totals; slot (R-1) kTgT + T-1
-  __shared__ A wsum[16][kTgThreads / 32][kTgT];    // per R and warp
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
   const int nt = g.n[3];
   const int hts = g.n0h * g.st[3];
   for (int i = threadIdx.x; i < 16 * kTgT; i += blockDim.x) acc64[i] = 0.0;
@@ -988,6 +987,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     TgNorm* Nb = reinterpret_cast<TgNorm*>(Pb + nm);   // NORMS: Nb[r nm + a] = N(a, r), r < NO
     TgNorm* Nc = Nb + NO * nm;                   // norms of the scan chunks
     TgNorm* Np = Nc + kTgChunks * nm;            // Np[a] = N(a, Nt)
+    A* wsum = reinterpret_cast<A*>(NORMS ? (void*)(Np + nm) : (void*)(Pb + nm));   // per R, warp and T
     const int a = kTgCols * warp + lane % kTgCols;
     const bool active = a < nm;
     __syncthreads();  // the previous plane's readers are done
@@ -1158,16 +1158,15 @@ __global__ void __launch_bounds__(kTgThreads, 1)
         if (upper) lo += half;
       }
       acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-      if ((lane & 1) == 0) wsum[Rl - 1][warp][lo] = acc[0];
+      if ((lane & 1) == 0) wsum[((Rl - 1) * nw + warp) * kTgT + lo] = acc[0];
 #pragma unroll
       for (int k = 0; k < kTgT; ++k) acc[k] = A(0);
     }
     __syncthreads();
     // the plane's sums, warps in a fixed order
-    const int nw = (int)(blockDim.x >> 5);
     for (int s = threadIdx.x; s < rmax * kTgT; s += blockDim.x) {
       double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += M::value(wsum[s / kTgT][w][s % kTgT]);
+      for (int w = 0; w < nw; ++w) t += M::value(wsum[(s / kTgT * nw + w) * kTgT + s % kTgT]);
       acc64[s] += t;
     }
   }
@@ -1483,6 +1482,7 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   const int64_t smem = ((int64_t)nr * tg_stride<RO>(nmax + rmax - 1) + 4 + (int64_t)nr * tg_stride<RO>(nmax) + 4 +
                         (int64_t)kTgChunks * nmax + nmax) *
                        (int64_t)sizeof(E) +
+                       (int64_t)rmax * (nth / 32) * kTgT * (int64_t)sizeof(typename TgMath<P>::A) +
                        (NORMS ? (int64_t)(kTgChunks * RO + kTgChunks + 1) * nmax * (int64_t)sizeof(TgNorm) : 0);
   const int64_t dyn_max = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
   if (smem > dyn_max) return cudaSuccess;

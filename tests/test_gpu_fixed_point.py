@@ -188,6 +188,13 @@ def test_fp64_wilson_loops_of_a_store_rounded_to_fp32_stay_in_temporal_gauge():
     assert _seconds(lambda: lat.wilson_loops(8, 8)) < 6 * unit
 
 
+def test_fp64_wilson_loops_at_64_time_slices_fit_the_temporal_gauge_kernel():
+    # planes of 24 columns with lines to 16 fill shared memory; nine times the time
+    # where they do not fit
+    short, full = (Lattice((24, 16, 16, nt), 2.4, seed=1, start="hot", prec="f64") for nt in (56, 64))
+    assert _seconds(lambda: full.wilson_loops(16, 16)) < 3 * _seconds(lambda: short.wilson_loops(16, 16))
+
+
 def test_batched_measurements_of_uneven_lattices():
     dims = [(4, 4, 4, 4), (16, 8, 12, 6), (2, 2, 2, 2), (6, 10, 4, 14), (8, 8, 8, 8)]
     for prec in ("f64", "f32", "f16q"):
