@@ -818,7 +818,7 @@ constexpr int kTgThreads = 512;          // planes of up to 64 columns
 // within 1.1e-6 = 2^-19.8): the kernel drops the time links' norms, which up to
 // there changes a loop by less than 1e-6.
 __device__ __forceinline__ Quat<float> qunit(const Quat<float>& q, bool& bad) {
-  const float e = fmaf(-q.w, q.w, fmaf(-q.x, q.x, fmaf(-q.y, q.y, fmaf(-q.z, q.z, 1.0f))));
+  const float e = fmaf(-q.x, q.x, fmaf(-q.w, q.w, 1.0f)) - fmaf(q.z, q.z, q.y * q.y);
   bad |= !(fabsf(e) <= 0x1p-18f);
   const float d = 0.5f * e;
   return qmake<float>(fmaf(q.w, d, q.w), fmaf(q.x, d, q.x), fmaf(q.y, d, q.y), fmaf(q.z, d, q.z));
@@ -907,6 +907,23 @@ __device__ __forceinline__ TgNorm tg_take_norm(FixQuat& q) {
   return n;
 }
 
+// The value of the lane n below.
+__device__ __forceinline__ float tg_lane_up(float v, int n) { return __shfl_up_sync(0xffffffffu, v, n); }
+__device__ __forceinline__ Fix tg_lane_up(const Fix& v, int n) {
+  return Fix{__shfl_up_sync(0xffffffffu, v.h, n), __shfl_up_sync(0xffffffffu, v.l, n)};
+}
+__device__ __forceinline__ TgNorm tg_lane_up(const TgNorm& v, int n) {
+  return TgNorm{__shfl_up_sync(0xffffffffu, v.d, n), __shfl_up_sync(0xffffffffu, v.i, n)};
+}
+template <class Q> __device__ __forceinline__ Q tg_lane_up(const Q& q, int n) {
+  Q r;
+  r.w = tg_lane_up(q.w, n);
+  r.x = tg_lane_up(q.x, n);
+  r.y = tg_lane_up(q.y, n);
+  r.z = tg_lane_up(q.z, n);
+  return r;
+}
+
 // Site (column a, slice 0) of the plane (mu, c1, c2).
 __device__ __forceinline__ Site plane_site(const Geom& g, int mu, int a, int c1, int c2) {
   Site y;
@@ -937,8 +954,10 @@ template <int RO> __device__ __forceinline__ int tg_row(int r, int stride) {
   return r * stride + (r < kTgChunks * RO ? tg_skew_unit<RO>() * ((r / RO) & 1) : 0);
 }
 
-// EXACT: Nt is a multiple of eight (every origin row starts loops), compiled
-// without the tests.
+// EXACT: Nt = 8 RO (every origin row starts loops), a constant to the compiler: with
+// Nt read at run time the rows' slices took integer divisions in phases 1 and 3
+// (48^3x8 FP32, W(1,4): 235 us, so 216; with the prefix over the chunks by
+// shuffles instead of through shared memory 186).
 // NORMS (FP64): links up to 2^-16 off unit norm (in |U|^2; a configuration stored
 // in FP32, say).  A loop carries the product of its time links' norms, N(a, r + T)
 // N(a + R, r + T) / (N(a, r) N(a + R, r)) with N(a, r) the norms' product along
@@ -958,7 +977,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double acc64[16 * kTgT];              // block totals; slot (R-1) kTgT + T-1
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  const int nt = g.n[3];
+  const int nt = EXACT ? NO : g.n[3];
   const int hts = g.n0h * g.st[3];
   for (int i = threadIdx.x; i < 16 * kTgT; i += blockDim.x) acc64[i] = 0.0;
   const int ntr0 = g.n[1] * g.n[2], ntr1 = g.n[0] * g.n[2], ntr2 = g.n[0] * g.n[1];
@@ -967,10 +986,13 @@ __global__ void __launch_bounds__(kTgThreads, 1)
   bool bad = false;
   int64_t over = 0;
   // slice of row r: rows past the last slice repeat the first ones
-  auto slice = [&](int r) {
-    if constexpr (EXACT) return r < nt ? r : (r - NO) % nt;
-    while (r >= nt) r -= nt;
-    return r;
+  auto slice = [&](int r) -> int {
+    if constexpr (EXACT) {
+      return r < NO ? r : (r - NO) % NO;
+    } else {
+      while (r >= nt) r -= nt;
+      return r;
+    }
   };
   for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
     const int mu = u < ntr0 ? 0 : (u < ntr0 + ntr1 ? 1 : 2);
@@ -982,11 +1004,9 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     const int SU = tg_stride<RO>(W), SS = tg_stride<RO>(nm);
     E* Ue = reinterpret_cast<E*>(smem_raw);      // Ue[tg_row(r, SU) + cc] = U'(cc, r), r < NO + kTgT
     E* Sb = Ue + (NO + kTgT) * SU + 4;           // Sb[tg_row(r, SS) + a]: G(a, r), then S'_R(a, r)
-    E* Ct = Sb + (NO + kTgT) * SS + 4;           // Ct[k nm + a]: product of scan chunk k
-    E* Pb = Ct + kTgChunks * nm;                 // Pb[a] = P(a)
+    E* Pb = Sb + (NO + kTgT) * SS + 4;           // Pb[a] = P(a)
     TgNorm* Nb = reinterpret_cast<TgNorm*>(Pb + nm);   // NORMS: Nb[r nm + a] = N(a, r), r < NO
-    TgNorm* Nc = Nb + NO * nm;                   // norms of the scan chunks
-    TgNorm* Np = Nc + kTgChunks * nm;            // Np[a] = N(a, Nt)
+    TgNorm* Np = Nb + NO * nm;                   // Np[a] = N(a, Nt)
     A* wsum = reinterpret_cast<A*>(NORMS ? (void*)(Np + nm) : (void*)(Pb + nm));   // per R, warp and T
     const int a = kTgCols * warp + lane % kTgCols;
     const bool active = a < nm;
@@ -994,7 +1014,8 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     // (1) this lane's links, loaded together: the time and spatial links of
     // its origin rows and the spatial links that its extended rows repeat;
     // then the time links' products within the chunk
-    E us[RO + kTgExt];
+    E us[RO + kTgExt], Q = M::one();
+    TgNorm n{0, 0};
     if (active) {
       E ut[RO];
       const Site y = plane_site(g, mu, a, c1, c2);
@@ -1012,40 +1033,42 @@ __global__ void __launch_bounds__(kTgThreads, 1)
         us[RO + e] = M::template load<NORMS>(Ls, 2 * mu + par, h, bad);
       }
       if constexpr (NORMS) {
-        TgNorm n{0, 0};
 #pragma unroll
         for (int i = 0; i < RO; ++i) {
           Nb[(r0 + i) * nm + a] = n;
           n = tg_times(n, tg_take_norm(ut[i]));
         }
-        Nc[c * nm + a] = n;
       }
-      E L = M::one();
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
-        Sb[tg_row<RO>(r0 + i, SS) + a] = L;
-        L = M::unit(M::mul(L, ut[i]), bad);
+        Sb[tg_row<RO>(r0 + i, SS) + a] = Q;
+        Q = M::unit(M::mul(Q, ut[i]), bad);
       }
-      Ct[c * nm + a] = L;
     }
-    __syncthreads();
-    // (2) prefix over the chunks: G(a, r) for the thread's rows, P(a) = G(a, Nt)
-    if (active) {
-      E Q = M::one();
-      for (int k = 0; k < c; ++k) Q = M::unit(M::mul(Q, Ct[k * nm + a]), bad);
-      if (c > 0) {
+    // (2) prefix over a column's chunks, the warp's lanes: G(a, r) for the
+    // thread's rows, P(a) = G(a, Nt).  Products of up to eight unit quaternions,
+    // normalised with G.
 #pragma unroll
-        for (int i = 0; i < RO; ++i) {
-          E* p = Sb + tg_row<RO>(r0 + i, SS) + a;
-          *p = M::unit(M::mul(Q, *p), bad);
-        }
-      }
-      if (c == kTgChunks - 1) Pb[a] = M::unit(M::mul(Q, Ct[c * nm + a]), bad);
+    for (int d = 1; d < kTgChunks; d *= 2) {
+      const E before = tg_lane_up(Q, d * kTgCols);
+      if (c >= d) Q = M::mul(before, Q);
       if constexpr (NORMS) {
-        TgNorm n{0, 0};
-        for (int k = 0; k < c; ++k) n = tg_times(n, Nc[k * nm + a]);
-        for (int i = 0; i < RO; ++i) Nb[(r0 + i) * nm + a] = tg_times(n, Nb[(r0 + i) * nm + a]);
-        if (c == kTgChunks - 1) Np[a] = tg_times(n, Nc[c * nm + a]);
+        const TgNorm m = tg_lane_up(n, d * kTgCols);
+        if (c >= d) n = tg_times(m, n);
+      }
+    }
+    if (active && c == kTgChunks - 1) {
+      Pb[a] = M::unit(Q, bad);
+      if constexpr (NORMS) Np[a] = n;
+    }
+    Q = tg_lane_up(Q, kTgCols);
+    if constexpr (NORMS) n = tg_lane_up(n, kTgCols);
+    if (active && c > 0) {
+#pragma unroll
+      for (int i = 0; i < RO; ++i) {
+        E* p = Sb + tg_row<RO>(r0 + i, SS) + a;
+        *p = M::unit(M::mul(Q, *p), bad);
+        if constexpr (NORMS) Nb[(r0 + i) * nm + a] = tg_times(n, Nb[(r0 + i) * nm + a]);
       }
     }
     __syncthreads();
@@ -1061,7 +1084,8 @@ __global__ void __launch_bounds__(kTgThreads, 1)
         E v = M::mul_nd(M::mul(Sb[gt + a], us[i]), Sb[gt + an]);
         if (EXACT ? i >= RO : r >= nt) v = M::mul_nd(M::mul(Pb[a], v), Pb[an]);
         const int ru = tg_row<RO>(r, SU);
-        for (int cc = a; cc < W; cc += nm) Ue[ru + cc] = v;
+        Ue[ru + a] = v;
+        if (a < rmax - 1) Ue[ru + a + nm] = v;
       }
     }
     __syncthreads();  // Sb now holds lines
@@ -1480,10 +1504,10 @@ static cudaError_t launch_wilson_tg_rows(const LatticeView& v, const void* spati
   cudaError_t e = cudaFuncGetAttributes(&fa, k_wilson_tg<P, RO, EXACT, NORMS>);
   if (e != cudaSuccess) return e;
   const int64_t smem = ((int64_t)nr * tg_stride<RO>(nmax + rmax - 1) + 4 + (int64_t)nr * tg_stride<RO>(nmax) + 4 +
-                        (int64_t)kTgChunks * nmax + nmax) *
+                        (int64_t)nmax) *
                        (int64_t)sizeof(E) +
                        (int64_t)rmax * (nth / 32) * kTgT * (int64_t)sizeof(typename TgMath<P>::A) +
-                       (NORMS ? (int64_t)(kTgChunks * RO + kTgChunks + 1) * nmax * (int64_t)sizeof(TgNorm) : 0);
+                       (NORMS ? (int64_t)(kTgChunks * RO + 1) * nmax * (int64_t)sizeof(TgNorm) : 0);
   const int64_t dyn_max = (int64_t)optin - (int64_t)fa.sharedSizeBytes;
   if (smem > dyn_max) return cudaSuccess;
   // raised once per device, as for the time-outer kernel
