@@ -1484,6 +1484,23 @@ static cudaError_t launch_wilson_rt(const LatticeView& v, const void* spatial, i
   return cudaErrorInvalidValue;
 }
 
+// Whether the time-outer kernel is the faster one below FP64: wide planes, whose
+// temporal-gauge block is alone on its SM and waits at its barriers, with so few
+// loops that the transform is not made good.  It counts more with few time slices
+// and where Nt does not fill the eight row chunks; from R = 5 on the time-outer
+// kernel's chunk of eight is well used.  FP32, temporal gauge against time-outer, us:
+// 64^3x2 W(16,2) 1150 and 635, W(1,1) 403 and 303; 48^3x10 W(4,1) 297 and 224,
+// W(8,8) 511 and 569; 48^3x48 W(16,1) 1155 and 998, W(4,1) 497 and 671.  Up to 32
+// columns temporal gauge is faster but for the longest lines at T = 1 (24^3x20
+// W(16,1) 1.07 times the other's); at 48^3x12 W(1,1) takes 267 against 313.
+static bool time_outer_is_faster(int nmax, int nt, int rmax, int tmax) {
+  if (nmax <= 32) return false;
+  const bool ragged = nt % kTgChunks != 0;
+  if (nt < 16) return tmax <= (rmax >= 5 ? 4 : rmax >= 3 ? 2 : ragged && nt <= 10);
+  if (nt < 32) return tmax <= (rmax >= 5 ? 2 : rmax >= 3 && ragged);
+  return tmax <= (rmax >= 5);
+}
+
 // The temporal-gauge kernel when R and T are at most 16, Nt is at most 64, one
 // block holds four columns a warp of the widest plane, and the staged plane
 // fits in shared memory; *used = false otherwise.
@@ -1549,6 +1566,8 @@ static cudaError_t launch_wilson_tg(const LatticeView& v, const void* spatial, i
                                     const Scratch& s, WilsonLinks links, double* flag, cudaStream_t st, bool* used) {
   *used = false;
   if (!SU2_WILSON_TG || rmax > 16 || tmax > kTgT || links == kWilsonAny) return cudaSuccess;
+  if (P != kF64 && time_outer_is_faster(std::max(v.g.n[0], std::max(v.g.n[1], v.g.n[2])), v.g.n[3], rmax, tmax))
+    return cudaSuccess;
   auto launch = [&](auto rows) -> cudaError_t {
     constexpr int RO = decltype(rows)::value;
     if constexpr (P == kF64) {

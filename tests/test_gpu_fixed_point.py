@@ -130,6 +130,20 @@ def test_wilson_loops_on_every_remainder_of_the_time_extent(nt, prec):
         np.testing.assert_allclose(lat.wilson_loops(rmax, tmax), ref[:rmax, :tmax], atol=MTOL[prec] * 5, rtol=0)
 
 
+@pytest.mark.parametrize("prec", ["f32", "f16q"])
+@pytest.mark.parametrize("nt", [4, 8, 10, 20, 24, 40])
+def test_wilson_loops_on_both_sides_of_the_time_outer_kernels_range(nt, prec):
+    # planes just wider than 32 columns: the kernel changes with R and T
+    dims = (34, 6, 6, nt)
+    U = inputs.random_field(dims, 32)
+    ref = oracle.wilson_loops(list(dims), as_stored(U, prec), 6, min(nt, 6))
+    lat = Lattice(dims, 2.0, prec=prec)
+    lat.set_links(U)
+    for rmax in (1, 2, 3, 4, 5, 6):
+        for tmax in range(1, min(nt, 6) + 1):
+            np.testing.assert_allclose(lat.wilson_loops(rmax, tmax), ref[:rmax, :tmax], atol=MTOL[prec] * 5, rtol=0)
+
+
 def _off_unit(nt, off, halves, dims=(6, 4, 6)):
     """Ordered links (large loops) whose norms differ by up to off from one, link
     by link or in the two halves of the lattice: a loop carries its own links'
