@@ -45,7 +45,7 @@ namespace su2 {
 // 48^4 (17 k per SM) 256 is faster (70.9 against 72.2 us; 16^4 12.3
 // against 14.0), as more, smaller blocks spread the few block iterations
 // evenly over the SMs.  The switch is at SU2_HB_BIG_PER_SM half-lattice
-// sites per SM.  FP64, 80 registers a thread: 256 throughout.
+// sites per SM.  FP64, 128 registers a thread: 256 throughout.
 #ifndef SU2_HB_BIG_PER_SM
 #define SU2_HB_BIG_PER_SM 32768
 #endif

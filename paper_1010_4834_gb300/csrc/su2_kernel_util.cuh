@@ -183,7 +183,10 @@ __device__ __forceinline__ void plaquette_from_block_sums(const double* meas, in
 #define SU2_HB_MINB 4
 #endif
 template <int P> struct Occ { static constexpr int hb = SU2_HB_MINB; };
-template <> struct Occ<kF64> { static constexpr int hb = 3; };
+// FP64: two blocks of 256 at 128 registers a thread; three at 80 spilled (24^3x8
+// sweep 179 -> 174 us, measured 24^3x32 sweep 472 -> 464, over-relaxation sweep
+// 347 -> 330).
+template <> struct Occ<kF64> { static constexpr int hb = 2; };
 
 template <int P, int CP = kFlat> static Links<P, CP> links_of(void* base, int64_t vh) {
   Links<P, CP> L;
