@@ -82,6 +82,10 @@ __device__ __forceinline__ bool group_barrier(GroupBarrier* gb, unsigned int n, 
 // The deferral queue holds two entries a thread.
 template <int BS> struct BatchQueue { static constexpr int value = 2 * BS; };
 
+// A lattice's geometry: FP64 in place, since its out-of-line paths take the address
+// (of a copy, that would be one in local memory).
+template <int P> using BatchGeom = std::conditional_t<P == kF64, const Geom&, const Geom>;
+
 // One substep (MU, p) of one lattice by the CTAs of a group, each link by
 // hb_link with coherent loads (other CTAs of the group wrote the links
 // before the last barrier): trial 1 inline, rejected links queued and
@@ -231,7 +235,7 @@ __global__ void __launch_bounds__(BatchBlock<BS, MEAS>::value, (P == kF64 ? 512 
   const uint32_t sweep0 = *sweep_base;
   // one substep (mu, p) of lattice l by this group's CTAs
   auto substep = [&](int l, uint32_t sweep, int mu, int p) {
-    const Geom g = desc[l].g;
+    BatchGeom<P> g = desc[l].g;
     Links<P, hb_addr<P, kClassOff>> L;
     L.set(desc[l].links, g.vh);
     const R beta = (R)desc[l].beta;
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(BatchBlock<BS, MEAS>::value, (P == kF64 ? 512 
   // 35.5 G updates/s for the 64-lattice batch at 32 groups)
   // `nor` over-relaxation sweeps precede each heat-bath sweep
   auto or_substep = [&](int l, int mu, int p) {
-    const Geom g = desc[l].g;
+    BatchGeom<P> g = desc[l].g;
     Links<P, hb_addr<P, kClassOff>> L;
     L.set(desc[l].links, g.vh);
     if constexpr (P == kF64) {

@@ -339,10 +339,12 @@ template <class R> __device__ __forceinline__ Quat<R> haar_from(uint4 r) {
 }
 
 // FP64 links and sums in fixed point and back.
+template <bool ANY = false>
 __device__ __forceinline__ FixQuat fix_of(const Quat<double>& q, int conj, FixBad& bad) {
-  return fix_link((uint32_t)__double2loint(q.w), (uint32_t)__double2hiint(q.w), (uint32_t)__double2loint(q.x),
-                        (uint32_t)__double2hiint(q.x), (uint32_t)__double2loint(q.y), (uint32_t)__double2hiint(q.y),
-                        (uint32_t)__double2loint(q.z), (uint32_t)__double2hiint(q.z), conj, bad);
+  const uint32_t w0 = (uint32_t)__double2loint(q.w), w1 = (uint32_t)__double2hiint(q.w), x0 = (uint32_t)__double2loint(q.x),
+                 x1 = (uint32_t)__double2hiint(q.x), y0 = (uint32_t)__double2loint(q.y), y1 = (uint32_t)__double2hiint(q.y),
+                 z0 = (uint32_t)__double2loint(q.z), z1 = (uint32_t)__double2hiint(q.z);
+  return ANY ? fix_any_link(w0, w1, x0, x1, y0, y1, z0, z1, conj, bad) : fix_link(w0, w1, x0, x1, y0, y1, z0, z1, conj, bad);
 }
 
 __device__ __forceinline__ Quat<double> fix_sum_to_double(const FixSum& s) {
@@ -1061,7 +1063,7 @@ __device__ __forceinline__ TermLinks term_links(const Links<kF64, CP>& L, const 
 __device__ __forceinline__ int half_step_mu(const Geom& g, const Site& x, int mu) { return half_step_rt(g, x, mu, true); }
 
 // The staple sum over nu < nd in FP64 and its partial sum over nu < mu: the
-// path of links outside fix_link's range.
+// path of links that are no near-unit quaternions.
 template <bool NC, bool MCG, int CP>
 __device__ __forceinline__ Quat<double> staple_rolled(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h,
                                                       int mu, int p, int nd, Quat<double>& lower) {
@@ -1079,9 +1081,9 @@ __device__ __forceinline__ Quat<double> staple_rolled(const Links<kF64, CP>& L, 
 }
 
 // The same in fixed point, with LOWER also the partial sum.  False if a link is
-// outside fix_link's range; the caller then takes staple_rolled.  A term's
-// links are loaded while the previous term is multiplied.
-template <bool LOWER, bool NC, bool MCG, int CP>
+// outside fix_link's (ANY: fix_any_link's) range.  A term's links are loaded while
+// the previous term is multiplied.
+template <bool LOWER, bool NC, bool MCG, bool ANY = false, int CP>
 __device__ __forceinline__ bool staple_fixed(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h, int mu,
                                              int p, int nd, FixSum& s, Quat<double>& lower) {
   s = fix_zero();
@@ -1093,11 +1095,24 @@ __device__ __forceinline__ bool staple_fixed(const Links<kF64, CP>& L, const Geo
   for (int k = 0; k < 2 * (nd - 1); ++k) {
     const TermLinks next = term_links<NC, MCG>(L, g, x, h, dmu, mu, p, k + 1 < 2 * (nd - 1) ? k + 1 : k);
     const int odd = -(k & 1);
-    fix_mac(s, fix_mul(fix_of(t.a, odd, bad), fix_of(t.b, 0, bad)), fix_of(t.c, ~odd, bad));
+    fix_mac(s, fix_mul(fix_of<ANY>(t.a, odd, bad), fix_of<ANY>(t.b, 0, bad)), fix_of<ANY>(t.c, ~odd, bad));
     if (LOWER && k + 1 == 2 * mu) lower = fix_sum_to_double(s);
+    if (ANY && !fix_ok(bad)) return false;
     t = next;
   }
   return fix_ok(bad);
+}
+
+// The path of links that staple_fixed refuses, out of line (kernels pass the geometry
+// by reference to a __grid_constant__ parameter or to global memory).
+struct OtherFrame { Frame<double> f; Quat<double> lower; };
+template <bool NC, bool MCG, int CP>
+static __device__ __noinline__ OtherFrame frame_other(Links<kF64, CP> L, const Geom& g, Site x, int h, int mu, int p, double beta) {
+  OtherFrame r;
+  FixSum s;
+  if (staple_fixed<true, NC, MCG, true>(L, g, x, h, mu, p, 4, s, r.lower)) r.f = staple_frame(s, beta);
+  else r.f = staple_frame(staple_rolled<NC, MCG>(L, g, x, h, mu, p, 4, r.lower), beta);
+  return r;
 }
 
 // W, alpha of link (x, mu) and, with MEAS, the staple's partial sum over nu <
@@ -1109,7 +1124,9 @@ __device__ __forceinline__ Frame<typename Real<P>::T> link_frame(const Links<P, 
   if constexpr (P == kF64) {
     FixSum s;
     if (__builtin_expect(staple_fixed<MEAS, NC, MCG>(L, g, x, h, mu, p, 4, s, lower), 1)) return staple_frame(s, beta);
-    return staple_frame(staple_rolled<NC, MCG>(L, g, x, h, mu, p, 4, lower), beta);
+    const OtherFrame r = frame_other<NC, MCG>(L, g, x, h, mu, p, beta);
+    lower = r.lower;
+    return r.f;
   } else if constexpr (MEAS) {
     return staple_frame(staple_split<P, MU, NC, CP, MCG>(L, g, x, h, p, lower), beta);
   } else {

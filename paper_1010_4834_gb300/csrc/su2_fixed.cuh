@@ -14,10 +14,11 @@
 // roundings of 2^-53 and more per addition) comes out within about 2^-54 in
 // the worst case and 2^-56 typically, several times closer than in FP64.
 //
-// What a link must be for this: components 0 or |v| in [2^-31, 2) and a norm
-// within 6% of one.  fix_link raises `bad` otherwise (values other than unit
-// quaternions, which a store set from outside may hold, zeros, NaN), and the
-// caller computes that thread's result in FP64, as for every link before.
+// What a link must be for this: components |v| in [2^-31, 2) and a norm within 6%
+// of one.  fix_link raises `bad` otherwise, and the thread starts again with
+// fix_any_link, which takes any |v| < 2 (zeros: cold starts, Abelian fields) and
+// costs twice the shifts; values other than near-unit quaternions, which a store
+// set from outside may hold, are computed in FP64.
 //
 // Sums.  With norms n <= 1.0607: |sum h h'| <= 2^58 n^2 per component of a
 // product (Cauchy-Schwarz); |sum (h l' + l h')| <= 2^29 (sum |h| + sum |h'|)
@@ -77,13 +78,7 @@ SU2_HD Fix fix_from(uint32_t lo, uint32_t hi, int neg, uint32_t& bad) {
 struct FixBad { uint32_t e, n; };
 SU2_HD bool fix_ok(const FixBad& b) { return (b.e & kFixBadExp) == 0u && (b.n >> 24) == 0u; }
 
-SU2_HD FixQuat fix_link(uint32_t w0, uint32_t w1, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1, uint32_t z0,
-                        uint32_t z1, int conj, FixBad& bad) {
-  FixQuat q;
-  q.w = fix_from(w0, w1, 0, bad.e);
-  q.x = fix_from(x0, x1, conj, bad.e);
-  q.y = fix_from(y0, y1, conj, bad.e);
-  q.z = fix_from(z0, z1, conj, bad.e);
+SU2_HD void fix_check_norm(const FixQuat& q, FixBad& bad) {
   // squared norm in units of 2^-58, less 1 - 1/8: in [0, 1/4) for norm^2
   // within 1 +- 1/8; components below 2 keep the sum below 2^62
   int64_t n = -((int64_t)7 << 55);
@@ -92,6 +87,16 @@ SU2_HD FixQuat fix_link(uint32_t w0, uint32_t w1, uint32_t x0, uint32_t x1, uint
   n += (int64_t)q.y.h * q.y.h;
   n += (int64_t)q.z.h * q.z.h;
   bad.n |= (uint32_t)((uint64_t)n >> 32);
+}
+
+SU2_HD FixQuat fix_link(uint32_t w0, uint32_t w1, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1, uint32_t z0,
+                        uint32_t z1, int conj, FixBad& bad) {
+  FixQuat q;
+  q.w = fix_from(w0, w1, 0, bad.e);
+  q.x = fix_from(x0, x1, conj, bad.e);
+  q.y = fix_from(y0, y1, conj, bad.e);
+  q.z = fix_from(z0, z1, conj, bad.e);
+  fix_check_norm(q, bad);
   return q;
 }
 
@@ -195,6 +200,17 @@ SU2_HD Fix fix_from_any(uint32_t lo, uint32_t hi) {
   const int64_t v = (int64_t)fix_shr(m, 1023u - ((hi >> 20) & 0x7FFu));
   const int64_t s = (int64_t)((int32_t)hi >> 31);
   return fix_split((v ^ s) - s);
+}
+
+// fix_link for components of any size, zero too: the path of links that it
+// refuses for them (cold starts, Abelian fields).
+SU2_HD FixQuat fix_any_link(uint32_t w0, uint32_t w1, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1, uint32_t z0,
+                            uint32_t z1, int conj, FixBad& bad) {
+  FixQuat q{fix_from_any(w0, w1), fix_from_any(x0, x1), fix_from_any(y0, y1), fix_from_any(z0, z1)};
+  if (conj) q.x = fix_neg(q.x), q.y = fix_neg(q.y), q.z = fix_neg(q.z);
+  if ((w1 | x1 | y1 | z1) & 0x40000000u) bad.e |= kFixBadExp;   // a component of 2 or more, NaN
+  fix_check_norm(q, bad);
+  return q;
 }
 
 // The positive double 1.m 2^e with the given words, e < 11, in units of 2^-62

@@ -156,14 +156,45 @@ __device__ __forceinline__ void hb_drain(const Links<P, CP>& L, Substep sub, con
   }
 }
 
+// FP64 in fixed point; false if a link is outside fix_link's (ANY: fix_any_link's)
+// range.
+template <bool NC, bool ANY, int CP>
+__device__ __forceinline__ bool or_fixed(const Links<kF64, CP>& L, const Geom& g, const Site& x, int h, int mu, int p,
+                                         const Quat<double>& u) {
+  FixSum s;
+  Quat<double> lower;
+  FixBad bad{0u, 0u};
+  const bool ok = staple_fixed<false, NC, false, ANY>(L, g, x, h, mu, p, 4, s, lower);
+  const FixQuat ud = fix_of<ANY>(u, -1, bad);
+  if (!ok || !fix_ok(bad)) return false;
+  const Frame<double> f = staple_frame(s, 1.0);
+  if (f.alpha == 0.0) return true;
+  s = fix_zero();
+  fix_mac(s, fix_mul(f.w, ud), f.w);
+  L.st(2 * mu + p, h, fix_sum_to_double(s));
+  return true;
+}
+// The links that it refuses, out of line.
+template <bool NC, int CP>
+static __device__ __noinline__ void or_other(Links<kF64, CP> L, const Geom& g, Site x, int h, int mu, int p) {
+  const Quat<double> u = ldl<kF64, NC>(L, 2 * mu + p, h);
+  if (or_fixed<NC, true>(L, g, x, h, mu, p, u)) return;
+  Quat<double> lower;
+  const Quat<double> sig = staple_rolled<NC, false>(L, g, x, h, mu, p, 4, lower);
+  const double k2 = qdot(sig, sig);
+  if (!(k2 >= Math<double>::kTiny)) return;
+  const Quat<double> w = qscale(sig, Math<double>::rsqrt(k2));
+  L.st(2 * mu + p, h, qmul(qmul_nd(w, u), w));
+}
+
 // One over-relaxation update (Section 2, Eq. 10 with W = Sigma/|Sigma| for
 // the orientation of Eq. 11): U' = W U^dagger W keeps Tr(U Sigma^dagger).
 // Unlike a heat-bath link, U' is built from the old link, so rounding would
 // accumulate over many over-relaxation sweeps: in FP32 each step multiplies
 // |U| by |W|^2 = 1 + O(2^-22), a random walk of about 1e-5 after a thousand
 // sweeps.  FP32 (and the F16Q arithmetic, whose stores are normalised again
-// on load) therefore normalises U' before storing it; in FP64 the walk stays
-// near 1e-15 and the update is stored as computed, like the oracle's.  NC:
+// on load) therefore normalises U' before storing it; in FP64 the walk (2e-15
+// rms in |U|^2 after a hundred sweeps, 9e-15 after a thousand) is let be and the update is stored as computed, like the oracle's.  NC:
 // read-only loads (no other block of the launch writes these links).
 template <int P, int MU, int PAR, bool NC, int CP>
 __device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Substep sub, int h) {
@@ -172,32 +203,19 @@ __device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Su
   using R = typename Real<P>::T;
   using M = Math<R>;
   const Site x = site_from_half(g, (uint32_t)h, p);
-  Quat<R> sig, u;
   if constexpr (P == kF64) {
-    u = ldl<P, NC>(L, 2 * mu + p, h);
-    FixSum s;
-    FixBad bad{0u, 0u};
-    const bool ok = staple_fixed<false, NC, false>(L, g, x, h, mu, p, 4, s, sig);
-    const FixQuat ud = fix_of(u, -1, bad);
-    if (__builtin_expect(ok && fix_ok(bad), 1)) {
-      const Frame<R> f = staple_frame(s, 1.0);
-      if (f.alpha == 0.0) return;
-      s = fix_zero();
-      fix_mac(s, fix_mul(f.w, ud), f.w);
-      L.st(2 * mu + p, h, fix_sum_to_double(s));
-      return;
-    }
-    sig = staple_rolled<NC, false>(L, g, x, h, mu, p, 4, sig);
+    const Quat<R> u = ldl<P, NC>(L, 2 * mu + p, h);
+    if (__builtin_expect(!or_fixed<NC, false>(L, g, x, h, mu, p, u), 0)) or_other<NC>(L, g, x, h, mu, p);
   } else {
-    sig = staple<P, MU, 0xF, NC>(L, g, x, h, p);
+    const Quat<R> sig = staple<P, MU, 0xF, NC>(L, g, x, h, p);
+    const R k2 = qdot_rn(sig, sig);
+    if (!(k2 >= M::kTiny)) return;
+    const Quat<R> w = qscale(sig, M::rsqrt(k2));
+    const Quat<R> u = ldl<P, NC>(L, 2 * mu + p, h);   // the staple's registers are free
+    Quat<R> v = qmul_rn(qmul_nd_rn(w, u), w);
+    v = qscale(v, M::rsqrt(qdot_rn(v, v)));
+    L.st(2 * mu + p, h, v);
   }
-  const R k2 = qdot_rn(sig, sig);
-  if (!(k2 >= M::kTiny)) return;
-  const Quat<R> w = qscale(sig, M::rsqrt(k2));
-  if constexpr (P != kF64) u = ldl<P, NC>(L, 2 * mu + p, h);   // the staple's registers are free
-  Quat<R> v = qmul_rn(qmul_nd_rn(w, u), w);
-  if constexpr (P != kF64) v = qscale(v, M::rsqrt(qdot_rn(v, v)));
-  L.st(2 * mu + p, h, v);
 }
 
 }  // namespace su2

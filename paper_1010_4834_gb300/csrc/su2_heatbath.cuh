@@ -78,7 +78,7 @@ template <int P, int BS> struct HbMinBlocks {
 
 template <int P, int MU, bool MEAS, int PAR, int BS>
 __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
-    k_heatbath(Links<P, hb_addr<P, kClassPtr>> L, Geom g, Substep sub, const uint32_t* sweep_base, uint32_t sweep_off,
+    k_heatbath(Links<P, hb_addr<P, kClassPtr>> L, const __grid_constant__ Geom g, Substep sub, const uint32_t* sweep_base, uint32_t sweep_off,
                const __grid_constant__ HBParams hp, unsigned long long* stats, double* meas) {
   const int mu = substep_of<MU, PAR>(sub).mu;
   using R = typename Real<P>::T;
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
 // 25.9 against 25.4, 8^4 18.1 against 17.1).
 template <int P, int MU, bool MEAS, int PAR, int BS>
 __global__ void __launch_bounds__(BS, 2 * SmallPerSM<P>::value / BS)
-    k_heatbath_small(Links<P, hb_addr<P, kClassPtr>> L, Geom g, Substep sub, const uint32_t* sweep_base,
+    k_heatbath_small(Links<P, hb_addr<P, kClassPtr>> L, const __grid_constant__ Geom g, Substep sub, const uint32_t* sweep_base,
                      uint32_t sweep_off, int late, const __grid_constant__ HBParams hp, double* meas) {
   sub = substep_of<MU, PAR>(sub);
   const int mu = sub.mu, p = sub.p;
@@ -308,7 +308,7 @@ template <int LANES> __device__ __forceinline__ void lanes_add(FixSum& s) {
 
 template <bool MEAS, int LANES>
 __global__ void __launch_bounds__(64, 8)
-    k_heatbath_lanes(Links<kF64> L, Geom g, Substep sub, const uint32_t* sweep_base, uint32_t sweep_off, int late,
+    k_heatbath_lanes(Links<kF64> L, const __grid_constant__ Geom g, Substep sub, const uint32_t* sweep_base, uint32_t sweep_off, int late,
                      const __grid_constant__ HBParams hp, double* meas) {
   const int mu = sub.mu, p = sub.p;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -350,8 +350,13 @@ __global__ void __launch_bounds__(64, 8)
   }
   const uint32_t off = __ballot_sync(0xffffffffu, !fix_ok(bad));
   Frame<double> f;
-  if (__builtin_expect((off >> group & ((1u << LANES) - 1u)) == 0u, 1)) f = staple_frame(s, hp.beta);
-  else f = staple_frame(staple_rolled<false, false>(L, g, x, h, mu, p, 4, lower), hp.beta);
+  if (__builtin_expect((off >> group & ((1u << LANES) - 1u)) == 0u, 1)) {
+    f = staple_frame(s, hp.beta);
+  } else {
+    const OtherFrame r = frame_other<false, false>(L, g, x, h, mu, p, hp.beta);
+    f = r.f;
+    lower = r.lower;
+  }
   Quat<double> nl = qone<double>();
   bool found = false, open = valid;
   if (!(f.alpha >= 1e-12)) {

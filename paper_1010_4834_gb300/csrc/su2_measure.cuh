@@ -64,6 +64,32 @@ __device__ __forceinline__ int64_t plaq_fixed(const Links<kF64>& L, int q, const
   return fix_dot(a, b, 0);
 }
 
+// The sums (spatial, space-time planes) of a site with links that plaq_fixed
+// refuses, out of line, a rolled loop over the planes: in fixed point with any
+// components, then in FP64.
+static __device__ __noinline__ double2 plaq_other(Links<kF64> L, int p, int h, int h0, int h1, int h2, int h3) {
+  const int q = p ^ 1;
+  double sum[2];
+  FixBad bad{0u, 0u};
+  for (int fp64 = 0; fp64 < 2; ++fp64) {
+    sum[0] = sum[1] = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < 6; ++k) {
+      const int nu = k < 1 ? 1 : k < 3 ? 2 : 3, mu = nu == 1 ? 0 : nu == 2 ? k - 1 : k - 3;
+      const int hm = mu == 0 ? h0 : mu == 1 ? h1 : h2, hn = nu == 1 ? h1 : nu == 2 ? h2 : h3;
+      const Quat<double> a = L.ld(2 * mu + p, h), b = L.ld(2 * nu + q, hm), c = L.ld(2 * nu + p, h), d = L.ld(2 * mu + q, hn);
+      const double v = fp64 ? qdot(qmul(a, b), qmul(c, d))
+                            : fix_to_double(fix_dot(fix_mul(fix_of<true>(a, 0, bad), fix_of<true>(b, 0, bad)),
+                                                    fix_mul(fix_of<true>(c, 0, bad), fix_of<true>(d, 0, bad)), 0));
+      if (nu == 3) sum[1] += v;
+      else sum[0] += v;
+      if (!fp64 && !fix_ok(bad)) break;
+    }
+    if (fix_ok(bad)) break;
+  }
+  return make_double2(sum[0], sum[1]);
+}
+
 // The two sums (spatial and space-time planes) of site s.
 template <int P>
 __device__ __forceinline__ void plaq_site(const Links<P>& L, const Geom& g, int s, float& ss, float& ts) {
@@ -88,16 +114,9 @@ __device__ __forceinline__ void plaq_site(const Links<kF64>& L, const Geom& g, i
   ss = fix_to_double(s01 + s02 + s12);
   ts = fix_to_double(s03 + s13 + s23);
   if (__builtin_expect(!fix_ok(bad), 0)) {
-    // a rolled loop over the planes, as in staple_rolled
-    ss = ts = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < 6; ++k) {
-      const int nu = k < 1 ? 1 : k < 3 ? 2 : 3, mu = nu == 1 ? 0 : nu == 2 ? k - 1 : k - 3;
-      const int hm = mu == 0 ? h0 : mu == 1 ? h1 : h2, hn = nu == 1 ? h1 : nu == 2 ? h2 : h3;
-      const double v = qdot(qmul(L.ld(2 * mu + p, h), L.ld(2 * nu + q, hm)), qmul(L.ld(2 * nu + p, h), L.ld(2 * mu + q, hn)));
-      if (nu == 3) ts += v;
-      else ss += v;
-    }
+    const double2 v = plaq_other(L, p, h, h0, h1, h2, h3);
+    ss = v.x;
+    ts = v.y;
   }
 }
 

@@ -6,10 +6,11 @@
 
 using namespace su2;
 
-static FixQuat link(const double* v, int conj, FixBad& bad) {
+static FixQuat link(const double* v, int conj, FixBad& bad, bool any = false) {
   uint32_t w[8];
   std::memcpy(w, v, sizeof w);
-  return fix_link(w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7], conj ? -1 : 0, bad);
+  return any ? fix_any_link(w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7], conj ? -1 : 0, bad)
+             : fix_link(w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7], conj ? -1 : 0, bad);
 }
 
 extern "C" {
@@ -17,13 +18,15 @@ int fixed_frac() { return kFixFrac; }
 int fixed_log_entry_alignment() { return (int)alignof(FixLog); }
 int fixed_log_entry_size() { return (int)sizeof(FixLog); }
 // out[4]: the converted components, v = h 2^29 + l; returns fix_ok
-int fixed_link(const double* v, int conj, int64_t* out) {
+static int convert(const double* v, int conj, int64_t* out, bool any) {
   FixBad bad{0, 0};
-  const FixQuat q = link(v, conj, bad);
+  const FixQuat q = link(v, conj, bad, any);
   const Fix f[4] = {q.w, q.x, q.y, q.z};
   for (int i = 0; i < 4; ++i) out[i] = (int64_t)f[i].h * (1 << kFixLow) + f[i].l;
   return fix_ok(bad);
 }
+int fixed_link(const double* v, int conj, int64_t* out) { return convert(v, conj, out, false); }
+int fixed_any_link(const double* v, int conj, int64_t* out) { return convert(v, conj, out, true); }
 int64_t fixed_any(double v) {
   uint32_t w[2];
   std::memcpy(w, &v, 8);

@@ -23,6 +23,7 @@ def lib(tmp_path_factory):
     p64 = C.POINTER(C.c_int64)
     dp = C.POINTER(C.c_double)
     L.fixed_link.argtypes = [dp, C.c_int, p64]
+    L.fixed_any_link.argtypes = L.fixed_link.argtypes
     L.fixed_any.argtypes, L.fixed_any.restype = [C.c_double], C.c_int64
     L.fixed_triples.argtypes = [dp, dp, dp, C.c_int, p64]
     L.fixed_neg_log.argtypes, L.fixed_neg_log.restype = [C.c_uint32], C.c_int64
@@ -75,6 +76,30 @@ def test_links_out_of_range_are_flagged(lib, v):
     for k in range(4):
         assert not _link(lib, np.roll(v, k))[0]
         assert not _link(lib, -np.roll(v, k), 1)[0]
+
+
+def test_links_with_components_of_any_size_convert(lib):
+    # zeros, tiny and subnormal components: refused by the first conversion, taken
+    # by the second, within one unit of 2^-58
+    rng = np.random.default_rng(5)
+    q = _units(rng, 500)
+    q[:, 1] = rng.choice([-1, 1], 500) * np.exp2(rng.uniform(-80, -32, 500))
+    q[::5, 2] = rng.choice([0.0, -0.0, 5e-324], 100)
+    q[:400] /= np.linalg.norm(q[:400], axis=1, keepdims=True)
+    axes = np.concatenate([np.eye(4), -np.eye(4)])
+    dp, ip = C.POINTER(C.c_double), C.POINTER(C.c_int64)
+    for v in np.concatenate([q, axes]):
+        for conj in (0, 1):
+            out = np.zeros(4, np.int64)
+            inside = abs(np.sum(v * v) - 1) < 0.124
+            assert not _link(lib, v, conj)[0]
+            assert lib.fixed_any_link(v.ctypes.data_as(dp), conj, out.ctypes.data_as(ip)) or not inside
+            for c in range(4):
+                assert abs(int(out[c]) * UNIT - (-1 if conj and c else 1) * Fraction(float(v[c]))) <= UNIT
+    for v in ([2.0, 0.0, 0.0, 0.0], [np.inf, 0, 0, 0], [np.nan, 0, 0, 0], [0.0] * 4, [0.9, 0, 0, 0], [1.07, 0, 0, 0], [1e300, 0, 0, 0]):
+        for k in range(4):
+            v_ = np.roll(np.array(v, np.float64), k)
+            assert not lib.fixed_any_link(v_.ctypes.data_as(dp), 0, out.ctypes.data_as(ip))
 
 
 def test_any_component_converts_within_one_unit(lib):
