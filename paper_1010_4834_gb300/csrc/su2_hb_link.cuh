@@ -194,8 +194,9 @@ static __device__ __noinline__ void or_other(Links<kF64, CP> L, const Geom& g, S
 // |U| by |W|^2 = 1 + O(2^-22), a random walk of about 1e-5 after a thousand
 // sweeps.  FP32 (and the F16Q arithmetic, whose stores are normalised again
 // on load) therefore normalises U' before storing it; in FP64 the walk (2e-15
-// rms in |U|^2 after a hundred sweeps, 9e-15 after a thousand) is let be and the update is stored as computed, like the oracle's.  NC:
-// read-only loads (no other block of the launch writes these links).
+// rms in |U|^2 after a hundred sweeps, 9e-15 after a thousand) is let be and
+// the update is stored as computed, like the oracle's.  NC: read-only loads
+// (no other block of the launch writes these links).
 template <int P, int MU, int PAR, bool NC, int CP>
 __device__ __forceinline__ void or_link(const Links<P, CP>& L, const Geom& g, Substep sub, int h) {
   sub = substep_of<MU, PAR>(sub);
