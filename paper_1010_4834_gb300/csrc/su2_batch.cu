@@ -34,8 +34,8 @@ struct su2_batch {
   uint32_t* d_sweep;
   Scratch scratch;
   double* d_results;
-  BatchBlock4* d_mblocks;  // the blocks of a measurement of every lattice
-  int n_mblocks;
+  BatchBlock4* d_mblocks[2];  // the blocks of a measurement of every lattice (plaquette, Polyakov)
+  int n_mblocks[2];
   double* h_results;
   double* d_mpart;  // measured sweeps: four partial-sum slots per CTA
   cudaStream_t stream;
@@ -99,18 +99,23 @@ void drop_graph(su2_batch* b) {
   b->graph_n = 0;
 }
 
-// The blocks of a measurement of every lattice: shares of about equal size,
-// four a multiprocessor in all, at least two sites a thread and one block a
-// lattice.
-std::vector<BatchBlock4> measure_blocks(const su2_batch* b) {
+// The blocks of a measurement of every lattice (plaquettes, or Polyakov loops: a
+// thread takes a segment of a time line): shares of about equal size, four a
+// multiprocessor in all, at least two sites a thread and one block a lattice.
+std::vector<BatchBlock4> measure_blocks(const su2_batch* b, bool polyakov) {
+  constexpr int kBlock = 256;
+  auto items = [&](int i) -> int64_t {
+    const Geom& g = b->desc[i].g;
+    return polyakov ? (2 * g.vh / g.n[3]) << polyakov_segments(g.n[3]) : 2 * g.vh;
+  };
   int64_t total = 0;
-  for (const BatchLattice& d : b->desc) total += 2 * d.g.vh;
-  const int64_t share = std::max<int64_t>(2 * 256, total / (4 * device_info().sms) + 1);
+  for (int i = 0; i < b->n; ++i) total += items(i);
+  const int64_t share = std::max<int64_t>((polyakov ? 1 : 2) * kBlock, total / (4 * device_info().sms) + 1);
+  std::vector<int> count(b->n);
+  for (int i = 0; i < b->n; ++i) count[i] = (int)((items(i) + share - 1) / share);
   std::vector<BatchBlock4> blocks;
-  for (int i = 0; i < b->n; ++i) {
-    const int count = (int)((2 * b->desc[i].g.vh + share - 1) / share);
-    for (int k = 0; k < count; ++k) blocks.push_back(BatchBlock4{i, k, count, 0});
-  }
+  for (int i = 0; i < b->n; ++i)
+    for (int k = 0; k < count[i]; ++k) blocks.push_back(BatchBlock4{i, k, count[i], 0});
   return blocks;
 }
 
@@ -300,9 +305,13 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   const size_t o_cnt = o; o = align256(o + (size_t)n * sizeof(unsigned int));
   const size_t o_out = o; o = align256(o + kScratchOut * sizeof(double));
   const size_t o_res = o; o = align256(o + 3 * (size_t)n * sizeof(double));
-  const std::vector<BatchBlock4> mblocks = measure_blocks(b);
-  b->n_mblocks = (int)mblocks.size();
-  const size_t o_mblk = o; o = align256(o + mblocks.size() * sizeof(BatchBlock4));
+  const std::vector<BatchBlock4> mblocks[2] = {measure_blocks(b, false), measure_blocks(b, true)};
+  size_t o_mblk[2];
+  for (int k = 0; k < 2; ++k) {
+    b->n_mblocks[k] = (int)mblocks[k].size();
+    o_mblk[k] = o;
+    o = align256(o + mblocks[k].size() * sizeof(BatchBlock4));
+  }
   const size_t o_mpart = o; o = align256(o + 4 * (size_t)kMaxCtas * sizeof(double));
   cudaError_t e = cudaMalloc(&b->base, o);
   if (e != cudaSuccess) {
@@ -323,7 +332,7 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   b->scratch.counter = (unsigned int*)(base + o_cnt);
   b->scratch.out = (double*)(base + o_out);
   b->d_results = (double*)(base + o_res);
-  b->d_mblocks = (BatchBlock4*)(base + o_mblk);
+  for (int k = 0; k < 2; ++k) b->d_mblocks[k] = (BatchBlock4*)(base + o_mblk[k]);
   b->d_mpart = (double*)(base + o_mpart);
   if (cuda_stream) {
     b->stream = (cudaStream_t)cuda_stream;
@@ -334,8 +343,9 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   SU2_CU_CLEAN(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMallocHost(&b->h_results, 3 * (size_t)n * sizeof(double)), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMemcpyAsync(b->d_desc, b->desc.data(), n * sizeof(BatchLattice), cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
-  SU2_CU_CLEAN(cudaMemcpyAsync(b->d_mblocks, mblocks.data(), mblocks.size() * sizeof(BatchBlock4),
-                               cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
+  for (int k = 0; k < 2; ++k)
+    SU2_CU_CLEAN(cudaMemcpyAsync(b->d_mblocks[k], mblocks[k].data(), mblocks[k].size() * sizeof(BatchBlock4),
+                                 cudaMemcpyHostToDevice, b->stream), su2_batch_destroy(b));
   SU2_CU_CLEAN(cudaMemsetAsync(b->d_bars, 0, kMaxGroups * sizeof(GroupBarrier), b->stream), su2_batch_destroy(b));
   BatchCtl ctl;
   std::memset(&ctl, 0, sizeof ctl);
@@ -576,7 +586,7 @@ static int batch_measure(su2_batch* b, int which, double* out) {
   if (!b || !out) return fail(SU2_EINVAL, "NULL argument");
   DeviceGuard dg(b->device);
   const int k = which == 0 ? 3 : 1;
-  SU2_CU(launch_batch_measure(b->prec, which != 0, b->d_desc, b->d_mblocks, b->n_mblocks, b->scratch.partials,
+  SU2_CU(launch_batch_measure(b->prec, which != 0, b->d_desc, b->d_mblocks[which], b->n_mblocks[which], b->scratch.partials,
                               b->scratch.counter, b->d_results, b->stream));
   SU2_CU(cudaMemcpyAsync(b->h_results, b->d_results, (size_t)k * b->n * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
   SU2_CU(cudaStreamSynchronize(b->stream));

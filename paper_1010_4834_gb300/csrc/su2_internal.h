@@ -101,6 +101,13 @@ cudaError_t launch_plaquette(const LatticeView& v, const Scratch& s, cudaStream_
 cudaError_t launch_time_lines(const LatticeView& v, int t0, int nt, int64_t x0, int64_t nx, double* out,
                               cudaStream_t st);
 // With `ep` the reduction partials must not overlap ep->meas.
+// log2 of the segments a time line is split into: the largest power of two up to 8
+// that divides nt and leaves segments of at least 8 links.
+__host__ __device__ inline int polyakov_segments(int nt) {
+  int lg = 0;
+  while (lg < 3 && nt % (2 << lg) == 0 && nt / (2 << lg) >= 8) ++lg;
+  return lg;
+}
 cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t st,
                             const SweepEpilogue* ep = nullptr);
 // APE: src has (at least) the 6 spatial classes; dst receives them.

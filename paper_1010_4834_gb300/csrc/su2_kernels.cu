@@ -180,12 +180,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_plaquette<kF64>(Links<kF64> L, 
 template <int P> struct PolyMinBlocks { static constexpr int value = 4; };
 template <> struct PolyMinBlocks<kF64> { static constexpr int value = 2; };
 
-template <int P, bool NC>
-__global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
-    k_polyakov(Links<P, kClassPtr> L, Geom g, int lg, double* partials, unsigned int* counter, double* out,
-               SweepEpilogue ep, int early) {
+// The sum of (1/2) Tr over block `block` of nblocks's lines, in q == 0's threads.
+template <int P, int CP, bool NC>
+__device__ __forceinline__ double polyakov_lines(const Links<P, CP>& L, const Geom& g, int lg, int block, int nblocks) {
   using R = typename Real<P>::T;
-  using LT = Links<P, kClassPtr>;
+  using LT = Links<P, CP>;
   __shared__ Quat<R> seg_prod[kThreads];
   Acc<R> acc;
   const int nsig = g.n[0] * g.n[1] * g.n[2];
@@ -196,9 +195,7 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
   const int q = threadIdx.x / lines;
   const int l = threadIdx.x - q * lines;
   const int t0 = q * seg;
-  const int zero = pdl_wait();
-  if (early) pdl_trigger();
-  for (int first = blockIdx.x * lines + zero; first < nsig; first += gridDim.x * lines) {
+  for (int first = block * lines; first < nsig; first += nblocks * lines) {
     const int xs = first + l;
     Quat<R> pr = qone<R>();
     if (xs < nsig) {
@@ -210,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
       const typename LT::E* b0 = swap ? L.cls_base(7) : L.cls_base(6);
       const typename LT::E* b1 = swap ? L.cls_base(6) : L.cls_base(7);
       const uint32_t e0 = hh + nsig_h * (uint32_t)t0;
-      pr = time_line<P, kClassPtr, NC>(b0, b1, e0, nsig_h, seg);
+      pr = time_line<P, CP, NC>(b0, b1, e0, nsig_h, seg);
     }
     if (G > 1) {
       seg_prod[threadIdx.x] = pr;
@@ -222,7 +219,17 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
     }
     if (q == 0 && xs < nsig) acc.add(pr.w);
   }
-  double v[1] = {acc.value()};
+  return acc.value();
+}
+
+template <int P, bool NC>
+__global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
+    k_polyakov(Links<P, kClassPtr> L, Geom g, int lg, double* partials, unsigned int* counter, double* out,
+               SweepEpilogue ep, int early) {
+  const int nsig = g.n[0] * g.n[1] * g.n[2];
+  const int zero = pdl_wait();
+  if (early) pdl_trigger();
+  double v[1] = {polyakov_lines<P, kClassPtr, NC>(L, g, lg, (int)blockIdx.x + zero, (int)gridDim.x)};
   if (block_partial<1>(v, partials, counter, blockIdx.x, gridDim.x)) {
     double tot[1];
     final_sum<1>(partials, gridDim.x, tot);
@@ -248,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
 // (eight sweeps and both: 3.79 against 2.30 ms).
 // ---------------------------------------------------------------------------
 template <int P, bool POLY>
-__global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : 3)
+__global__ void __launch_bounds__(kThreads, measure_blocks_per_sm(P))
     k_batch_measure(const BatchLattice* __restrict__ desc, const BatchBlock4* __restrict__ blocks, double* partials,
                     unsigned int* counters, double* out) {
   using R = typename Real<P>::T;
@@ -256,21 +263,13 @@ __global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : 3)
   const Geom& g = desc[b.lattice].g;
   Links<P> L;
   L.set(desc[b.lattice].links, g.vh);
-  const int first = b.rank * kThreads + (int)threadIdx.x, stride = b.count * kThreads;
   constexpr int NV = POLY ? 1 : 2;
   double v[NV];
   if constexpr (POLY) {
-    Acc<R> acc;
-    const int nsig = g.n[0] * g.n[1] * g.n[2];
-    for (int xs = first; xs < nsig; xs += stride) {
-      const int odd = parity(site_from_index(g, (uint32_t)xs));   // of (xs, t = 0)
-      acc.add(time_line<P, kFlat, true>(L.cls_base(6 + odd), L.cls_base(7 - odd), (uint32_t)(xs >> 1), (uint32_t)(nsig / 2),
-                                  g.n[3]).w);
-    }
-    v[0] = acc.value();
+    v[0] = polyakov_lines<P, kFlat, true>(L, g, polyakov_segments(g.n[3]), b.rank, b.count);
   } else {
     Acc<R> sp, tm;
-    for (int s = first; s < (int)(2 * g.vh); s += stride) {
+    for (int s = b.rank * kThreads + (int)threadIdx.x; s < (int)(2 * g.vh); s += b.count * kThreads) {
       R ss, ts;
       plaq_site(L, g, s, ss, ts);
       sp.add(ss);
@@ -1358,10 +1357,7 @@ cudaError_t launch_polyakov(const LatticeView& v, const Scratch& s, cudaStream_t
   SU2_DISPATCH(v.prec, {
     auto L = links_of<P, kClassPtr>(v.links, v.g.vh);
     const int64_t nsig = 2 * v.g.vh / v.g.n[3];
-    // segments per time line: the largest power of two <= 8 that divides nt
-    // and leaves segments of at least 8 links
-    int lg = 0;
-    while (lg < 3 && v.g.n[3] % (2 << lg) == 0 && v.g.n[3] / (2 << lg) >= 8) ++lg;
+    const int lg = polyakov_segments(v.g.n[3]);
     auto launch = [&](auto kernel) {
       const int gr = grid_for(kernel, nsig << lg);
       return launch_pdl(overlaps(v), kernel, dim3(gr), kThreads, st, L, v.g, lg, s.partials, s.counter, s.out, e, (int)overlaps(v));

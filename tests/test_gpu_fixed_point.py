@@ -222,3 +222,27 @@ def test_batched_measurements_of_uneven_lattices():
                 ref = as_stored(U, prec)
                 np.testing.assert_allclose(plaq[i], oracle.plaquette(list(d), ref), atol=MTOL[prec], rtol=0)
                 assert abs(poly[i] - oracle.polyakov(list(d), ref)) < MTOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16q"])
+def test_batched_polyakov_loops_of_long_time_extents(prec):
+    # lines in one, two, four and eight segments, the last of a length that is no
+    # multiple of the loads' eight; a lattice of fewer lines than a block has threads
+    dims = [(4, 2, 2, 14), (2, 2, 2, 16), (4, 4, 2, 40), (2, 4, 2, 72), (6, 6, 6, 136)]
+    b = Batch(dims, [2.0] * len(dims), seed=1, start="cold", prec=prec)
+    fields = [inputs.random_field(d, 70 + i) for i, d in enumerate(dims)]
+    for i, U in enumerate(fields):
+        b.set_links(i, U)
+    for _ in range(2):
+        poly, plaq = b.polyakov(), b.plaquette()
+        for i, (d, U) in enumerate(zip(dims, fields)):
+            ref = as_stored(U, prec)
+            assert abs(poly[i] - oracle.polyakov(list(d), ref)) < MTOL[prec]
+            np.testing.assert_allclose(plaq[i], oracle.plaquette(list(d), ref), atol=MTOL[prec], rtol=0)
+
+
+def test_a_batch_measures_long_time_extents_like_a_lattice():
+    # one thread a line took three times a single lattice's time
+    dims = (8, 8, 8, 512)
+    lat, b = Lattice(dims, 2.4, prec="f64"), Batch([dims], [2.4], prec="f64")
+    assert _seconds(b.polyakov) < 2 * _seconds(lat.polyakov)
