@@ -32,8 +32,9 @@ constexpr int kBatchThreads = 256;  // default
 struct BatchBlock4 {
   int lattice, rank, count, pad;
 };
-// Resident blocks of 256 of the batched measurements an SM.
-constexpr int measure_blocks_per_sm(int prec) { return prec == kF64 ? 2 : 3; }
+// Resident blocks of 256 of the batched measurements an SM: 64 registers a thread
+// below FP64.
+constexpr int measure_blocks_per_sm(int prec) { return prec == kF64 ? 2 : 4; }
 // Plaquette means (3 doubles a lattice) or Polyakov loops (1) of every lattice;
 // counters: one zero word a lattice, left zero.
 cudaError_t launch_batch_measure(int prec, bool polyakov, const BatchLattice* desc, const BatchBlock4* blocks,
