@@ -392,24 +392,9 @@ __device__ __forceinline__ void ape_sites(const Links<P, kClassPtr>& src, const 
 // Sharing the forward products among a site's three links as above keeps three
 // sums of 16 registers and spilled 2 KB a thread; the nine further loads and
 // conversions cost less.
-template <bool NC, bool ANY>
-__device__ __forceinline__ bool ape_fixed(const Links<kF64>& src, const Links<kF64>& dst, const Geom& g, const Site& x,
-                                          int h, int mu, int p, double c0, double c1) {
-  FixSum s;
-  Quat<double> lower;
-  if (!staple_fixed<false, NC, false, ANY>(src, g, x, h, mu, p, 3, s, lower)) return false;
-  ape_store<kF64>(dst, 2 * mu + p, h, ldl<kF64, NC>(src, 2 * mu + p, h), fix_sum_to_double(s), c0, c1);
-  return true;
-}
-// The links that fix_link refuses, out of line.
-template <bool NC>
-static __device__ __noinline__ void ape_other(Links<kF64> src, Links<kF64> dst, const Geom& g, Site x, int h, int mu, int p,
-                                              double c0, double c1) {
-  if (ape_fixed<NC, true>(src, dst, g, x, h, mu, p, c0, c1)) return;
-  Quat<double> lower;
-  const Quat<double> sig = staple_rolled<NC, false>(src, g, x, h, mu, p, 3, lower);
-  ape_store<kF64>(dst, 2 * mu + p, h, ldl<kF64, NC>(src, 2 * mu + p, h), sig, c0, c1);
-}
+// Links that fix_link refuses are computed in FP64 at once: a second conversion, as in
+// the heat bath, would cost all fields 2% here, and out of line 1.8 us a step (20 x 12
+// x 18 x 10: 18.0 -> 19.8); a cold 24^3x32 takes 398 us a step for 149.
 template <bool NC>
 __device__ __forceinline__ void ape_links_fixed(const Links<kF64>& src, const Links<kF64>& dst, const Geom& g, int mu,
                                                 int p, double c0, double c1) {
@@ -417,14 +402,19 @@ __device__ __forceinline__ void ape_links_fixed(const Links<kF64>& src, const Li
   const int stride = gridDim.x * blockDim.x;
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < vh; h += stride) {
     const Site x = site_from_half(g, (uint32_t)h, p);
-    if (__builtin_expect(!ape_fixed<NC, false>(src, dst, g, x, h, mu, p, c0, c1), 0))
-      ape_other<NC>(src, dst, g, x, h, mu, p, c0, c1);
+    FixSum s;
+    Quat<double> sig;
+    if (__builtin_expect(staple_fixed<false, NC, false>(src, g, x, h, mu, p, 3, s, sig), 1))
+      sig = fix_sum_to_double(s);
+    else
+      sig = staple_rolled<NC, false>(src, g, x, h, mu, p, 3, sig);
+    ape_store<kF64>(dst, 2 * mu + p, h, ldl<kF64, NC>(src, 2 * mu + p, h), sig, c0, c1);
   }
 }
 
 template <int P, bool NC>
 __global__ void __launch_bounds__(kThreads, P == kF64 ? 2 : SU2_APE3_MINB)
-    k_ape(Links<P, hb_addr<P, kClassPtr>> src, Links<P, hb_addr<P, kClassPtr>> dst, const __grid_constant__ Geom g, double alpha_d, int early) {
+    k_ape(Links<P, hb_addr<P, kClassPtr>> src, Links<P, hb_addr<P, kClassPtr>> dst, Geom g, double alpha_d, int early) {
   using R = typename Real<P>::T;
   const int zero = pdl_wait();
   if (early) pdl_trigger();
