@@ -248,9 +248,9 @@ template <class R> struct Math;
 
 // FP64 roots and reciprocals from an FP32 approximation of the significand
 // (2^-22, taken and put back by bit operations: the FP64 pipe also does the
-// conversions) and one third-order step: 5, 6 and 3 FP64 operations, where
-// 1/sqrt(v), sqrt(v) and a division take about 20, 10 and 10.  Errors below
-// one unit in the last place of v > 0 normal.
+// conversions) and one third-order step (Householder's method): 5, 6 and 3 FP64
+// operations, where 1/sqrt(v), sqrt(v) and a division take about 20, 10 and 10.
+// Errors below one unit in the last place for v > 0 normal (not correctly rounded).
 __device__ __forceinline__ float significand32(double v, int exponent) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   return __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7FFFFFu) | ((uint32_t)(127 + exponent) << 23));

@@ -8,11 +8,15 @@
 // A component v of a link is held as two signed 32-bit limbs,
 //   v = h 2^-29 + l 2^-58,  |l| < 2^29,
 // and a product of two components as (h h') 2^-58 + (h l' + l h') 2^-87, the
-// two parts in 64-bit sums; l l' < 2^-58 is left out.  Errors, absolute:
-// a converted component is truncated at 2^-58, a product's omitted part and
-// its rounding are below 2^-58 each; a staple sum (magnitude up to 6, FP64
-// roundings of 2^-53 and more per addition) comes out within about 2^-54 in
-// the worst case and 2^-56 typically, several times closer than in FP64.
+// two parts in 64-bit sums; l l' < 2^-58 is left out.  Errors, absolute, in units
+// of 2^-58, for norms n <= 1.0607 (a quaternion's components then add up to 2 n at
+// most): a converted component is truncated below 1; a component of a product of two
+// links carries 4 n from their conversions, below 4 from four l l' and 4 from its
+// rounding to 8 units, 12.3 together; a term of a staple, that product times a
+// third link, 2 n 12.3 + 2 n^2 + 2 = 30.3 (the product's low limbs are centred); the
+// sum of six and its rounding 186, or 2^-50.4.  Measured: a product 6.7 at most, 2.4
+// rms; a staple sum 2^-53.3 at most, 2^-55.3 rms, several times closer than in FP64
+// (magnitude up to 6, roundings of 2^-53 and more per addition).
 //
 // What a link must be for this: components |v| in [2^-31, 2) and a norm within 6%
 // of one.  fix_link raises `bad` otherwise, and the thread starts again with
@@ -283,7 +287,8 @@ static __device__ const FixLog fix_log_table[128] = {SU2_FIX_LOG_TABLE};
 #endif
 static const FixLog fix_log_table_host[128] = {SU2_FIX_LOG_TABLE};
 
-// -ln u in units of 2^-58 (at most 22.9), error below 2^-57 (1 - ln u): with z =
+// -ln u in units of 2^-58 (at most 22.9), absolute error below 2^-57 (1 - ln u)
+// (near u = 1 few digits of the logarithm itself: a0 takes it absolutely): with z =
 // m 2^(63 - lz), 1 <= m < 2, -ln u = (lz - 30) ln 2 + t - ln(1 + r), where r = m
 // I 2^-16 - 1 is exact in 48 bits, |r| < 2^-7.9, and ln(1 + r) = r - r q, q =
 // p 2^-8 - p^2 2^-14/3 + p^3 2^-23 - ... in p = 2^7 r (Taylor to r^7).

@@ -142,9 +142,11 @@ def test_sums_of_products_are_closer_than_fp64(lib):
         worst = max(worst, float(e))
         off += [float(int(out[k]) * UNIT - ref[k]) for k in range(4)]
         off64 += [float(Fraction(float(f64[k])) - ref[k]) for k in range(4)]
-    # 18 conversions (2^-58 each, times the other two norms) and 48 products'
-    # omitted parts and roundings bound the sum by 2^-52; typically 2^-55
-    assert worst < 2.0 ** -53
+    # a product of two links: 4 n (conversions) + 4 (low limbs left out) + 4 (rounding)
+    # units of 2^-58, n = 1.0607; times a third link 2 n times that, + 2 n^2 + 2; six
+    # terms and the sum's rounding
+    n = 1.0607
+    assert worst < (6 * (2 * n * (4 * n + 8) + 2 * n * n + 2) + 4) * float(UNIT)
     assert np.sqrt(np.mean(np.square(off))) < 0.25 * np.sqrt(np.mean(np.square(off64)))
 
 

@@ -4,6 +4,9 @@ temporal-gauge Wilson kernel on time extents of every remainder.  FP64 against
 the oracle at 1e-12 (values up to 6 and about a hundred operations of 2^-53
 each leave 1e-14; loops up to W = |U|^64 on scaled links are compared relative to
 their size)."""
+import ctypes as C
+import os
+import subprocess
 import time
 
 import numpy as np
@@ -11,6 +14,7 @@ import pytest
 
 import oracle
 from paper_1010_4834_gb300 import Batch, Lattice, inputs
+from paper_1010_4834_gb300.build import ARCH, CSRC, INCLUDE, nvcc_path
 from test_gpu_parity import MTOL, as_stored, substep_compare
 
 pytestmark = pytest.mark.gpu
@@ -246,3 +250,30 @@ def test_a_batch_measures_long_time_extents_like_a_lattice():
     dims = (8, 8, 8, 512)
     lat, b = Lattice(dims, 2.4, prec="f64"), Batch([dims], [2.4], prec="f64")
     assert _seconds(b.polyakov) < 2 * _seconds(lat.polyakov)
+
+
+def test_roots_and_reciprocal_within_a_unit_in_the_last_place(tmp_path):
+    # against numpy's extended arithmetic: every exponent that a staple's square or
+    # an alpha can have and far beyond, both parities of it, significands near 1 and 2
+    if np.finfo(np.longdouble).nmant < 63:
+        pytest.skip("long double has no more bits than double here")
+    so = str(tmp_path / "roots.so")
+    here = os.path.dirname(os.path.abspath(__file__))
+    subprocess.run([nvcc_path(), *ARCH, "-O3", "-std=c++17", "-ftz=true", "-shared", "-Xcompiler", "-fPIC", "-I", INCLUDE,
+                    "-I", CSRC, os.path.join(here, "roots_device.cu"), "-o", so], check=True)
+    rng = np.random.default_rng(6)
+    v = np.exp2(rng.uniform(-40, 70, 300000))
+    v = np.concatenate([v, np.exp2(np.arange(-900, 901.0)), np.nextafter(np.exp2(np.arange(-900, 901.0)), 0),
+                        np.nextafter(np.exp2(np.arange(-900, 901.0)), np.inf), np.exp2(rng.uniform(-900, 900, 20000))])
+    out = np.zeros((3, v.size))
+    dp = C.POINTER(C.c_double)
+    assert C.CDLL(so).roots(v.ctypes.data_as(dp), C.c_int(v.size), out.ctypes.data_as(dp)) == 0
+    x = v.astype(np.longdouble)
+    for got, ref in zip(out, (1 / np.sqrt(x), np.sqrt(x), 0.5 / x)):
+        ulp = np.spacing(ref.astype(np.float64))
+        assert (np.abs(got.astype(np.longdouble) - ref) / ulp).max() < 1
+    # zero, negative and subnormal under the root; an infinite alpha
+    edge = np.array([0.0, -0.0, -1.0, 5e-324, np.inf, 1e300 * 1e8])
+    out = np.zeros((3, edge.size))
+    assert C.CDLL(so).roots(edge.ctypes.data_as(dp), C.c_int(edge.size), out.ctypes.data_as(dp)) == 0
+    assert (out[1, :4] == 0).all() and (out[2, 4:] == 0).all()
