@@ -22,7 +22,7 @@
 // of one.  fix_link raises `bad` otherwise, and the thread starts again with
 // fix_any_link, which takes any |v| < 2 (zeros: cold starts, Abelian fields) and
 // costs twice the shifts; values other than near-unit quaternions, which a store
-// set from outside may hold, are computed in FP64.
+// set from outside may hold, are computed in FP64 (smearing does so at once).
 //
 // Sums.  With norms n <= 1.0607: |sum h h'| <= 2^58 n^2 per component of a
 // product (Cauchy-Schwarz); |sum (h l' + l h')| <= 2^29 (sum |h| + sum |h'|)
