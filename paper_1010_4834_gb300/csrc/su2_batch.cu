@@ -32,7 +32,7 @@ struct su2_batch {
   GroupBarrier* d_bars;
   BatchCtl* d_ctl;
   uint32_t* d_sweep;
-  Scratch scratch;
+  Scratch scratch;  // partials and counters of the measurements
   double* d_results;
   BatchBlock4* d_mblocks[2];  // the blocks of a measurement of every lattice (plaquette, Polyakov)
   int n_mblocks[2];
@@ -310,7 +310,6 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   const size_t o_sweep = o; o = align256(o + 64);
   const size_t o_part = o; o = align256(o + kScratchPartials * sizeof(double));
   const size_t o_cnt = o; o = align256(o + (size_t)n * sizeof(unsigned int));
-  const size_t o_out = o; o = align256(o + kScratchOut * sizeof(double));
   const size_t o_res = o; o = align256(o + 3 * (size_t)n * sizeof(double));
   const std::vector<BatchBlock4> mblocks[2] = {measure_blocks(b, false), measure_blocks(b, true)};
   size_t o_mblk[2];
@@ -337,7 +336,6 @@ extern "C" int su2_batch_init(su2_batch** out, int n, const int* dims, const dou
   b->d_sweep = (uint32_t*)(base + o_sweep);
   b->scratch.partials = (double*)(base + o_part);
   b->scratch.counter = (unsigned int*)(base + o_cnt);
-  b->scratch.out = (double*)(base + o_out);
   b->d_results = (double*)(base + o_res);
   for (int k = 0; k < 2; ++k) b->d_mblocks[k] = (BatchBlock4*)(base + o_mblk[k]);
   b->d_mpart = (double*)(base + o_mpart);
