@@ -180,11 +180,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_plaquette<kF64>(Links<kF64> L, 
 template <int P> struct PolyMinBlocks { static constexpr int value = 4; };
 template <> struct PolyMinBlocks<kF64> { static constexpr int value = 2; };
 
-// The sum of (1/2) Tr over block `block` of nblocks's lines, in q == 0's threads.
-template <int P, int CP, bool NC>
-__device__ __forceinline__ double polyakov_lines(const Links<P, CP>& L, const Geom& g, int lg, int block, int nblocks) {
+template <int P, bool NC>
+__global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
+    k_polyakov(Links<P, kClassPtr> L, Geom g, int lg, double* partials, unsigned int* counter, double* out,
+               SweepEpilogue ep, int early) {
   using R = typename Real<P>::T;
-  using LT = Links<P, CP>;
+  using LT = Links<P, kClassPtr>;
   __shared__ Quat<R> seg_prod[kThreads];
   Acc<R> acc;
   const int nsig = g.n[0] * g.n[1] * g.n[2];
@@ -195,7 +196,9 @@ __device__ __forceinline__ double polyakov_lines(const Links<P, CP>& L, const Ge
   const int q = threadIdx.x / lines;
   const int l = threadIdx.x - q * lines;
   const int t0 = q * seg;
-  for (int first = block * lines; first < nsig; first += nblocks * lines) {
+  const int zero = pdl_wait();
+  if (early) pdl_trigger();
+  for (int first = blockIdx.x * lines + zero; first < nsig; first += gridDim.x * lines) {
     const int xs = first + l;
     Quat<R> pr = qone<R>();
     if (xs < nsig) {
@@ -207,7 +210,7 @@ __device__ __forceinline__ double polyakov_lines(const Links<P, CP>& L, const Ge
       const typename LT::E* b0 = swap ? L.cls_base(7) : L.cls_base(6);
       const typename LT::E* b1 = swap ? L.cls_base(6) : L.cls_base(7);
       const uint32_t e0 = hh + nsig_h * (uint32_t)t0;
-      pr = time_line<P, CP, NC>(b0, b1, e0, nsig_h, seg);
+      pr = time_line<P, kClassPtr, NC>(b0, b1, e0, nsig_h, seg);
     }
     if (G > 1) {
       seg_prod[threadIdx.x] = pr;
@@ -219,17 +222,7 @@ __device__ __forceinline__ double polyakov_lines(const Links<P, CP>& L, const Ge
     }
     if (q == 0 && xs < nsig) acc.add(pr.w);
   }
-  return acc.value();
-}
-
-template <int P, bool NC>
-__global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
-    k_polyakov(Links<P, kClassPtr> L, Geom g, int lg, double* partials, unsigned int* counter, double* out,
-               SweepEpilogue ep, int early) {
-  const int nsig = g.n[0] * g.n[1] * g.n[2];
-  const int zero = pdl_wait();
-  if (early) pdl_trigger();
-  double v[1] = {polyakov_lines<P, kClassPtr, NC>(L, g, lg, (int)blockIdx.x + zero, (int)gridDim.x)};
+  double v[1] = {acc.value()};
   if (block_partial<1>(v, partials, counter, blockIdx.x, gridDim.x)) {
     double tot[1];
     final_sum<1>(partials, gridDim.x, tot);
@@ -254,6 +247,50 @@ __global__ void __launch_bounds__(kThreads, PolyMinBlocks<P>::value)
 // lattice, the two measurements of 64 lattices of 8^4 to 24^3 x 6 took 1.5 ms more
 // (eight sweeps and both: 3.79 against 2.30 ms).
 // ---------------------------------------------------------------------------
+// A block's sum of (1/2) Tr over its share of a lattice's time lines, split into
+// segments as in k_polyakov (which, as a caller of this, took other registers and
+// with them 1 us more of a measured sweep: 32^3x4, F16Q).
+template <int P>
+__device__ __forceinline__ double polyakov_lines(const Links<P>& L, const Geom& g, int lg, int block, int nblocks) {
+  using R = typename Real<P>::T;
+  using LT = Links<P>;
+  __shared__ Quat<R> seg_prod[kThreads];
+  Acc<R> acc;
+  const int nsig = g.n[0] * g.n[1] * g.n[2];
+  const uint32_t nsig_h = (uint32_t)(nsig / 2);
+  const int G = 1 << lg;
+  const int lines = kThreads >> lg;  // lines per block, a multiple of 32
+  const int seg = g.n[3] >> lg;
+  const int q = threadIdx.x / lines;
+  const int l = threadIdx.x - q * lines;
+  const int t0 = q * seg;
+  for (int first = block * lines; first < nsig; first += nblocks * lines) {
+    const int xs = first + l;
+    Quat<R> pr = qone<R>();
+    if (xs < nsig) {
+      const Site x = site_from_index(g, (uint32_t)xs);
+      const uint32_t hh = (uint32_t)(xs >> 1);
+      // the time links of x alternate between the two parity classes: b0
+      // holds those at t of the parity of t0, b1 the others
+      const bool swap = (parity(x) ^ (t0 & 1)) != 0;
+      const typename LT::E* b0 = swap ? L.cls_base(7) : L.cls_base(6);
+      const typename LT::E* b1 = swap ? L.cls_base(6) : L.cls_base(7);
+      const uint32_t e0 = hh + nsig_h * (uint32_t)t0;
+      pr = time_line<P, kFlat, true>(b0, b1, e0, nsig_h, seg);
+    }
+    if (G > 1) {
+      seg_prod[threadIdx.x] = pr;
+      __syncthreads();
+      if (q == 0) {
+        for (int k = 1; k < G; ++k) pr = qmul(pr, seg_prod[k * lines + l]);
+      }
+      __syncthreads();
+    }
+    if (q == 0 && xs < nsig) acc.add(pr.w);
+  }
+  return acc.value();
+}
+
 template <int P, bool POLY>
 __global__ void __launch_bounds__(kThreads, measure_blocks_per_sm(P))
     k_batch_measure(const BatchLattice* __restrict__ desc, const BatchBlock4* __restrict__ blocks, double* partials,
@@ -266,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, measure_blocks_per_sm(P))
   constexpr int NV = POLY ? 1 : 2;
   double v[NV];
   if constexpr (POLY) {
-    v[0] = polyakov_lines<P, kFlat, true>(L, g, polyakov_segments(g.n[3]), b.rank, b.count);
+    v[0] = polyakov_lines<P>(L, g, polyakov_segments(g.n[3]), b.rank, b.count);
   } else {
     Acc<R> sp, tm;
     for (int s = b.rank * kThreads + (int)threadIdx.x; s < (int)(2 * g.vh); s += b.count * kThreads) {
