@@ -101,15 +101,14 @@ __device__ __forceinline__ void batch_substep(const Links<P, hb_addr<P, kClassOf
   using Def = Deferred<R, MEAS>;
   Def* queue = static_cast<Def*>(queue_mem);
   constexpr int kQ = BatchQueue<BS>::value;
-  HBCount cnt;
   const int vh = (int)g.vh;
   for (int base = rank * BS; base < vh; base += cpg * BS) {
     const int h = base + threadIdx.x;
     if (h < vh)
-      hb_link<P, MU, MEAS, PAR, false, kQ, hb_addr<P, kClassOff>, false>(L, g, sub, h, tag, sweep, beta, hp, queue, qn, plaq, cnt);
+      hb_link<P, MU, MEAS, PAR, false, kQ, hb_addr<P, kClassOff>, false>(L, g, sub, h, tag, sweep, beta, hp, queue, qn, plaq);
   }
   __syncthreads();
-  hb_drain<P, MU, MEAS, PAR, hb_addr<P, kClassOff>, false>(L, sub, queue, min(*qn, kQ), tag, sweep, hp, plaq, cnt);
+  hb_drain<P, MU, MEAS, PAR, hb_addr<P, kClassOff>, false>(L, sub, queue, min(*qn, kQ), tag, sweep, hp, plaq);
   __syncthreads();
   if (threadIdx.x == 0) *qn = 0;
 }

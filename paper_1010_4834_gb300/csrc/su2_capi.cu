@@ -54,7 +54,6 @@ struct su2_lattice {
   void* ape[2];
   Scratch scratch;
   uint32_t* d_sweep;
-  unsigned long long* d_stats;
   double* d_hist;
   double* staging;
   int64_t staging_sites;
@@ -211,7 +210,6 @@ static int init_common(su2_lattice** out, const int dims[4], double beta, uint64
   h->scratch.partials = (double*)(b + L.partials);
   h->scratch.counter = (unsigned int*)(b + L.counter);
   h->d_sweep = (uint32_t*)(b + L.state);
-  h->d_stats = (unsigned long long*)(b + L.state + 64);
   h->d_pair = (PairCtl*)(b + L.pair);
   h->d_done0 = (unsigned int*)(b + L.pair + sizeof(PairCtl));
   h->schedule = SU2_SCHED_AUTO;
@@ -380,7 +378,7 @@ static cudaError_t enqueue_sweep(su2_lattice* h, uint32_t off, cudaStream_t st) 
   }
   for (int mu = 0; mu < 4; ++mu)
     for (int p = 0; p < 2; ++p) {
-      e = launch_heatbath(v, mu, p, h->d_sweep, off, hp, nullptr, st);
+      e = launch_heatbath(v, mu, p, h->d_sweep, off, hp, st);
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
@@ -410,7 +408,7 @@ static cudaError_t enqueue_measured_sweep(su2_lattice* h, cudaStream_t st) {
       continue;
     }
     for (int p = 0; p < 2; ++p) {
-      e = launch_heatbath(v, mu, p, h->d_sweep, 0u, hp, nullptr, st, p == 1 ? meas : nullptr,
+      e = launch_heatbath(v, mu, p, h->d_sweep, 0u, hp, st, p == 1 ? meas : nullptr,
                           p == 1 ? nb : nullptr);
       if (e != cudaSuccess) return e;
     }
@@ -619,7 +617,7 @@ extern "C" int su2_heatbath_substep(su2_lattice* h, int mu, int parity, uint32_t
   if (!h) return fail(SU2_EINVAL, "handle is NULL");
   if (mu < 0 || mu > 3 || parity < 0 || parity > 1) return fail(SU2_EINVAL, "mu must be 0..3 and parity 0..1");
   DeviceGuard dg(h->device);
-  SU2_CU(launch_heatbath(view(h), mu, parity, nullptr, sweep, hb_params(h), nullptr, h->stream));
+  SU2_CU(launch_heatbath(view(h), mu, parity, nullptr, sweep, hb_params(h), h->stream));
   h->smeared = 0;
   return SU2_OK;
 }

@@ -43,11 +43,6 @@ template <class R> struct __align__(16) Deferred<R, true> {
   Quat<R> lower;
 };
 
-// Trial, capped and Haar counts of the links a thread finished.
-struct HBCount {
-  unsigned int trials = 0, capped = 0, haar = 0;
-};
-
 template <class R, bool MEAS>
 __device__ __forceinline__ int finish_deferred(const Deferred<R, MEAS>& d, uint4 ctr, const HBParams& hp,
                                                Quat<R>* out) {
@@ -82,7 +77,7 @@ template <int P, int MU, bool MEAS, int PAR, bool MCG, int CAP, int CP, bool NC 
 __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Substep sub, int h, uint32_t tag, uint32_t sweep,
                                         typename Real<P>::T beta, const HBParams& hp,
                                         Deferred<typename Real<P>::T, MEAS>* queue, int* qn,
-                                        PlainAcc<typename Real<P>::T>& plaq, HBCount& cnt) {
+                                        PlainAcc<typename Real<P>::T>& plaq) {
   sub = substep_of<MU, PAR>(sub);
   const int mu = sub.mu, p = sub.p;
   using R = typename Real<P>::T;
@@ -99,7 +94,6 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
     const Quat<R> nl = haar_from<R>(philox(c, hp.rk));
     if constexpr (MEAS) plaq.add(qdot_rn(L.put(2 * mu + p, h, nl), lower));
     else L.st(2 * mu + p, h, nl);
-    cnt.haar += 1;
     return;
   }
   const R inv2a = trial_inv2a(alpha);
@@ -111,7 +105,6 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
     const Quat<R> nl = compose_link<R>(a0, w, ctr, rt, hp);
     if constexpr (MEAS) plaq.add(qdot_rn(L.put(2 * mu + p, h, nl), lower));
     else L.st(2 * mu + p, h, nl);
-    cnt.trials += 1;
   } else if (hp.max_tries > 1) {
     const int slot = atomicAdd(qn, 1);
     Def d;
@@ -127,13 +120,9 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
       const int n = finish_deferred<R, MEAS>(d, ctr, hp, &nl);
       if constexpr (MEAS) plaq.add(qdot_rn(n ? L.put(2 * mu + p, h, nl) : ldl<P, NC>(L, 2 * mu + p, h), lower));
       else if (n) L.st(2 * mu + p, h, nl);
-      cnt.trials += n ? (unsigned)n : (unsigned)hp.max_tries;
-      cnt.capped += n == 0;
     }
   } else {
     if constexpr (MEAS) plaq.add(qdot_rn(ldl<P, NC>(L, 2 * mu + p, h), lower));
-    cnt.trials += 1;
-    cnt.capped += 1;
   }
 }
 
@@ -141,7 +130,7 @@ __device__ __forceinline__ void hb_link(const Links<P, CP>& L, const Geom& g, Su
 template <int P, int MU, bool MEAS, int PAR, int CP, bool NC = true>
 __device__ __forceinline__ void hb_drain(const Links<P, CP>& L, Substep sub, const Deferred<typename Real<P>::T, MEAS>* queue, int n,
                                          uint32_t tag, uint32_t sweep, const HBParams& hp,
-                                         PlainAcc<typename Real<P>::T>& plaq, HBCount& cnt) {
+                                         PlainAcc<typename Real<P>::T>& plaq) {
   sub = substep_of<MU, PAR>(sub);
   const int mu = sub.mu, p = sub.p;
   using R = typename Real<P>::T;
@@ -151,8 +140,6 @@ __device__ __forceinline__ void hb_drain(const Links<P, CP>& L, Substep sub, con
     const int t = finish_deferred<R, MEAS>(d, make_uint4(d.site, tag, sweep, 0u), hp, &nl);
     if constexpr (MEAS) plaq.add(qdot_rn(t ? L.put(2 * mu + p, d.h, nl) : ldl<P, NC>(L, 2 * mu + p, d.h), d.lower));
     else if (t) L.st(2 * mu + p, d.h, nl);
-    cnt.trials += t ? (unsigned)t : (unsigned)hp.max_tries;
-    cnt.capped += t == 0;
   }
 }
 

@@ -7,13 +7,13 @@ namespace su2 {
 
 template <int P>
 cudaError_t launch_heatbath_prec(const LatticeView& v, int mu, int parity, const uint32_t* sweep_base,
-                                 uint32_t sweep_off, const HBParams& hp, unsigned long long* stats, cudaStream_t st,
+                                 uint32_t sweep_off, const HBParams& hp, cudaStream_t st,
                                  double* meas, int* meas_blocks);
 
 cudaError_t launch_heatbath(const LatticeView& v, int mu, int parity, const uint32_t* sweep_base,
-                            uint32_t sweep_off, const HBParams& hp, unsigned long long* stats,
+                            uint32_t sweep_off, const HBParams& hp,
                             cudaStream_t st, double* meas, int* meas_blocks) {
-  SU2_DISPATCH(v.prec, return launch_heatbath_prec<P>(v, mu, parity, sweep_base, sweep_off, hp, stats, st, meas, meas_blocks));
+  SU2_DISPATCH(v.prec, return launch_heatbath_prec<P>(v, mu, parity, sweep_base, sweep_off, hp, st, meas, meas_blocks));
   return cudaErrorInvalidValue;
 }
 

@@ -79,7 +79,7 @@ template <int P, int BS> struct HbMinBlocks {
 template <int P, int MU, bool MEAS, int PAR, int BS>
 __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
     k_heatbath(Links<P, hb_addr<P, kClassPtr>> L, const __grid_constant__ Geom g, Substep sub, const uint32_t* sweep_base, uint32_t sweep_off,
-               const __grid_constant__ HBParams hp, unsigned long long* stats, double* meas) {
+               const __grid_constant__ HBParams hp, double* meas) {
   const int mu = substep_of<MU, PAR>(sub).mu;
   using R = typename Real<P>::T;
   using Def = Deferred<R, MEAS>;
@@ -91,7 +91,6 @@ __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
   const R beta = (R)hp.beta;
   const uint32_t sweep = (sweep_base ? *sweep_base : 0u) + sweep_off;
   const uint32_t tag = (uint32_t)mu | hp.lattice_tag;
-  HBCount cnt;
   // MEAS: plaquettes of the planes (NU < MU, MU).  A plain sum: a thread adds
   // vh / (grid size) terms of magnitude <= 2 (about 55 on 64^4), so FP32
   // rounding stays near 1e-6 relative per thread before the FP64 block sums.
@@ -103,10 +102,10 @@ __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
   int it = 0;
   for (int base = blockIdx.x * blockDim.x + zero; base < vh; base += stride, ++it) {
     const int h = base + threadIdx.x;
-    if (h < vh) hb_link<P, MU, MEAS, PAR, false, kDeferCap>(L, g, sub, h, tag, sweep, beta, hp, queue, &qn, plaq, cnt);
+    if (h < vh) hb_link<P, MU, MEAS, PAR, false, kDeferCap>(L, g, sub, h, tag, sweep, beta, hp, queue, &qn, plaq);
     if ((it % DeferEvery<MEAS>::value) == DeferEvery<MEAS>::value - 1 || base + stride >= vh) {
       __syncthreads();
-      hb_drain<P, MU, MEAS, PAR>(L, sub, queue, min(qn, kDeferCap), tag, sweep, hp, plaq, cnt);
+      hb_drain<P, MU, MEAS, PAR>(L, sub, queue, min(qn, kDeferCap), tag, sweep, hp, plaq);
       __syncthreads();
       if (threadIdx.x == 0) qn = 0;
       __syncthreads();
@@ -122,16 +121,6 @@ __global__ void __launch_bounds__(BS, HbMinBlocks<P, BS>::value)
       for (int w = 0; w < kHbThreads / 32; ++w) t += shp[w];
       meas[blockIdx.x] = t;
     }
-  }
-  if (stats) {
-    __shared__ unsigned int sh[3];
-    if (threadIdx.x < 3) sh[threadIdx.x] = 0;
-    __syncthreads();
-    if (cnt.trials) atomicAdd(&sh[0], cnt.trials);
-    if (cnt.capped) atomicAdd(&sh[1], cnt.capped);
-    if (cnt.haar) atomicAdd(&sh[2], cnt.haar);
-    __syncthreads();
-    if (threadIdx.x < 3 && sh[threadIdx.x]) atomicAdd(stats + threadIdx.x, (unsigned long long)sh[threadIdx.x]);
   }
 }
 
@@ -408,7 +397,7 @@ __global__ void __launch_bounds__(64, 8)
 // ---------------------------------------------------------------------------
 template <int P>
 cudaError_t launch_heatbath_prec(const LatticeView& v, int mu, int parity, const uint32_t* sweep_base,
-                                 uint32_t sweep_off, const HBParams& hp, unsigned long long* stats, cudaStream_t st,
+                                 uint32_t sweep_off, const HBParams& hp, cudaStream_t st,
                                  double* meas, int* meas_blocks) {
   if (meas && (mu < 1 || parity != 1 || !meas_blocks)) return cudaErrorInvalidValue;
   SU2_DISPATCH_MU(mu, {
@@ -424,9 +413,9 @@ cudaError_t launch_heatbath_prec(const LatticeView& v, int mu, int parity, const
         if (gr > kMeasStride) return cudaErrorInvalidConfiguration;
         *meas_blocks = gr;
       }
-      return launch_pdl(true, kernel, dim3((unsigned)gr), nthreads, st, L, v.g, sub, sweep_base, sweep_off, hp, stats, m);
+      return launch_pdl(true, kernel, dim3((unsigned)gr), nthreads, st, L, v.g, sub, sweep_base, sweep_off, hp, m);
     };
-    const bool small = !stats && overlaps(v);
+    const bool small = overlaps(v);
     const bool one_each = v.g.vh > 128 * sms && v.g.vh <= 256 * sms;
     auto launch_small = [&](auto kernel, int nthreads, double* m, int lanes = 1) -> cudaError_t {
       const int gr = (int)((v.g.vh * lanes + nthreads - 1) / nthreads);

@@ -3,7 +3,6 @@
 
 namespace su2 {
 
-template cudaError_t launch_heatbath_prec<kF16Q>(const LatticeView&, int, int, const uint32_t*, uint32_t, const HBParams&,
-                                              unsigned long long*, cudaStream_t, double*, int*);
+template cudaError_t launch_heatbath_prec<kF16Q>(const LatticeView&, int, int, const uint32_t*, uint32_t, const HBParams&, cudaStream_t, double*, int*);
 
 }  // namespace su2

@@ -44,7 +44,7 @@ cudaError_t launch_init(const LatticeView& v, int start, PhiloxKey key, uint32_t
 // With `meas` (only for mu >= 1, parity 1) the substep also writes one
 // plaquette block sum per block to meas[0, *meas_blocks) (see k_heatbath).
 cudaError_t launch_heatbath(const LatticeView& v, int mu, int parity, const uint32_t* sweep_base,
-                            uint32_t sweep_off, const HBParams& hp, unsigned long long* stats,
+                            uint32_t sweep_off, const HBParams& hp,
                             cudaStream_t st, double* meas = nullptr, int* meas_blocks = nullptr);
 // Block sums of the three measuring substeps sit at meas + k * kMeasStride
 // (k = 0, 1, 2 for mu = 1, 2, 3; nb[k] blocks each).

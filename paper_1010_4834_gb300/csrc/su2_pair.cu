@@ -173,7 +173,6 @@ __global__ void __launch_bounds__(kPairThreads, kPairBlocksPerSM)
   const unsigned int total = 2u * (unsigned int)shp.nt * (unsigned int)shp.cps;
   const int chunk_links = BS * kPairLinksPerThread;
   PlainAcc<R> plaq;
-  HBCount cnt;
   unsigned int next = 0;
   if (threadIdx.x == 0) {
     qn = 0;
@@ -196,19 +195,18 @@ __global__ void __launch_bounds__(kPairThreads, kPairBlocksPerSM)
       for (int k = 0; k < kPairLinksPerThread; ++k) {
         const int h = h0 + k * BS + (int)threadIdx.x;
         if (h < h1) hb_link<P, MU, false, 0, false, CAP>(L, g, Substep{MU, 0}, h, tag, sweep, beta, hp,
-                                                         reinterpret_cast<Deferred<R, false>*>(queue), &qn, plaq, cnt);
+                                                         reinterpret_cast<Deferred<R, false>*>(queue), &qn, plaq);
       }
       __syncthreads();
-      hb_drain<P, MU, false, 0>(L, Substep{MU, 0}, reinterpret_cast<Deferred<R, false>*>(queue), min(qn, CAP), tag, sweep, hp, plaq,
-                                cnt);
+      hb_drain<P, MU, false, 0>(L, Substep{MU, 0}, reinterpret_cast<Deferred<R, false>*>(queue), min(qn, CAP), tag, sweep, hp, plaq);
     } else {
 #pragma unroll
       for (int k = 0; k < kPairLinksPerThread; ++k) {
         const int h = h0 + k * BS + (int)threadIdx.x;
-        if (h < h1) hb_link<P, MU, MEAS, 1, true, CAP>(L, g, Substep{MU, 1}, h, tag, sweep, beta, hp, queue, &qn, plaq, cnt);
+        if (h < h1) hb_link<P, MU, MEAS, 1, true, CAP>(L, g, Substep{MU, 1}, h, tag, sweep, beta, hp, queue, &qn, plaq);
       }
       __syncthreads();
-      hb_drain<P, MU, MEAS, 1>(L, Substep{MU, 1}, queue, min(qn, CAP), tag, sweep, hp, plaq, cnt);
+      hb_drain<P, MU, MEAS, 1>(L, Substep{MU, 1}, queue, min(qn, CAP), tag, sweep, hp, plaq);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
