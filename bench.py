@@ -26,6 +26,7 @@ Multi-GPU (torchrun): independent replicas, one lattice per rank (the
 method's lattices do not shard here), weak scaling, max time over ranks.
 """
 import argparse
+import glob
 import hashlib
 import json
 import os
@@ -295,17 +296,30 @@ def batched_run(torch, peaks):
     return out
 
 
-def batch_source_sha():
-    """Hash of the batched kernel's sources (code only) and build flags."""
+def _csrc(*names):
+    """Paths of the named files of csrc (patterns allowed), sorted."""
+    csrc = os.path.join(ROOT, "paper_1010_4834_gb300", "csrc")
+    return sorted(f for n in names for f in glob.glob(os.path.join(csrc, n)))
+
+
+def _sha_of(files):
+    """Hash of these sources (code only) and of the build flags."""
     h = hashlib.sha256()
-    pkg = os.path.join(ROOT, "paper_1010_4834_gb300")
-    for f in ("su2_batch.cu", "su2_batch.h", "su2_batch_kernel.cuh", "su2_device.cuh", "su2_fixed.cuh", "su2_hb_link.cuh",
-              "su2_kernel_util.cuh", "su2_internal.h"):
-        with open(os.path.join(pkg, "csrc", f), encoding="utf-8") as fh:
+    for f in files:
+        with open(f, encoding="utf-8") as fh:
             h.update(_code_only(fh.read()).encode())
-    with open(os.path.join(pkg, "build.py"), encoding="utf-8") as fh:
+    with open(os.path.join(ROOT, "paper_1010_4834_gb300", "build.py"), encoding="utf-8") as fh:
         h.update(_code_only(fh.read(), python=True).encode())
     return h.hexdigest()[:16]
+
+
+# what every heat-bath kernel's code depends on
+_HB_HEADERS = ("su2_device.cuh", "su2_fixed.cuh", "su2_hb_link.cuh", "su2_kernel_util.cuh", "su2_internal.h")
+
+
+def batch_source_sha():
+    """Hash of the batched kernel's sources, its instantiations' among them."""
+    return _sha_of(_csrc("su2_batch*.cu*", "su2_batch.h", *_HB_HEADERS))
 
 
 def static_potential_run():
@@ -444,16 +458,8 @@ def _code_only(text, python=False):
 
 
 def source_sha():
-    """Hash of the heat-bath kernels' sources (code only) and build flags."""
-    h = hashlib.sha256()
-    pkg = os.path.join(ROOT, "paper_1010_4834_gb300")
-    for f in (os.path.join(pkg, "csrc", "su2_device.cuh"), os.path.join(pkg, "csrc", "su2_heatbath.cuh"),
-              os.path.join(pkg, "csrc", "su2_hb_link.cuh"), os.path.join(pkg, "csrc", "su2_pair.cu"), os.path.join(pkg, "csrc", "su2_fixed.cuh"),
-              os.path.join(pkg, "csrc", "su2_kernel_util.cuh"), os.path.join(pkg, "csrc", "su2_internal.h"),
-              os.path.join(pkg, "build.py")):
-        with open(f, encoding="utf-8") as fh:
-            h.update(_code_only(fh.read(), python=f.endswith(".py")).encode())
-    return h.hexdigest()[:16]
+    """Hash of the heat-bath kernels' sources, the instantiations' among them."""
+    return _sha_of(_csrc("su2_heatbath*.cu*", "su2_pair.cu", *_HB_HEADERS))
 
 
 def _profile_values(name):
@@ -479,31 +485,6 @@ def profiled_traffic(kind, updates_per_launch):
         return float(vals["dram_bytes_per_update"]) * updates_per_launch
     except (KeyError, ValueError):
         return None
-
-
-def profiled_f64_flops():
-    """FP64 flops per heat-bath link update (2 DFMA + DMUL + DADD thread
-    instructions, from the committed ncu summary of an FP64 substep), or None
-    if the kernel source changed since the capture."""
-    vals = _profile_values("hb_substep_f64.md")
-    if vals.get("source_sha") != source_sha():
-        return None
-    try:
-        return float(vals["fp64_flops_per_update"])
-    except (KeyError, ValueError):
-        return None
-
-
-def f64_roofline(updates_per_s, fp64_peak):
-    """The FP64 heat bath against the probe-measured FP64 FMA rate (its bound:
-    GB300 issues FP64 at 1/64 of the FP32 rate)."""
-    fl = profiled_f64_flops()
-    if fl is None or not fp64_peak:
-        return {"bound": "alu", "achieved": None, "peak": fp64_peak, "unit": "FLOP/s", "frac": None,
-                "note": "FP64 flops per update not profiled for this source"}
-    ach = fl * updates_per_s
-    return {"bound": "alu", "achieved": ach, "peak": fp64_peak, "unit": "FLOP/s", "frac": round(ach / fp64_peak, 4),
-            "flops_per_update": fl, "peak_kind": "measured (su2_probe_fma, FP64)"}
 
 
 def measured_peaks():
@@ -715,24 +696,19 @@ def run_gpu_on_stream(args):
                                    "kernel on one site-major array (element 4 s + mu), the paper's layout"}
         lat.close()
         del lat
-        fp64_peak = probe_fma("f64")
-        extra["fma_peaks"] = {"f64": fp64_peak, "f32": probe_fma("f32"), "unit": "FLOP/s",
+        extra["fma_peaks"] = {"f64": probe_fma("f64"), "f32": probe_fma("f32"), "unit": "FLOP/s",
                               "what": "su2_probe_fma: eight independent FMA chains per thread over a full grid"}
         for prec, n in (("f64", 4), ("f16q", 20)):
             l2 = Lattice(DIMS, BETA, seed=1, start="hot", prec=prec)
             l2.sweep(2)
             extra[prec] = {"value": n * 4 * V / timed_sweeps(torch, l2, n, reps=2), "unit": UNIT,
                            "what": "%s 64^4 heat-bath sweeps alone, %d sweeps" % (prec, n)}
-            if prec == "f64":
-                extra[prec]["roofline"] = f64_roofline(extra[prec]["value"], fp64_peak)
-            else:
+            if prec != "f64":                                # FP64: integer issue, no traffic or flop roofline
                 g = extra[prec]["value"] * 64 / 1e9          # 8 links of 8 B per update
                 extra[prec]["achieved_gbs"] = round(g, 1)
                 extra[prec]["frac"] = round(g / peaks["hbm_gbs"], 4)
             l2.close()
         extra["configs"] = small_configs(torch)
-        c1 = extra["configs"]["values"]["8^4_f64_cold_100sweeps_measured"]
-        extra["configs"]["8^4_f64_roofline"] = f64_roofline(c1, fp64_peak)
         extra["static_potential"] = static_potential_run()
         if not args.no_cpu:
             extra["oracle_configs"] = oracle_per_config()

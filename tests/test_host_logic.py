@@ -60,6 +60,26 @@ def test_source_hash_ignores_comments_and_follows_code():
     assert len(sha) == 16 and all(ch in "0123456789abcdef" for ch in sha)
 
 
+def test_profile_hashes_cover_every_file_of_the_kernels(tmp_path, monkeypatch):
+    # the instantiations too: one of them switches the products' rounding
+    import bench
+    import shutil
+    pkg = tmp_path / "paper_1010_4834_gb300"
+    shutil.copytree(os.path.join(ROOT, "paper_1010_4834_gb300", "csrc"), pkg / "csrc")
+    shutil.copy(os.path.join(ROOT, "paper_1010_4834_gb300", "build.py"), pkg)
+    here = bench.source_sha(), bench.batch_source_sha()
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert (bench.source_sha(), bench.batch_source_sha()) == here
+    for name, which in (("su2_batch_f32.cu", 1), ("su2_batch_f64_measured.cu", 1), ("su2_heatbath_f32.cu", 0), ("su2_pair.cu", 0),
+                        ("su2_fixed.cuh", 0), ("su2_fixed.cuh", 1), ("su2_batch.h", 1)):
+        f = pkg / "csrc" / name
+        text = f.read_text()
+        f.write_text("#define SOMETHING\n" + text)
+        assert (bench.source_sha(), bench.batch_source_sha())[which] != here[which], name
+        f.write_text(text)
+
+
+
 def test_reference_arm_prints_one_contract_line():
     # the oracle arm of the benchmark (CPU only), on a small extent so the
     # test is quick: one JSON line with the keys the benchmark contract needs
