@@ -757,12 +757,11 @@ extern "C" int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smea
   return SU2_OK;
 }
 
-// The device-visible address of page-locked host memory (cudaHostAlloc,
-// cudaHostRegister: the conversion kernel then reads it directly over the
-// host link, at the copy engine's rate), or NULL for pageable memory.
 // The address a kernel on `device` reads `p` through: page-locked host memory
-// (mapped), or device / managed memory of that device; nullptr for pageable
-// host memory.  *other_device is set for device memory of another GPU.
+// (cudaHostAlloc, cudaHostRegister: the conversion kernel reads it directly over
+// the host link, at the copy engine's rate), or device / managed memory of that
+// device; nullptr for pageable host memory.  *other_device is set for device
+// memory of another GPU.
 static void* device_readable(const void* p, int device, bool* other_device) {
   *other_device = false;
   cudaPointerAttributes a;

@@ -90,8 +90,8 @@ template <class R> __device__ __forceinline__ R qdot(const Quat<R>& a, const Qua
 
 // Products with every rounding spelled out: a sum of two products leaves the
 // compiler the choice which of them it fuses, and kernels that must agree bit
-// for bit (plain, measured and small-lattice substeps, pairs, time slabs) did
-// differ.
+// for bit (plain, measured and small-lattice substeps, pairs, time slabs; in FP64
+// batches too) did differ.
 template <> __device__ __forceinline__ double qdot<double>(const Quat<double>& a, const Quat<double>& b) {
   return __fma_rn(a.z, b.z, __fma_rn(a.y, b.y, __fma_rn(a.x, b.x, __dmul_rn(a.w, b.w))));
 }
@@ -110,12 +110,16 @@ template <> __device__ __forceinline__ Quat<double> qmul_dn<double>(const Quat<d
   return qmul<double>(qmake<double>(a.w, -a.x, -a.y, -a.z), b);
 }
 
-// The updates' products.  In the heat-bath substeps' files FP32 fuses the first
-// product of each sum, or the first positive one, as those kernels were compiled
-// before.  Files whose kernels need no such agreement define SU2_COMPILER_FUSES:
-// FP32 batches, whose links stay those of earlier versions so, and measurements
-// and over-relaxation, which schedule better (64^4: plaquette 344 us, 366 spelled
-// out, FP32; over-relaxation 1376 us a sweep and 1411, F16Q).
+// The updates' products below FP64.  The heat-bath substeps, the pairs and the F16Q
+// batches fuse the first product of each sum, or the first positive one, as the
+// substeps' kernels were compiled before.  A file that defines SU2_COMPILER_FUSES
+// before its includes leaves the choice to the compiler: the FP32 batches, whose links
+// stay those of earlier versions so, and su2_kernels.cu, whose measurements and
+// over-relaxation schedule better (64^4: plaquette 344 us, 366 spelled out, FP32;
+// over-relaxation 1376 us a sweep and 1411, F16Q).  A lattice alone and in a batch
+// therefore leaves the same links in FP64 only; below, FP32 differs in the last bits
+// of the heat bath, F16Q in those of over-relaxation.  No kernel is compiled in two
+// files, so none has two bodies.
 #ifdef SU2_COMPILER_FUSES
 constexpr bool kCompilerFuses = true;
 #else

@@ -1,7 +1,9 @@
-// One link's heat-bath update (Section 2, Eqs. 5-9, 11), shared by the
-// substep kernel (su2_heatbath.cu), the fused parity-pair kernel
-// (su2_pair.cu) and the batched kernel (su2_batch.cu), so all of them run
-// the same arithmetic and leave the same links.
+// One link's heat-bath update (Section 2, Eqs. 5-9, 11) and over-relaxation
+// update, shared by the substep kernel (su2_heatbath.cuh), the fused parity-pair
+// kernel (su2_pair.cu), the over-relaxation kernel (su2_kernels.cu) and the batched
+// kernel (su2_batch_kernel.cuh).  The heat bath of a lattice leaves the same links by
+// every schedule; how batches compare with it is said at SU2_COMPILER_FUSES
+// (su2_device.cuh).
 // Paper: Cardoso & Bicudo, arXiv:1010.4834.
 //
 // Every lane makes the link's first a0 trial inline.  A link that rejects it

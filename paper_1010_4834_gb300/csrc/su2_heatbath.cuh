@@ -429,7 +429,7 @@ cudaError_t launch_heatbath_prec(const LatticeView& v, int mu, int parity, const
       constexpr bool M = decltype(meas_c)::value;
       constexpr int KM = hb_dir<P, MU>, PP = hb_dir<P, decltype(par_c)::value>;
       if constexpr (P == kF64) {
-        // as many lanes a link as the small kernel's threads allow
+        // eight lanes a link, or two, while the small kernel's threads allow
         if (small && 8 * v.g.vh <= SmallPerSM<P>::value * sms) return launch_small(k_heatbath_lanes<M, 8>, 64, m, 8);
         if (small && 2 * v.g.vh <= SmallPerSM<P>::value * sms) return launch_small(k_heatbath_lanes<M, 2>, 64, m, 2);
       }

@@ -28,11 +28,12 @@ struct LatticeView {
   int prec;
 };
 
-// Reduction scratch carved from the handle's device memory.
+// Reduction scratch: partials and counters in the handle's device memory.
 struct Scratch {
   double* partials;      // >= kScratchPartials doubles
   unsigned int* counter; // one zero-initialised ticket counter per reduction
-  double* out;           // >= kScratchOut doubles, results of the last reduction
+  double* out;           // >= kScratchOut doubles of mapped host memory, results of the last
+                         // reduction (single lattices)
 };
 constexpr size_t kScratchPartials = (size_t)1 << 20;  // 8 MiB of doubles
 constexpr size_t kScratchOut = 2048;
@@ -50,8 +51,8 @@ cudaError_t launch_heatbath(const LatticeView& v, int mu, int parity, const uint
 // (k = 0, 1, 2 for mu = 1, 2, 3; nb[k] blocks each).
 constexpr int kMeasStride = 8192;
 // Measured sweeps record {plaquette all, spatial, space-time, Polyakov} of
-// sweep s in row s mod kHistRing of a device ring, so that a run of them is
-// position-independent and replays as one CUDA graph.
+// sweep s in row s mod kHistRing of a ring in mapped host memory, so that a run of
+// them is position-independent and replays as one CUDA graph.
 constexpr int kHistRing = 1024;
 // What the Polyakov kernel's last block does after a measured sweep: its
 // mean and the plaquette from the sweep's block sums go to row

@@ -1,5 +1,6 @@
-// Kernels of the SU(2) heat-bath Monte Carlo for sm_103a, except the
-// heat-bath substep itself (su2_heatbath.cu): start configurations, the
+// Kernels of the SU(2) heat-bath Monte Carlo for sm_103a, except the heat-bath
+// substep itself (su2_heatbath.cuh, su2_pair.cu) and batched sweeps
+// (su2_batch_kernel.cuh): start configurations, the
 // over-relaxation substep, the fused plaquette / Polyakov reductions, APE
 // smearing, Wilson loops and the canonical-layout conversions.  Paper: Cardoso & Bicudo,
 // arXiv:1010.4834 (Sections 2 and 4).

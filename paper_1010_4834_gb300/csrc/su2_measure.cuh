@@ -1,5 +1,5 @@
 // One site's plaquettes and one spatial site's time line, for the reductions of
-// single lattices (su2_kernels.cu) and of batches (su2_batch_kernel.cuh).
+// single lattices and of batches (k_batch_measure), all in su2_kernels.cu.
 // Read-only loads unless a kernel can start beside one that writes links (NC =
 // false; see pdl_wait).
 // Paper: Cardoso & Bicudo, arXiv:1010.4834.
