@@ -1087,8 +1087,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
     }
     // (2) prefix over a column's chunks, the warp's lanes: G(a, r) for the
     // thread's rows, P(a) = G(a, Nt).  Products of up to eight unit quaternions,
-    // normalised with G; their rounding (1e-6 in FP32) says nothing of the links.
-    bool rounding = false;
+    // normalised with G.
 #pragma unroll
     for (int d = 1; d < kTgChunks; d *= 2) {
       const E before = tg_lane_up(Q, d * kTgCols);
@@ -1099,7 +1098,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
       }
     }
     if (active && c == kTgChunks - 1) {
-      Pb[a] = M::unit(Q, rounding);
+      Pb[a] = M::unit(Q, bad);
       if constexpr (NORMS) Np[a] = n;
     }
     Q = tg_lane_up(Q, kTgCols);
@@ -1108,7 +1107,7 @@ __global__ void __launch_bounds__(kTgThreads, 1)
 #pragma unroll
       for (int i = 0; i < RO; ++i) {
         E* p = Sb + tg_row<RO>(r0 + i, SS) + a;
-        *p = M::unit(M::mul(Q, *p), rounding);
+        *p = M::unit(M::mul(Q, *p), bad);
         if constexpr (NORMS) Nb[(r0 + i) * nm + a] = tg_times(n, Nb[(r0 + i) * nm + a]);
       }
     }
