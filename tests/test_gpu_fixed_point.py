@@ -148,39 +148,41 @@ def test_wilson_loops_on_both_sides_of_the_time_outer_kernels_range(nt, prec):
             np.testing.assert_allclose(lat.wilson_loops(rmax, tmax), ref[:rmax, :tmax], atol=MTOL[prec] * 5, rtol=0)
 
 
-def _off_unit(nt, off, halves, dims=(6, 4, 6)):
+def _off_unit(nt, off, where, dims=(6, 4, 6)):
     """Ordered links (large loops) whose norms differ by up to off from one, link
-    by link or in the two halves of the lattice: a loop carries its own links'
-    norms."""
+    by link, up and down in the two halves of the lattice, or all alike: a loop
+    carries its own links' norms."""
     dims = (*dims, nt)
     rng = np.random.default_rng(nt)
     U = np.array([1.0, 0.0, 0.0, 0.0]) + 0.3 * inputs.random_field(dims, 5)
     U /= np.linalg.norm(U, axis=-1, keepdims=True)
-    w = np.sign(np.arange(U.shape[0]) - U.shape[0] // 2 + 0.5)[:, None] if halves else rng.uniform(-1, 1, U.shape[:2])
+    w = {"links": rng.uniform(-1, 1, U.shape[:2]), "halves": np.sign(np.arange(U.shape[0]) - U.shape[0] // 2 + 0.5)[:, None],
+         "all": np.ones((1, 1))}[where]
     return dims, U * (1 + off * w)[..., None]
 
 
 @pytest.mark.parametrize("nt", [12, 16, 24])
 @pytest.mark.parametrize("off", [1e-6, 1e-5, 1e-2])
-@pytest.mark.parametrize("halves", [False, True])
-def test_fp32_wilson_loops_on_links_off_unit_norm(nt, off, halves):
-    # below 2^-18 in |U|^2 norms may be dropped: 24 time links of 1e-6, in the
-    # loops' mean at most the halves' difference, within 5e-6 with FP32's own
-    # rounding
-    dims, U = _off_unit(nt, off, halves)
+@pytest.mark.parametrize("where", ["links", "halves", "all"])
+def test_fp32_wilson_loops_on_links_off_unit_norm(nt, off, where):
+    # below 2^-18 in |U|^2 the norms of a loop's 2 T time links are dropped: 24 x 1e-6
+    # where all links are off alike, in the mean over loops much less where they
+    # differ; 5e-6 for FP32's own rounding
+    atol = 5e-6 + (24 * off if where == "all" and off < 1.9e-6 else 0.0)
+    dims, U = _off_unit(nt, off, where)
     lat = Lattice(dims, 2.0, prec="f32")
     lat.set_links(U)
     ref = oracle.wilson_loops(list(dims), as_stored(U, "f32"), 4, 12)
     for _ in range(2):
-        np.testing.assert_allclose(lat.wilson_loops(4, 12), ref, atol=5e-6, rtol=0)
+        np.testing.assert_allclose(lat.wilson_loops(4, 12), ref, atol=atol, rtol=0)
 
 
 @pytest.mark.parametrize("nt", [12, 16, 24])
 @pytest.mark.parametrize("off", [1e-15, 1e-13, 1e-11, 1e-9, 1e-7, 1e-4])
-@pytest.mark.parametrize("halves", [False, True])
-def test_fp64_wilson_loops_on_links_off_unit_norm(nt, off, halves):
+@pytest.mark.parametrize("where", ["links", "halves", "all"])
+def test_fp64_wilson_loops_on_links_off_unit_norm(nt, off, where):
     # 32 links of a loop, four products each of 2^-53
-    dims, U = _off_unit(nt, off, halves)
+    dims, U = _off_unit(nt, off, where)
     lat = Lattice(dims, 2.0, prec="f64")
     lat.set_links(U)
     ref = oracle.wilson_loops(list(dims), U, 4, 12)
