@@ -331,11 +331,11 @@ int su2_ape_smear(su2_lattice* h, double alpha, int n);
  * (the loop is gauge invariant: after the transform each is one dot
  * product of two spatial lines), which equals the direct product up to
  * rounding; FP32 links count as unit within 4e-6 in |U|^2, and their norms
- * (2 T 2e-6 of a loop at most) are dropped.  FP64 links further from unit norm than a chain leaves them
- * (|U|^2 off one by 7e-15; rounded to FP32, say) take a second pass that
- * keeps norms (32^4, W(16,16): 8.1 ms against 3.4 ms).  Other shapes, and
- * links off by 4e-6 in FP32 or 1.5e-5 in FP64, multiply the loops out
- * (85 ms).  Synchronises.
+ * (2 T 2e-6 of a loop at most) are dropped.  FP64 links further from unit
+ * norm than a chain leaves them (|U|^2 off one by 7e-15; rounded to FP32,
+ * say) take a second pass that keeps norms (32^4, W(16,16): 8.1 ms against
+ * 3.4 ms).  Other shapes, and links off by 4e-6 in FP32 or 1.5e-5 in FP64,
+ * multiply the loops out (85 ms).  Synchronises.
  */
 int su2_wilson_loops(su2_lattice* h, int Rmax, int Tmax, int use_smeared, double* out);
 
